@@ -10,6 +10,7 @@
 #include <vector>
 
 #include "../../include/gda.h"
+#include "energy_tc.h"
 #include "gda_internal.h"
 #include "kernels.h"
 #include "res.h"
@@ -38,11 +39,10 @@ struct gda_ctx {
   unsigned char* J8 = nullptr;  // [Np][Np] E4M3, row-scaled (FP8 path, on first use)
   float* jscale = nullptr;      // [Np] row scales of J8
   bool j8_ready = false;
-  int* Jint = nullptr;
   double* g64 = nullptr;  // [Np]
   float* g32 = nullptr;   // [Np]
   float* h1 = nullptr;    // [Np]
-  bool int_exact = false;
+  double jmax = -1.0;     // largest |J_ij| when every J_ij is an integer, else -1
   double diag = 0.0;      // -sum_i J_ii
   // instance checks
   int* d_flags = nullptr;
@@ -76,19 +76,16 @@ struct gda_ctx {
   float* K = nullptr;  // GD-mod per-restart couplings [K_R][N][Np]
   size_t K_cap = 0;
   int K_R = 0;         // restarts K was initialised for (0: none)
-  double* S64 = nullptr;
-  int* Sint = nullptr;
+  double* S64 = nullptr;      // complex spins of the final energies
   double* part64 = nullptr;
-  long long* partint = nullptr;
+  int* erexp = nullptr;       // final energies: row exponents and digit tiles of J, digit tiles of the spins
+  unsigned char* eJd = nullptr;
+  unsigned char* eSd = nullptr;
+  size_t eJd_cap = 0, eSd_cap = 0;
+  bool eJ_ready = false;      // eJd holds the whole current J
   double* E64 = nullptr;
   double* bestE = nullptr;
   int* bestR = nullptr;
-  double* E32 = nullptr;    // ranking: compensated FP32 energies [rank_cap]
-  int* cidx = nullptr;      // ranking: candidate restarts [rank_cap]
-  int* d_count = nullptr;
-  double* d_abs = nullptr;
-  int rank_cap = 0;
-  double abs_sum = -1.0;    // sum |J0| + sum |g| of the current instance (-1: not computed)
   signed char* cfg8 = nullptr;
   double* cfgth = nullptr;
   long long* t_step = nullptr;
@@ -177,7 +174,7 @@ void free_state(gda_ctx* c) {
     dfree(c->rho[k]);
   }
   dfree(c->acc); dfree(c->S32); dfree(c->gam); dfree(c->gstg); dfree(c->gacc); dfree(c->epart);
-  dfree(c->ops); dfree(c->S64); dfree(c->Sint); dfree(c->part64); dfree(c->partint); dfree(c->E64);
+  dfree(c->ops); dfree(c->S64); dfree(c->part64); dfree(c->E64);
   if (c->plan) tc_plan_destroy(c->plan);
   c->plan = nullptr;
   dfree(c->ops8);
@@ -212,17 +209,11 @@ gda_status ensure_state(gda_ctx* c, int R) {
   CK(dalloc(&c->gstg, rn));
   CK(dalloc(&c->gacc, rn));
   CK(dalloc(&c->epart, MT * Rp));
-  CK(dalloc(&c->S64, cn));
+  if (c->cplx) CK(dalloc(&c->S64, cn));
   CK(dalloc(&c->part64, MT * Rp));
   CK(dalloc(&c->E64, Rp));
-  if (c->int_exact || c->model == GDA_ISING) {
-    CK(dalloc(&c->Sint, cn));
-    CK(dalloc(&c->partint, MT * Rp));
-  }
   float* zf[] = {c->psi[0], c->psi[1], c->stg[0], c->stg[1], c->acc, c->S32};
   for (float* p : zf) CK(cudaMemsetAsync(p, 0, cn * sizeof(float), c->stream));
-  CK(cudaMemsetAsync(c->S64, 0, cn * sizeof(double), c->stream));
-  if (c->Sint) CK(cudaMemsetAsync(c->Sint, 0, cn * sizeof(int), c->stream));
   CK(cudaMemsetAsync(c->gam, 0, rn * sizeof(float), c->stream));
   CK(cudaMemsetAsync(c->gstg, 0, rn * sizeof(float), c->stream));
   CK(cudaMemsetAsync(c->gacc, 0, rn * sizeof(float), c->stream));
@@ -251,7 +242,6 @@ gda_status load_instance(gda_ctx* c, const double* J, const double* g, cudaMemcp
   c->K_R = 0;  // a GD-mod coupling state belongs to the previous J
   LK(launch_snapshot_reset(c->snapE, c->snapR, c->snapStep, c->stream));
   c->ell_maxdeg = -1;
-  c->abs_sum = -1.0;
   CK(cudaMemsetAsync(c->d_flags, 0, sizeof(int), c->stream));
   CK(cudaMemsetAsync(c->d_maxabs, 0, sizeof(unsigned long long), c->stream));
   LK(launch_check_instance(c->J64, c->g64, c->N, c->Np, c->d_flags, c->d_maxabs, c->d_diag, c->stream));
@@ -266,15 +256,9 @@ gda_status load_instance(gda_ctx* c, const double* J, const double* g, cudaMemcp
   if (flags & 8) return fail(c, GDA_ERR_INVALID, "g has a non-finite entry");
   double maxabs;
   std::memcpy(&maxabs, &mbits, sizeof(maxabs));
-  const bool was_int = c->int_exact;
-  c->int_exact = c->model == GDA_ISING && !(flags & 4) && !(flags & 16) && maxabs * double(N) < 2147483647.0;
-  if (c->int_exact && !c->Jint) CK(dalloc(&c->Jint, Np * Np));
-  if (c->int_exact && !was_int && c->psi[0] && !c->Sint) {
-    CK(dalloc(&c->Sint, size_t(c->Cp) * Np));
-    CK(cudaMemsetAsync(c->Sint, 0, size_t(c->Cp) * Np * sizeof(int), c->stream));
-    CK(dalloc(&c->partint, size_t(c->MT) * c->Rp));
-  }
-  LK(launch_prepare_J(c->J64, c->Np, c->J32, c->J16, c->int_exact ? c->Jint : nullptr, c->stream));
+  c->jmax = (flags & 4) ? -1.0 : maxabs;
+  c->eJ_ready = false;
+  LK(launch_prepare_J(c->J64, c->Np, c->J32, c->J16, c->stream));
   c->j8_ready = false;
   return GDA_OK;
 }
@@ -470,16 +454,73 @@ gda_status run_gdmod(gda_ctx* c, const gda_params* p, int R, int64_t steps) {
   return GDA_OK;
 }
 
-gda_status compute_energies(gda_ctx* c) {
-  if (!c->have_state) return fail(c, GDA_ERR_STATE, "no state: call gda_run or gda_set_state first");
-  if (c->int_exact) {
-    LK(launch_energy_int(c->psi[c->cur], c->Jint, c->Sint, c->partint, c->E64, c->N, c->Np, c->R, c->Rp, c->C,
-                         c->stream));
-  } else {
-    LK(launch_energy64(c->psi[c->cur], c->J64, c->g64, c->S64, c->part64, c->E64, c->N, c->Np, c->R, c->Rp, c->C,
-                       pmode(c), c->stream));
+// Grows a digit workspace to at least `blocks` blocks of `per` bytes, halving
+// the request while memory is short; *blocks receives what fits.
+gda_status ensure_digits(gda_ctx* c, unsigned char** p, size_t* cap, size_t per, int* blocks) {
+  while (*cap < size_t(*blocks) * per) {
+    dfree(*p);
+    *cap = 0;
+    const cudaError_t e = dalloc(p, size_t(*blocks) * per);
+    if (e == cudaSuccess) {
+      *cap = size_t(*blocks) * per;
+    } else if (e == cudaErrorMemoryAllocation && *blocks > 1) {
+      cudaGetLastError();
+      *blocks = (*blocks + 1) / 2;
+    } else {
+      return cuda_fail(c, e, "energy workspace");
+    }
   }
   return GDA_OK;
+}
+
+// FP64 Eq. (1) energies of R restarts (C columns) of psi into E64
+// (energy_tc.cu), in panels that fit the digit workspaces.
+gda_status energies_of(gda_ctx* c, const float* psi, int R, int C) {
+  EnergyProb p = energy_prob(c->N, c->Np, c->Np, R, C, pmode(c), c->jmax);
+  p.J = c->J64;
+  p.g = c->g64;
+  p.psi = psi;
+  p.S64 = c->S64;
+  p.part = c->part64;
+  p.ldp = c->Rp;
+  if (!c->erexp) CK(dalloc(&c->erexp, size_t(c->Np)));
+  p.rexp = c->erexp;
+  const int MT = p.mtn, NT = p.ntn;
+  const size_t perJ = energy_J_bytes(p) / MT, perS = energy_S_bytes(p) / NT;
+  int mp = int(std::min<size_t>(MT, std::max<size_t>(1, kEnergyJBytes / perJ)));
+  int np = int(std::min<size_t>(NT, std::max<size_t>(1, kEnergySBytes / perS)));
+  if (c->eJd_cap < size_t(mp) * perJ) c->eJ_ready = false;
+  gda_status s = ensure_digits(c, &c->eJd, &c->eJd_cap, perJ, &mp);
+  if (s == GDA_OK) s = ensure_digits(c, &c->eSd, &c->eSd_cap, perS, &np);
+  if (s != GDA_OK) return s;
+  p.Jd = c->eJd;
+  p.Sd = c->eSd;
+  for (int m = 0; m < MT; m += mp) {
+    p.mt0 = m;
+    p.mtn = std::min(mp, MT - m);
+    EnergyUnits u{};
+    u.KBmax = p.KB;
+    u.n_row = p.mtn;
+    if (!c->eJ_ready) {
+      LK(launch_energy_slice_J(p, u, c->stream));
+      c->eJ_ready = mp == MT;
+    }
+    for (int n = 0; n < NT; n += np) {
+      p.nt0 = n;
+      p.ntn = std::min(np, NT - n);
+      u.n_col = p.ntn;
+      u.n_tile = p.mtn * p.ntn;
+      if (m == 0 || np < NT) LK(launch_energy_slice_S(p, u, c->stream));
+      LK(launch_energy_product(p, u, c->err, c->stream));
+    }
+  }
+  LK(launch_energy_sum(c->part64, MT, R, c->Rp, c->E64, c->stream));
+  return GDA_OK;
+}
+
+gda_status compute_energies(gda_ctx* c) {
+  if (!c->have_state) return fail(c, GDA_ERR_STATE, "no state: call gda_run or gda_set_state first");
+  return energies_of(c, c->psi[c->cur], c->R, c->C);
 }
 
 gda_status check_err(gda_ctx* c) {
@@ -543,10 +584,10 @@ int64_t gda_kernel_launches(const gda_ctx* c) { return c ? c->launches : 0; }
 void gda_destroy(gda_ctx* c) {
   if (!c) return;
   free_state(c);
-  dfree(c->J64); dfree(c->J32); dfree(c->J16); dfree(c->J8); dfree(c->jscale); dfree(c->Jint); dfree(c->g64); dfree(c->g32); dfree(c->h1);
+  dfree(c->J64); dfree(c->J32); dfree(c->J16); dfree(c->J8); dfree(c->jscale); dfree(c->g64); dfree(c->g32); dfree(c->h1);
   dfree(c->d_flags); dfree(c->d_maxabs); dfree(c->d_diag);
   dfree(c->bestE); dfree(c->bestR); dfree(c->cfg8); dfree(c->cfgth);
-  dfree(c->E32); dfree(c->cidx); dfree(c->d_count); dfree(c->d_abs);
+  dfree(c->erexp); dfree(c->eJd); dfree(c->eSd);
   dfree(c->t_step); dfree(c->t_E); dfree(c->t_r); dfree(c->t_count); dfree(c->err); dfree(c->flags);
   dfree(c->seg_flags);
   dfree(c->lastE); dfree(c->lastR); dfree(c->snapE); dfree(c->snapR); dfree(c->snapStep); dfree(c->snap);
@@ -934,62 +975,12 @@ gda_status gda_energy(gda_ctx* c, double* E) {
   return check_err(c);
 }
 
-// FP64 argmin through candidate ranking (non-integer energies, R >= 32):
-// compensated FP32 energies of all restarts carry an error below
-// delta = 48 u (sum |J0| + sum |g|) (u = 2^-24: J rounded to FP32, spins
-// rounded once, 16-term FMA blocks plus an exact two-sum, double partials);
-// every restart within 2 (delta + delta64) of the lowest FP32 value is
-// evaluated in FP64 (delta64 covers the FP64 sums themselves), which contains
-// the FP64 argmin over all restarts.  Sets *done = false when ranking does
-// not narrow the set (the caller then evaluates every restart).
-gda_status best_ranked(gda_ctx* c, bool* done) {
-  *done = false;
-  if (c->int_exact || c->R < 32) return GDA_OK;
-  if (c->rank_cap < c->Rp) {
-    dfree(c->E32);
-    dfree(c->cidx);
-    c->rank_cap = 0;
-    CK(dalloc(&c->E32, size_t(c->Rp)));
-    CK(dalloc(&c->cidx, size_t(c->Rp)));
-    c->rank_cap = c->Rp;
-  }
-  if (!c->d_count) CK(dalloc(&c->d_count, 1));
-  if (!c->d_abs) CK(dalloc(&c->d_abs, 1));
-  if (c->abs_sum < 0.0) {
-    LK(launch_abs_sum(c->J64, c->g64, c->N, c->Np, c->d_abs, c->stream));
-    CK(cudaMemcpyAsync(&c->abs_sum, c->d_abs, sizeof(double), cudaMemcpyDeviceToHost, c->stream));
-    CK(cudaStreamSynchronize(c->stream));
-  }
-  const double u = std::ldexp(1.0, -24);
-  const double delta = 48.0 * u * c->abs_sum;
-  const double delta64 = 1e-9 * (c->abs_sum + std::fabs(c->diag)) + 1e-300;
-  const double margin = 2.0 * (delta + delta64);
-  LK(launch_rank(c->psi[c->cur], c->J32, c->g64, c->S32, c->part64, c->E32, c->cidx, c->d_count, c->N, c->Np, c->R,
-                 c->Rp, c->C, pmode(c), c->diag, margin, c->stream));
-  int count = 0;
-  CK(cudaMemcpyAsync(&count, c->d_count, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
-  CK(cudaStreamSynchronize(c->stream));
-  if (count < 1 || count > c->R / 2) return GDA_OK;
-  LK(launch_gather_cols(c->psi[c->cur], c->Np, c->cidx, count, c->cplx, c->stg[0], c->stream));
-  LK(launch_energy64(c->stg[0], c->J64, c->g64, c->S64, c->part64, c->E64, c->N, c->Np, count, c->Rp,
-                     count * (c->cplx ? 2 : 1), pmode(c), c->stream));
-  LK(launch_argmin(c->E64, count, c->bestE, c->bestR, c->stream));
-  LK(launch_map_best(c->cidx, c->bestR, c->stream));
-  *done = true;
-  return GDA_OK;
-}
-
 gda_status gda_best(gda_ctx* c, double* E, int32_t* r, void* cfg) {
   if (!c) return GDA_ERR_INVALID;
   if (!c->have_state) return fail(c, GDA_ERR_STATE, "no state: call gda_run or gda_set_state first");
-  bool ranked = false;
-  gda_status s = best_ranked(c, &ranked);
+  gda_status s = compute_energies(c);
   if (s != GDA_OK) return s;
-  if (!ranked) {
-    s = compute_energies(c);
-    if (s != GDA_OK) return s;
-    LK(launch_argmin(c->E64, c->R, c->bestE, c->bestR, c->stream));
-  }
+  LK(launch_argmin(c->E64, c->R, c->bestE, c->bestR, c->stream));
   double e = 0.0;
   int rr = 0;
   CK(cudaMemcpyAsync(&e, c->bestE, sizeof(double), cudaMemcpyDeviceToHost, c->stream));
@@ -1016,13 +1007,8 @@ gda_status gda_best_seen(gda_ctx* c, double* E, int32_t* r, int64_t* step, void*
   CK(cudaMemcpyAsync(&st, c->snapStep, sizeof(long long), cudaMemcpyDeviceToHost, c->stream));
   CK(cudaStreamSynchronize(c->stream));
   if (rr < 0 || !c->have_state) return fail(c, GDA_ERR_STATE, "no tracked state: run with energy_every > 0 first");
-  const int W = c->cplx ? 2 : 1;
-  if (c->int_exact) {
-    LK(launch_energy_int(c->snap, c->Jint, c->Sint, c->partint, c->E64, c->N, c->Np, 1, c->Rp, W, c->stream));
-  } else {
-    LK(launch_energy64(c->snap, c->J64, c->g64, c->S64, c->part64, c->E64, c->N, c->Np, 1, c->Rp, W, pmode(c),
-                       c->stream));
-  }
+  gda_status s = energies_of(c, c->snap, 1, c->cplx ? 2 : 1);
+  if (s != GDA_OK) return s;
   double e = 0.0;
   CK(cudaMemcpyAsync(&e, c->E64, sizeof(double), cudaMemcpyDeviceToHost, c->stream));
   if (cfg) {
@@ -1032,7 +1018,7 @@ gda_status gda_best_seen(gda_ctx* c, double* E, int32_t* r, int64_t* step, void*
     else
       CK(cudaMemcpyAsync(cfg, c->cfg8, size_t(c->N), cudaMemcpyDeviceToHost, c->stream));
   }
-  gda_status s = check_err(c);
+  s = check_err(c);
   if (s != GDA_OK) return s;
   if (E) *E = e;
   if (r) *r = rr;
@@ -1054,12 +1040,8 @@ gda_status gda_trace_energy(gda_ctx* c, int32_t first, int32_t count, double* E)
   for (int k0 = 0; k0 < count; k0 += c->R) {
     const int m = std::min(c->R, count - k0);
     const float* src = c->hist + size_t(first + k0) * W * c->Np;
-    if (c->int_exact) {
-      LK(launch_energy_int(src, c->Jint, c->Sint, c->partint, c->E64, c->N, c->Np, m, c->Rp, m * W, c->stream));
-    } else {
-      LK(launch_energy64(src, c->J64, c->g64, c->S64, c->part64, c->E64, c->N, c->Np, m, c->Rp, m * W, pmode(c),
-                         c->stream));
-    }
+    gda_status s = energies_of(c, src, m, m * W);
+    if (s != GDA_OK) return s;
     CK(cudaMemcpyAsync(E + k0, c->E64, size_t(m) * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
   }
   return check_err(c);

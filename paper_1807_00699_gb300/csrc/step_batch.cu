@@ -31,6 +31,7 @@
 #include <vector>
 
 #include "../../include/gda.h"
+#include "energy_tc.h"
 #include "gda_internal.h"
 #include "tc_epilogue.cuh"
 #include "tc_ptx.cuh"
@@ -416,84 +417,13 @@ __global__ void k_batch_init(const BatchInst* inst, int n_inst, float* psi, floa
 
 __global__ void k_batch_advance(unsigned* step_base, unsigned by) { *step_base += by; }
 
-// FP64 Eq. (1) energies per instance and restart: one block per
-// (instance, 64-row tile, 64-column tile) unit; projection on the fly from
-// the FP32 amplitudes of buffer parity cur.
-__global__ void __launch_bounds__(256) k_batch_energy(const BatchInst* inst, const int4* units, const double* J64,
-                                                      const long long* off_J, const double* g64,
-                                                      const long long* off_g, const float* psi, int cur,
-                                                      double* part, const long long* off_part) {
-  const int4 U = units[blockIdx.x];
-  const BatchInst I = inst[U.x];
-  const int W = I.cplx ? 2 : 1, N = I.N, C = I.C;
-  const float* p = psi + I.off_psi + size_t(cur) * I.Cp * I.Np;
-  const double* J = J64 + off_J[U.x];
-  __shared__ double As[16][65];
-  __shared__ double Bs[16][65];
-  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-  const int m0 = U.y * 64, n0 = U.z * 64;
-  auto spin = [&](int c, int j) -> double {  // projected spin, column c = W r + part
-    if (W == 1) return p[size_t(c) * I.Np + j] >= 0.0f ? 1.0 : -1.0;
-    const int r = c >> 1;
-    const double re = p[size_t(2 * r) * I.Np + j], im = p[size_t(2 * r + 1) * I.Np + j];
-    const double m = sqrt(re * re + im * im);
-    if (!(m > 0.0)) return (c & 1) ? 0.0 : 1.0;
-    return ((c & 1) ? im : re) / m;
-  };
-  double acc[4][4] = {};
-  const int lr = tid >> 2, lk = (tid & 3) * 4;
-  for (int k0 = 0; k0 < N; k0 += 16) {
-    __syncthreads();
-    for (int t = 0; t < 4; ++t) {
-      const int row = m0 + lr, col = n0 + lr, k = k0 + lk + t;
-      As[lk + t][lr] = (row < N && k < N) ? J[size_t(row) * N + k] : 0.0;
-      Bs[lk + t][lr] = (col < C && k < N) ? spin(col, k) : 0.0;
-    }
-    __syncthreads();
-#pragma unroll
-    for (int k = 0; k < 16; ++k) {
-      double bv[4];
-#pragma unroll
-      for (int v = 0; v < 4; ++v) bv[v] = Bs[k][4 * ty + v];
-#pragma unroll
-      for (int a = 0; a < 4; ++a) {
-        const double av = As[k][tx + 16 * a];
-#pragma unroll
-        for (int v = 0; v < 4; ++v) acc[a][v] += av * bv[v];
-      }
-    }
-  }
-  double rs[4] = {0.0, 0.0, 0.0, 0.0};
-  const int c0 = n0 + 4 * ty;
-  for (int a = 0; a < 4; ++a) {
-    const int i = m0 + tx + 16 * a;
-    if (i >= N) continue;
-    const double gi = g64[off_g[U.x] + i];
-    for (int u = 0; u < 4 / W; ++u) {
-      const int c = c0 + W * u;
-      if (c >= C) continue;
-      const double sr = spin(c, i);
-      double e = -sr * acc[a][W * u] + gi * sr;
-      if (W == 2) e -= spin(c + 1, i) * acc[a][W * u + 1];
-      rs[u] += e;
-    }
-  }
-  for (int u = 0; u < 4; ++u)
-    for (int off = 8; off; off >>= 1) rs[u] += __shfl_xor_sync(0xffffffffu, rs[u], off);
-  if (tx == 0)
-    for (int u = 0; u < 4 / W; ++u) {
-      const int r = c0 / W + u;
-      if (r < I.R) part[off_part[U.x] + size_t(U.y) * I.R + r] = rs[u];
-    }
-}
-
 // Per instance: E_r = sum of its row-tile partials, then the argmin (ties to
 // the lowest restart).  One block per instance.
 __global__ void k_batch_best(const BatchInst* inst, const double* part, const long long* off_part, double* E_all,
                              const long long* off_E, double* bestE, int* bestR) {
   const int b = blockIdx.x;
   const BatchInst I = inst[b];
-  const int tiles = (I.N + 63) / 64;
+  const int tiles = (I.N + 127) / 128;
   __shared__ double sE[32];
   __shared__ int sR[32];
   double best = 1.0 / 0.0;
@@ -566,6 +496,11 @@ struct BatchPlan {
   int n_units = 0;
 };
 
+// Panels [prob0, ...) of one group: offsets of its unit lists in eunits.
+struct EnergyGroup {
+  int row0 = 0, n_row = 0, col0 = 0, n_col = 0, tile0 = 0, n_tile = 0, KBmax = 0;
+};
+
 struct gda_batch {
   int n = 0, dev = 0, sms = 148, pitch = 0;
   cudaStream_t stream = nullptr;
@@ -588,8 +523,16 @@ struct gda_batch {
   long long* off_E = nullptr;
   double* bestE = nullptr;
   int* bestR = nullptr;
+  // final energies (energy_tc.cu): panels of instances, and the groups of
+  // panels whose digits share the workspace at one time
+  std::vector<long long> oJ, oG, oP;
+  std::vector<double> jmax;       // per instance: largest |J_ij| of an integer J, else -1
+  std::vector<EnergyGroup> egroups;
+  EnergyProb* eprobs[2] = {nullptr, nullptr};  // panels for either state parity
   int4* eunits = nullptr;
-  int n_eunits = 0;
+  int* erexp = nullptr;
+  unsigned char* edigits = nullptr;
+  bool eJ_ready = false;          // one group: its J digits are kept between calls
   unsigned* step_base = nullptr;
   unsigned* flags = nullptr;  // per-unit step flags [n_flags]
   int n_flags = 0;
@@ -761,6 +704,155 @@ gda_status upload_settings(gda_batch* b, const gda_params* p) {
   return GDA_OK;
 }
 
+// Plans the final energies on first use: every instance is cut into panels
+// (row blocks x column blocks) whose digits fit the workspace bounds, and
+// panels are grouped while the digits and spins of a group fit together
+// (in `bound` bytes, unless one row block against one column block needs more).
+gda_status plan_energies(gda_batch* b, size_t bound) {
+  void* stale[] = {b->erexp, b->eunits, b->eprobs[0], b->eprobs[1]};  // of an attempt that failed
+  for (void* p : stale)
+    if (p) cudaFree(p);
+  b->erexp = nullptr;
+  b->eunits = nullptr;
+  b->eprobs[0] = b->eprobs[1] = nullptr;
+  auto align = [](size_t x) { return (x + 1023) / 1024 * 1024; };
+  struct Place {
+    int inst;
+    size_t jd, sd, s64;  // offsets in the workspace of the panel's group
+  };
+  std::vector<EnergyProb> probs;
+  std::vector<Place> place;
+  std::vector<int4> row, col, tile;
+  std::vector<EnergyGroup> groups(1);
+  size_t used = 0, top = 0;
+  long long n_rexp = 0;
+  std::vector<long long> orexp(b->n);
+  for (int k = 0; k < b->n; ++k) {
+    const BatchInst& I = b->host[k];
+    orexp[k] = n_rexp;
+    n_rexp += I.N;
+    const EnergyProb whole = energy_prob(I.N, I.Np, I.N, I.R, I.C, I.cplx, b->jmax[k]);
+    const int MT = whole.mtn, NT = whole.ntn;
+    const size_t perJ = energy_J_bytes(whole) / MT;
+    const size_t perS = energy_S_bytes(whole) / NT + (I.cplx ? size_t(128) * I.Np * sizeof(double) : 0);
+    const int mp = int(std::min<size_t>(MT, std::max<size_t>(1, bound / 5 * 4 / perJ)));
+    const int np = int(std::min<size_t>(NT, std::max<size_t>(1, bound / 5 / perS)));
+    for (int m = 0; m < MT; m += mp)
+      for (int c = 0; c < NT; c += np) {
+        EnergyProb p = whole;
+        p.mt0 = m;
+        p.mtn = std::min(mp, MT - m);
+        p.nt0 = c;
+        p.ntn = std::min(np, NT - c);
+        Place at{k, 0, 0, 0};
+        const size_t sj = align(energy_J_bytes(p)), ss = align(energy_S_bytes(p));
+        const size_t s64 = I.cplx ? align(size_t(p.ntn) * 128 * I.Np * sizeof(double)) : 0;
+        if (used && used + sj + ss + s64 > bound) {
+          EnergyGroup g;
+          g.row0 = int(row.size());
+          g.col0 = int(col.size());
+          g.tile0 = int(tile.size());
+          groups.push_back(g);
+          used = 0;
+        }
+        at.jd = used;
+        at.sd = at.jd + sj;
+        at.s64 = at.sd + ss;
+        used = at.s64 + s64;
+        top = std::max(top, used);
+        EnergyGroup& g = groups.back();
+        const int id = int(probs.size());
+        for (int y = 0; y < p.mtn; ++y) row.push_back(make_int4(id, y, 0, 0));
+        for (int z = 0; z < p.ntn; ++z) col.push_back(make_int4(id, 0, z, 0));
+        for (int z = 0; z < p.ntn; ++z)
+          for (int y = 0; y < p.mtn; ++y) tile.push_back(make_int4(id, y, z, 0));
+        g.n_row = int(row.size()) - g.row0;
+        g.n_col = int(col.size()) - g.col0;
+        g.n_tile = int(tile.size()) - g.tile0;
+        g.KBmax = std::max(g.KBmax, p.KB);
+        probs.push_back(p);
+        place.push_back(at);
+      }
+  }
+  // column units carry their block in .y for the slicing kernel's unit form
+  for (int4& c : col) c.y = c.z;
+  // longest tiles first within a group, so that the last wave is short
+  for (const EnergyGroup& g : groups)
+    std::stable_sort(tile.begin() + g.tile0, tile.begin() + g.tile0 + g.n_tile, [&](const int4& x, const int4& y) {
+      const EnergyProb &p = probs[x.x], &q = probs[y.x];
+      return p.KB * p.nsJ * p.nsS > q.KB * q.nsJ * q.nsS;
+    });
+  unsigned char* ws = nullptr;
+  BCK(balloc(&b->erexp, size_t(n_rexp)));
+  BCK(balloc(&b->eunits, row.size() + col.size() + tile.size()));
+  BCK(cudaMemcpy(b->eunits, row.data(), row.size() * sizeof(int4), cudaMemcpyHostToDevice));
+  BCK(cudaMemcpy(b->eunits + row.size(), col.data(), col.size() * sizeof(int4), cudaMemcpyHostToDevice));
+  BCK(cudaMemcpy(b->eunits + row.size() + col.size(), tile.data(), tile.size() * sizeof(int4),
+                 cudaMemcpyHostToDevice));
+  BCK(balloc(&ws, top));
+  for (int cur = 0; cur < 2; ++cur) {
+    for (size_t q = 0; q < probs.size(); ++q) {
+      const int k = place[q].inst;
+      const BatchInst& I = b->host[k];
+      EnergyProb& p = probs[q];
+      p.J = b->J64 + b->oJ[k];
+      p.g = b->g64 + b->oG[k];
+      p.psi = b->psi + I.off_psi + size_t(cur) * I.Cp * I.Np;
+      p.rexp = b->erexp + orexp[k];
+      p.Jd = ws + place[q].jd;
+      p.Sd = ws + place[q].sd;
+      // the panel's spins, addressed by the instance's column numbers
+      p.S64 = I.cplx ? reinterpret_cast<double*>(ws + place[q].s64) - (long long)p.nt0 * 128 * I.Np : nullptr;
+      p.part = b->part + b->oP[k];
+      p.ldp = I.R;
+    }
+    cudaError_t e = balloc(&b->eprobs[cur], probs.size());
+    if (e == cudaSuccess)
+      e = cudaMemcpy(b->eprobs[cur], probs.data(), probs.size() * sizeof(EnergyProb), cudaMemcpyHostToDevice);
+    if (e != cudaSuccess) {
+      cudaFree(ws);
+      BCK(e);
+    }
+  }
+  for (EnergyGroup& g : groups) {
+    g.col0 += int(row.size());
+    g.tile0 += int(row.size() + col.size());
+  }
+  b->egroups = std::move(groups);
+  b->edigits = ws;  // last: marks the plan complete
+  return GDA_OK;
+}
+
+// FP64 Eq. (1) energies of every restart: partial sums per 128-row block in part.
+gda_status batch_energies(gda_batch* b) {
+  size_t bound = kEnergyJBytes + kEnergySBytes;
+  while (!b->edigits) {
+    const gda_status s = plan_energies(b, bound);
+    if (s == GDA_ERR_OOM && bound > (size_t(64) << 20)) {
+      bound /= 4;
+      continue;
+    }
+    if (s != GDA_OK) return s;
+  }
+  for (const EnergyGroup& g : b->egroups) {
+    EnergyUnits u{};
+    u.probs = b->eprobs[b->step & 1ULL];
+    u.row = b->eunits + g.row0;
+    u.col = b->eunits + g.col0;
+    u.tile = b->eunits + g.tile0;
+    u.n_row = g.n_row;
+    u.n_col = g.n_col;
+    u.n_tile = g.n_tile;
+    u.KBmax = g.KBmax;
+    const EnergyProb none{};
+    if (!b->eJ_ready) BCK(launch_energy_slice_J(none, u, b->stream));
+    BCK(launch_energy_slice_S(none, u, b->stream));
+    BCK(launch_energy_product(none, u, b->err, b->stream));
+  }
+  b->eJ_ready = b->egroups.size() == 1;
+  return GDA_OK;
+}
+
 }  // namespace
 
 extern "C" {
@@ -770,15 +862,21 @@ gda_status gda_batch_create(int32_t n, const int32_t* N, const int32_t* model, c
   if (!out) return GDA_ERR_INVALID;
   *out = nullptr;
   if (n < 1 || !N || !model || !R || !J) return GDA_ERR_INVALID;
+  std::vector<double> jmax(n);
   for (int k = 0; k < n; ++k) {
     if (N[k] < 1 || N[k] > 65536 || R[k] < 1 || (model[k] != GDA_ISING && model[k] != GDA_XY) || !J[k])
       return GDA_ERR_INVALID;
     const int64_t nn = N[k];
+    bool integer = true;
+    double m = 0.0;
     for (int64_t i = 0; i < nn; ++i)
       for (int64_t j = 0; j < nn; ++j) {
         const double v = J[k][i * nn + j];
         if (!std::isfinite(v) || v != J[k][j * nn + i]) return GDA_ERR_INVALID;
+        integer = integer && v == std::rint(v);
+        m = std::max(m, std::fabs(v));
       }
+    jmax[k] = integer ? m : -1.0;
     if (g && g[k])
       for (int64_t i = 0; i < nn; ++i)
         if (!std::isfinite(g[k][i])) return GDA_ERR_INVALID;
@@ -800,10 +898,14 @@ gda_status gda_batch_create(int32_t n, const int32_t* N, const int32_t* model, c
   }
   cudaDeviceGetAttribute(&b->sms, cudaDevAttrMultiProcessorCount, b->dev);
   b->n = n;
+  b->jmax = std::move(jmax);
   b->host.resize(n);
   long long off_psi = 0, off_gam = 0, off_h1 = 0, off_beta = 0, off_J = 0, off_g = 0, off_part = 0, off_E = 0;
   long long off_base = 0, n_flags = 0;
-  std::vector<long long> oJ(n), oG(n), oP(n), oE(n);
+  std::vector<long long> &oJ = b->oJ, &oG = b->oG, &oP = b->oP, oE(n);
+  oJ.resize(n);
+  oG.resize(n);
+  oP.resize(n);
   int pitch = 64;
   b->own.assign(n, 0);
   for (int k = 0; k < n; ++k) {
@@ -845,7 +947,7 @@ gda_status gda_batch_create(int32_t n, const int32_t* N, const int32_t* model, c
     oG[k] = off_g;
     off_g += I.N;
     oP[k] = off_part;
-    off_part += (long long)((I.N + 63) / 64) * I.R;
+    off_part += (long long)I.mt * I.R;
     oE[k] = off_E;
     off_E += I.R;
     pitch = std::max(pitch, I.Np);
@@ -901,16 +1003,6 @@ gda_status gda_batch_create(int32_t n, const int32_t* N, const int32_t* model, c
                                                                                b->host[k].rowJ, pitch);
       BCK(cudaGetLastError());
     }
-    // FP64 energy units: (instance, 64-row tile, 64-column tile)
-    std::vector<int4> eu;
-    for (int k = 0; k < n; ++k) {
-      const BatchInst& I = b->host[k];
-      for (int mt = 0; mt < (I.N + 63) / 64; ++mt)
-        for (int nt = 0; nt < (I.C + 63) / 64; ++nt) eu.push_back(make_int4(k, mt, nt, 0));
-    }
-    b->n_eunits = int(eu.size());
-    BCK(balloc(&b->eunits, eu.size()));
-    BCK(cudaMemcpy(b->eunits, eu.data(), eu.size() * sizeof(int4), cudaMemcpyHostToDevice));
     if (!encode(&b->tmA, b->J16, pitch, int(b->rowsJ), 128) || !encode(&b->tmB128, b->ops, pitch, int(b->rowsX), 128) ||
         !encode(&b->tmB256, b->ops, pitch, int(b->rowsX), 256))
       return bfail(b, GDA_ERR_CUDA, "tensor map encoding failed");
@@ -1084,10 +1176,8 @@ int32_t gda_batch_launch_mode(const gda_batch* b) { return !b ? -1 : (b->graph ?
 gda_status gda_batch_best(gda_batch* b, double* E, int32_t* r) {
   if (!b) return GDA_ERR_INVALID;
   if (!b->have_state) return bfail(b, GDA_ERR_STATE, "no state");
-  const int cur = int(b->step & 1ULL);
-  k_batch_energy<<<b->n_eunits, 256, 0, b->stream>>>(b->inst, b->eunits, b->J64, b->off_J, b->g64, b->off_g, b->psi,
-                                                      cur, b->part, b->off_part);
-  BCK(cudaGetLastError());
+  gda_status es = batch_energies(b);
+  if (es != GDA_OK) return es;
   k_batch_best<<<b->n, 256, 0, b->stream>>>(b->inst, b->part, b->off_part, b->E_all, b->off_E, b->bestE, b->bestR);
   BCK(cudaGetLastError());
   if (E) BCK(cudaMemcpyAsync(E, b->bestE, size_t(b->n) * sizeof(double), cudaMemcpyDeviceToHost, b->stream));
@@ -1134,7 +1224,7 @@ void gda_batch_destroy(gda_batch* b) {
       if (P.units) cudaFree(P.units);
       if (P.cta_begin) cudaFree(P.cta_begin);
     }
-  void* ptrs[] = {b->inst, b->J16, b->ops, b->J64, b->g64, b->off_J, b->off_g, b->psi, b->gam, b->h1, b->beta,
+  void* ptrs[] = {b->eprobs[0], b->eprobs[1], b->erexp, b->edigits, b->inst, b->J16, b->ops, b->J64, b->g64, b->off_J, b->off_g, b->psi, b->gam, b->h1, b->beta,
                   b->part, b->off_part, b->E_all, b->off_E, b->bestE, b->bestR, b->eunits, b->step_base, b->err,
                   b->flags, b->base};
   for (void* p : ptrs)
