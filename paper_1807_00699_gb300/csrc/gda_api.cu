@@ -63,9 +63,7 @@ struct gda_ctx {
   __nv_bfloat16* ops = nullptr;  // [3][Cp][Np]: operand ping-pong + projected spins
   unsigned char* ops8 = nullptr;  // [2][Cp][Np]: E4M3 operand ping-pong (FP8 path)
   TcPlan* plan8 = nullptr;
-  int* ell_col = nullptr;     // sparse J0: [GDA_SPARSE_MAX_DEG][Np] column indices
-  float* ell_val = nullptr;   // [GDA_SPARSE_MAX_DEG][Np] values
-  int* ell_deg = nullptr;     // [Np] nonzeros per row
+  int2* ell = nullptr;        // sparse J0: [GDA_SPARSE_MAX_DEG][Np] (column, value bits)
   int* d_maxdeg = nullptr;
   int ell_maxdeg = -1;        // largest row count of the current J (-1: not built)
   bool run_sparse = false;    // steps of the current call use the sparse product
@@ -267,18 +265,14 @@ gda_status load_instance(gda_ctx* c, const double* J, const double* g, cudaMemcp
 // GDA_SPARSE_MAX_DEG per row).  Synchronises once to read the largest count.
 gda_status ensure_ell(gda_ctx* c) {
   const size_t Np = c->Np;
-  if (!c->ell_col) {
-    CK(dalloc(&c->ell_col, size_t(GDA_SPARSE_MAX_DEG) * Np));
-    CK(dalloc(&c->ell_val, size_t(GDA_SPARSE_MAX_DEG) * Np));
-    CK(dalloc(&c->ell_deg, Np));
+  if (!c->ell) {
+    CK(dalloc(&c->ell, size_t(GDA_SPARSE_MAX_DEG) * Np));
     CK(dalloc(&c->d_maxdeg, 1));
   }
   if (c->ell_maxdeg < 0) {
-    CK(cudaMemsetAsync(c->ell_col, 0, size_t(GDA_SPARSE_MAX_DEG) * Np * sizeof(int), c->stream));
-    CK(cudaMemsetAsync(c->ell_val, 0, size_t(GDA_SPARSE_MAX_DEG) * Np * sizeof(float), c->stream));
+    CK(cudaMemsetAsync(c->ell, 0, size_t(GDA_SPARSE_MAX_DEG) * Np * sizeof(int2), c->stream));
     CK(cudaMemsetAsync(c->d_maxdeg, 0, sizeof(int), c->stream));
-    LK(launch_prepare_ell(c->J32, c->N, int(Np), GDA_SPARSE_MAX_DEG, c->ell_col, c->ell_val, c->ell_deg,
-                          c->d_maxdeg, c->stream));
+    LK(launch_prepare_ell(c->J32, c->N, int(Np), GDA_SPARSE_MAX_DEG, c->ell, c->d_maxdeg, c->stream));
     int m = 0;
     CK(cudaMemcpyAsync(&m, c->d_maxdeg, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
     CK(cudaStreamSynchronize(c->stream));
@@ -312,6 +306,11 @@ gda_status ensure_fp8(gda_ctx* c) {
 }
 
 bool finite(double x) { return std::isfinite(x); }
+
+int device_sms(int dev) {
+  int sms = 0;
+  return cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && sms > 0 ? sms : 148;
+}
 
 gda_status check_params(gda_ctx* c, const gda_params* p) {
   if (!p) return fail(c, GDA_ERR_INVALID, "params is NULL");
@@ -384,7 +383,7 @@ StepArgs base_args(gda_ctx* c, const gda_params* p, bool tc) {
 
 gda_status launch_step(gda_ctx* c, const StepArgs& a, bool tc, const float* operand32, int op_buf) {
   if (c->run_sparse && !tc) {
-    LK(launch_step_sparse(a, c->ell_col, c->ell_val, c->ell_deg, operand32, c->ell_maxdeg, c->stream));
+    LK(launch_step_sparse(a, c->ell, operand32, c->ell_maxdeg, c->stream));
   } else if (a.row_scale) {
     LK(launch_step_tc8(c->plan8, a, op_buf, c->stream, c->run_pair));
   } else if (tc) {
@@ -595,7 +594,7 @@ void gda_destroy(gda_ctx* c) {
   dfree(c->d_zero);
   dfree(c->stamps);
   dfree(c->K);
-  dfree(c->ell_col); dfree(c->ell_val); dfree(c->ell_deg); dfree(c->d_maxdeg);
+  dfree(c->ell); dfree(c->d_maxdeg);
   for (float*& t : c->opT) dfree(t);
   dfree(c->fw[0]);
   dfree(c->fw[1]);
@@ -764,10 +763,12 @@ gda_status gda_run(gda_ctx* c, const gda_params* p, int32_t R, int64_t steps) {
   c->rcur = 0;
   if (decay) LK(launch_rho_partials(tc, c->psi[c->cur], c->N, c->Np, c->R, c->Rp, c->cplx, c->rho[0], c->stream));
 
-  // sparse product: the gathers read a spin-major copy of the operand (the 4
-  // columns of a thread's quad in one 16-byte load), kept in step by the epilogue
+  // sparse product of the gather kernel: it reads a spin-major copy of the
+  // operand (the 4 columns of a thread's quad in one 16-byte load), kept in
+  // step by the epilogue
   int tcur = 0;
-  if (c->run_sparse) {
+  const bool spin_major = c->run_sparse && (p->integ == GDA_RK4 || !sparse_stages(c->Np));
+  if (spin_major) {
     const size_t tn = size_t(c->Np) * c->Cp;
     if (c->opT_cap < tn) {
       for (float*& t : c->opT) dfree(t);
@@ -894,6 +895,36 @@ gda_status gda_run(gda_ctx* c, const gda_params* p, int32_t R, int64_t steps) {
     return GDA_OK;
   }
 
+  // Sparse Euler runs whose columns fit on chip: one launch per tracking
+  // segment.  A segment of one step gains nothing over the per-step kernel.
+  base.rho_out = decay ? c->rho[c->rcur ^ 1] : nullptr;
+  const int seg_cols = c->run_sparse && p->integ == GDA_EULER ? sparse_seg_columns(base, device_sms(c->dev)) : 0;
+  const int64_t seg_len = p->energy_every > 0 ? p->energy_every : std::min<int64_t>(steps, 1 << 16);
+  if (seg_cols && seg_len > 1) {
+    for (int64_t k = 0; k < steps; k += seg_len) {
+      const int64_t len = std::min<int64_t>(seg_len, steps - k);
+      StepArgs a = base;
+      a.mode = M_EULER;
+      a.step = static_cast<unsigned int>(c->step + k);
+      a.psi_n = c->psi[c->cur];
+      a.psi_out = c->psi[c->cur ^ 1];
+      a.beta_in = c->beta[c->bcur];
+      a.beta_out = c->beta[c->bcur ^ 1];
+      a.rho_in = c->rho[c->rcur];
+      a.rho_out = decay ? c->rho[c->rcur ^ 1] : nullptr;
+      LK(launch_sparse_seg(a, c->ell, c->ell_maxdeg, int(len), seg_cols, c->stream));
+      c->cur ^= 1;
+      c->bcur ^= 1;
+      if (decay) c->rcur ^= 1;
+      if (p->energy_every > 0 && len == seg_len) {
+        s = track(c, p, tc, c->step + k + len);
+        if (s != GDA_OK) return s;
+      }
+    }
+    c->step += steps;
+    return GDA_OK;
+  }
+
   for (int64_t k = 0; k < steps; ++k) {
     const long long n = c->step + k;
     StepArgs a = base;
@@ -909,7 +940,7 @@ gda_status gda_run(gda_ctx* c, const gda_params* p, int32_t R, int64_t steps) {
       a.psi_out = c->psi[c->cur ^ 1];
       a.op_out = (tc && !f8) ? c->ops + (c->opcur ^ 1) * opsz : nullptr;
       a.op8_out = f8 ? c->ops8 + (c->opcur ^ 1) * opsz : nullptr;
-      if (c->run_sparse) {
+      if (spin_major) {
         a.opT_in = c->opT[tcur];
         a.opT_out = c->opT[(tcur + 1) % 3];
       }
@@ -930,7 +961,7 @@ gda_status gda_run(gda_ctx* c, const gda_params* p, int32_t R, int64_t steps) {
         const int in_buf = c->opcur ^ (st & 1);
         a.op_out = (tc && !f8) ? c->ops + (in_buf ^ 1) * opsz : nullptr;
         a.op8_out = f8 ? c->ops8 + (in_buf ^ 1) * opsz : nullptr;
-        if (c->run_sparse) {  // psi in T[tcur]; stages through T[A], T[B], T[A]; psi^{n+1} back to T[tcur]
+        if (spin_major) {  // psi in T[tcur]; stages through T[A], T[B], T[A]; psi^{n+1} back to T[tcur]
           const int A = (tcur + 1) % 3, B = (tcur + 2) % 3;
           const int tin[4] = {tcur, A, B, A}, tout[4] = {A, B, A, tcur};
           a.opT_in = c->opT[tin[st]];

@@ -93,12 +93,17 @@ double ptx_cycles_per_second();
 // Launchers (return cudaGetLastError() of the launch).
 cudaError_t launch_step_simt(const StepArgs& a, const float* J32, const float* operand, cudaStream_t s);
 int simt_mtiles(int N);
-// Sparse J0 (ELL [dmax][Np], ascending columns): the SIMT step with the SGEMM
-// replaced by a gather over the nonzeros; same tiles and epilogue.
-cudaError_t launch_step_sparse(const StepArgs& a, const int* col, const float* val, const int* deg,
-                               const float* operand, int maxdeg, cudaStream_t s);
-cudaError_t launch_prepare_ell(const float* J32, int N, int Np, int dmax, int* col, float* val, int* deg, int* maxdeg,
-                               cudaStream_t s);
+// Sparse J0 (ELL [dmax][Np] of (column, value), ascending columns): the SIMT
+// step with the SGEMM replaced by a gather over the nonzeros; same tiles and
+// epilogue.
+cudaError_t launch_step_sparse(const StepArgs& a, const int2* cv, const float* operand, int maxdeg, cudaStream_t s);
+cudaError_t launch_prepare_ell(const float* J32, int N, int Np, int dmax, int2* cv, int* maxdeg, cudaStream_t s);
+// A segment of forward-Euler steps in one launch (psi_n -> psi_out, beta_in ->
+// beta_out, rho_in -> rho_out, gam in place); columns per CTA from
+// sparse_seg_columns (0: not applicable).
+int sparse_seg_columns(const StepArgs& a, int sms);
+cudaError_t launch_sparse_seg(const StepArgs& a, const int2* cv, int maxdeg, int steps, int columns, cudaStream_t s);
+bool sparse_stages(int Np);
 // out[i][c] = x[c][i] for c < Cp, i < Np (column-major state -> spin-major operand).
 cudaError_t launch_transpose_state(const float* x, int Np, int Cp, float* out, cudaStream_t s);
 

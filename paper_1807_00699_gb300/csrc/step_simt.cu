@@ -4,7 +4,7 @@
 // path whose amplitudes are compared with the FP64 oracle.
 //
 // The sparse variant (SPARSE = true) replaces the SGEMM by a gather over the
-// nonzeros of J0 in ELL form (col / val [dmax][Np], deg [Np]): thread (tx, ty)
+// nonzeros of J0 in ELL form ((column, value) [dmax][Np]): thread (tx, ty)
 // sums, for its 4 rows and 4 columns, val_ik X[c][col_ik] in ascending k.  The
 // tile shape, the thread-to-element map and the epilogue (with its partial-sum
 // order) are the dense kernel's, so density partials, noise decay and the
@@ -19,10 +19,9 @@ namespace {
 constexpr int BM = 64, BN = 64, BK = 16, PAD = 4;
 constexpr size_t kPairSmemMax = 200 * 1024;  // the staged sparse kernel: N rounded up to 128 <= 25600
 
+// J0's nonzeros, (column, value bits) in one 8-byte load: [dmax][Np], (0, 0) past a row's count.
 struct Ell {
-  const int* col;   // [dmax][Np]
-  const float* val; // [dmax][Np]
-  const int* deg;   // [Np], 0 beyond N
+  const int2* cv;
 };
 
 // DW (sparse): the ELL width the loop runs over, a power of two >= the largest
@@ -67,8 +66,9 @@ __global__ void __launch_bounds__(256) step_simt_kernel(StepArgs a, const float*
 #pragma unroll
         for (int k = 0; k < KC; ++k) {
           const size_t o = size_t(k0 + k) * Np + m0 + tx + 16 * q;
-          jj[q][k] = ell.col[o];
-          vv[q][k] = ell.val[o];
+          const int2 e = ell.cv[o];
+          jj[q][k] = e.x;
+          vv[q][k] = __int_as_float(e.y);
         }
       if (a.opT_in) {  // spin-major operand: the 4 columns of spin j are one 16-byte load
         float4 x[4][KC];
@@ -199,7 +199,7 @@ cudaError_t launch_modes(const StepArgs& a, const float* J32, const float* opera
 }
 
 cudaError_t launch_step_simt(const StepArgs& a, const float* J32, const float* operand, cudaStream_t s) {
-  const Ell none{nullptr, nullptr, nullptr};
+  const Ell none{nullptr};
   return a.cplx ? launch_modes<true, false, 0>(a, J32, operand, none, s)
                 : launch_modes<false, false, 0>(a, J32, operand, none, s);
 }
@@ -299,8 +299,9 @@ __global__ void __launch_bounds__(PAIR_THREADS) k_sparse_euler_pair(StepArgs a, 
 #pragma unroll
     for (int k = 0; k < DW; ++k) {
       const size_t o = size_t(k) * Np + ic;
-      const int j = ell.col[o];
-      const float v = ell.val[o];
+      const int2 cv = ell.cv[o];
+      const int j = cv.x;
+      const float v = __int_as_float(cv.y);
       y0 = __fmaf_rn(v, x0[j], y0);
       y1 = __fmaf_rn(v, x1[j], y1);
     }
@@ -409,6 +410,237 @@ cudaError_t launch_pair(const StepArgs& a, const Ell& ell, cudaStream_t s) {
 
 }  // namespace
 
+namespace {
+
+// A segment of forward-Euler steps over a sparse J0 in one launch.  A column
+// of the state only ever reads itself, so a CTA that owns NC columns (NC
+// Ising restarts, NC / 2 XY restarts) runs all steps of a segment without
+// meeting another CTA: the amplitudes stay in shared memory, spin-major and
+// double-buffered (xs[2][Np][NC]: a neighbour's NC values are one load), the
+// gains in registers, and only the couplings' table is read again (from L2)
+// every step.  Rows go to threads as in k_sparse_euler_pair (16-thread groups
+// per 64-row tile, rows tx + 16 q) and every sum has that kernel's order, so
+// the results have the same bits.
+//
+// Bound by instruction issue and the shared-memory gathers (a row of four
+// columns: 3 table loads, 3 gathers, ~80 arithmetic instructions).  Measured
+// (GB300, N = 6000, R = 512, 3-regular, 1000 steps with tracking every 100 and
+// the best restart): 7.9 ms, 18.0 ms with a launch per step.  IT: tiles per
+// group.  DW: entries per row, 0: maxdeg of them, a run-time count.
+template <bool CPLX, int DW, int NC, int IT>
+__global__ void __launch_bounds__(NC == 4 && IT == 2 ? 896 : 1024) k_sparse_euler_seg(StepArgs a, Ell ell, int maxdeg,
+                                                                                   int steps) {
+  constexpr int W = CPLX ? 2 : 1;
+  constexpr int U = NC / W;  // restarts
+  extern __shared__ __align__(16) float xs[];
+  __shared__ float s_dsc[U];
+  __shared__ int s_bad;
+  const int tid = threadIdx.x, nthr = blockDim.x;
+  const int grp = tid >> 4, tx = tid & 15, ngrp = nthr >> 4;
+  const int Np = a.Np, N = a.N;
+  const int c0 = NC * int(blockIdx.x);  // < Cp (a multiple of 256)
+  const int r0 = c0 / W;
+  const bool decay = a.rho_out != nullptr;
+  float* s_rho = xs + size_t(2) * NC * Np;  // [mt_count][U], noise decay only
+  const unsigned half = (tid & 16) ? 0xffff0000u : 0x0000ffffu;
+
+  for (int i = tid; i < Np; i += nthr)
+#pragma unroll
+    for (int c = 0; c < NC; ++c) xs[size_t(i) * NC + c] = a.psi_n[size_t(c0 + c) * Np + i];
+  if (decay)
+    for (int k = tid; k < a.mt_count * U; k += nthr)
+      s_rho[k] = r0 + k % U < a.R ? a.rho_in[size_t(k / U) * a.Rp + r0 + k % U] : 0.0f;
+  float gam[IT][4][U], beta[U];
+#pragma unroll
+  for (int u = 0; u < U; ++u) beta[u] = r0 + u < a.R ? a.beta_in[r0 + u] : 1.0f;
+#pragma unroll
+  for (int t = 0; t < IT; ++t)
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int i = (grp + t * ngrp) * 64 + tx + 16 * q;
+#pragma unroll
+      for (int u = 0; u < U; ++u) gam[t][q][u] = i < N && r0 + u < a.R ? a.gam[size_t(r0 + u) * Np + i] : 0.0f;
+    }
+  if (tid == 0) s_bad = 0;
+  __syncthreads();
+
+  int bad = 0;
+  StepArgs na = a;  // the noise scale's view: this CTA's density sums
+  na.mode = M_EULER;
+  na.rho_in = s_rho;
+  na.Rp = U;
+  for (int n = 0; n < steps; ++n) {
+    float dsc[U];
+    if (decay) {
+      if (tid < U) s_dsc[tid] = r0 + tid < a.R ? noise_scale(na, tid) : 0.0f;
+      __syncthreads();
+    }
+    bool noise = false;
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      dsc[u] = decay ? s_dsc[u] : (r0 + u < a.R ? noise_scale(na, u) : 0.0f);
+      noise |= dsc[u] != 0.0f;
+    }
+    const float* x = xs + size_t(n & 1) * NC * Np;
+    float* xn = xs + size_t((n + 1) & 1) * NC * Np;
+#pragma unroll
+    for (int t = 0; t < IT; ++t) {
+      const int tile = grp + t * ngrp;
+      float red[U] = {};
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const int i = tile * 64 + tx + 16 * q;
+        if (i >= N) continue;
+        float y[NC] = {}, xi[NC], xo[NC];
+        auto gather = [&](int k) {
+          const int2 cv = __ldg(ell.cv + size_t(k) * Np + i);
+          const float v = __int_as_float(cv.y);
+          float xj[NC];
+          if (NC == 4)
+            *reinterpret_cast<float4*>(xj) = *reinterpret_cast<const float4*>(x + size_t(cv.x) * NC);
+          else
+            *reinterpret_cast<float2*>(xj) = *reinterpret_cast<const float2*>(x + size_t(cv.x) * NC);
+#pragma unroll
+          for (int c = 0; c < NC; ++c) y[c] = __fmaf_rn(v, xj[c], y[c]);
+        };
+        if (DW > 0) {
+#pragma unroll
+          for (int k = 0; k < DW; ++k) gather(k);
+        } else {
+          for (int k = 0; k < maxdeg; ++k) gather(k);
+        }
+        if (NC == 4)
+          *reinterpret_cast<float4*>(xi) = *reinterpret_cast<const float4*>(x + size_t(i) * NC);
+        else
+          *reinterpret_cast<float2*>(xi) = *reinterpret_cast<const float2*>(x + size_t(i) * NC);
+        const float h = __ldg(a.h1 + i);
+        float z[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+        if (noise) {
+          philox_normal4(uint32_t(i), uint32_t(c0 >> 2), a.step + unsigned(n), 0u, a.seed, z);
+          if (NC == 2 && (c0 & 2)) {  // the quad's second pair of columns
+            z[0] = z[2];
+            z[1] = z[3];
+          }
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          const float xr = xi[u * W], xim = CPLX ? xi[u * W + 1] : 0.0f;
+          float kr, ki, kg;
+          gd_rhs(xr, xim, gam[t][q][u], y[u * W], CPLX ? y[u * W + 1] : 0.0f, beta[u], h, a.eps, a.rho_th, kr, ki, kg);
+          if (CPLX && a.q) resonant_drive(xr, xim, a.q, a.hq, kr, ki);
+          float nr = axpy(a.dt, kr, xr);
+          float ni = axpy(a.dt, ki, xim);
+          gam[t][q][u] = axpy(a.dt, kg, gam[t][q][u]);
+          nr = axpy(dsc[u], z[u * W], nr);
+          if (CPLX) ni = axpy(dsc[u], z[u * W + 1], ni);
+          xo[u * W] = nr;
+          if (CPLX) xo[u * W + 1] = ni;
+          const float rn = density(nr, ni);
+          red[u] += rn;
+          bad |= r0 + u < a.R && !(rn < 1e30f);
+        }
+        if (NC == 4)
+          *reinterpret_cast<float4*>(xn + size_t(i) * NC) = *reinterpret_cast<const float4*>(xo);
+        else
+          *reinterpret_cast<float2*>(xn + size_t(i) * NC) = *reinterpret_cast<const float2*>(xo);
+      }
+      if (decay && tile < a.mt_count) {
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          float v = red[u];
+#pragma unroll
+          for (int off = 8; off; off >>= 1) v += __shfl_xor_sync(half, v, off);
+          if (tx == 0) s_rho[tile * U + u] = v;
+        }
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) beta[u] = next_beta(na, beta[u]);
+    __syncthreads();
+  }
+
+  const float* x = xs + size_t(steps & 1) * NC * Np;
+  for (int i = tid; i < N; i += nthr)
+#pragma unroll
+    for (int c = 0; c < NC; ++c)
+      if (c0 + c < a.C) a.psi_out[size_t(c0 + c) * Np + i] = x[size_t(i) * NC + c];
+  if (decay)
+    for (int k = tid; k < a.mt_count * U; k += nthr)
+      if (r0 + k % U < a.R) a.rho_out[size_t(k / U) * a.Rp + r0 + k % U] = s_rho[k];
+#pragma unroll
+  for (int t = 0; t < IT; ++t)
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int i = (grp + t * ngrp) * 64 + tx + 16 * q;
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+        if (i < N && r0 + u < a.R) a.gam[size_t(r0 + u) * Np + i] = gam[t][q][u];
+    }
+#pragma unroll
+  for (int u = 0; u < U; ++u)
+    if (tid == u && r0 + u < a.R) a.beta_out[r0 + u] = beta[u];
+  if (bad) atomicOr(&s_bad, 1);
+  __syncthreads();
+  if (tid == 0 && s_bad) atomicOr(a.err, E_DIVERGED);
+}
+
+constexpr size_t kSegSmemMax = 224 * 1024;
+
+size_t seg_smem(const StepArgs& a, int nc) {
+  const size_t u = a.cplx ? nc / 2 : nc;
+  return size_t(2) * nc * a.Np * sizeof(float) + (a.rho_out ? size_t(a.mt_count) * u * sizeof(float) : 0);
+}
+
+template <bool CPLX, int DW, int NC, int IT>
+cudaError_t launch_seg_it(const StepArgs& a, const Ell& ell, int maxdeg, int steps, cudaStream_t s) {
+  auto kern = k_sparse_euler_seg<CPLX, DW, NC, IT>;
+  const size_t smem = seg_smem(a, NC);
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kSegSmemMax));
+  if (e != cudaSuccess) return e;
+  const int groups = (a.mt_count + IT - 1) / IT;
+  kern<<<(a.C + NC - 1) / NC, (groups * 16 + 31) / 32 * 32, smem, s>>>(a, ell, maxdeg, steps);
+  return cudaGetLastError();
+}
+
+template <bool CPLX, int DW>
+cudaError_t launch_seg(const StepArgs& a, const Ell& ell, int maxdeg, int steps, cudaStream_t s, int nc) {
+  const int it = (a.mt_count + 63) / 64;
+  if (nc == 4)
+    return it == 1 ? launch_seg_it<CPLX, DW, 4, 1>(a, ell, maxdeg, steps, s)
+                   : launch_seg_it<CPLX, DW, 4, 2>(a, ell, maxdeg, steps, s);
+  switch (it) {
+    case 1: return launch_seg_it<CPLX, DW, 2, 1>(a, ell, maxdeg, steps, s);
+    case 2: return launch_seg_it<CPLX, DW, 2, 2>(a, ell, maxdeg, steps, s);
+    case 3: return launch_seg_it<CPLX, DW, 2, 3>(a, ell, maxdeg, steps, s);
+    default: return launch_seg_it<CPLX, DW, 2, 4>(a, ell, maxdeg, steps, s);
+  }
+}
+
+}  // namespace
+
+// The columns per CTA of a segment launch, 0 if the amplitudes of two columns
+// do not fit in shared memory twice (N > ~14 300).  Four columns share a row's
+// table loads and gathers: about 90 instructions a row against 2 x 53 for two
+// CTAs of two columns, so they win wherever they leave no more rounds of SMs.
+int sparse_seg_columns(const StepArgs& a, int sms) {
+  if (seg_smem(a, 2) > kSegSmemMax || a.mt_count > 256) return 0;
+  if (seg_smem(a, 4) > kSegSmemMax || a.mt_count > 112) return 2;
+  const long long w2 = ((a.C + 1) / 2 + sms - 1) / sms * 53LL, w4 = ((a.C + 3) / 4 + sms - 1) / sms * 90LL;
+  return w4 <= w2 ? 4 : 2;
+}
+
+cudaError_t launch_sparse_seg(const StepArgs& a, const int2* cv, int maxdeg, int steps, int columns, cudaStream_t s) {
+  const Ell ell{cv};
+  if (maxdeg <= 3)  // the paper's 3-regular graphs
+    return a.cplx ? launch_seg<true, 3>(a, ell, maxdeg, steps, s, columns)
+                  : launch_seg<false, 3>(a, ell, maxdeg, steps, s, columns);
+  return a.cplx ? launch_seg<true, 0>(a, ell, maxdeg, steps, s, columns)
+                : launch_seg<false, 0>(a, ell, maxdeg, steps, s, columns);
+}
+
+// True if Euler steps run in the staged kernel, which needs no spin-major operand.
+bool sparse_stages(int Np) { return size_t(2) * Np * sizeof(float) <= kPairSmemMax; }
+
 template <int DW>
 cudaError_t launch_sparse_w(const StepArgs& a, const Ell& ell, const float* operand, cudaStream_t s) {
   // Euler steps whose column pair fits in shared memory: the staged kernel
@@ -418,9 +650,8 @@ cudaError_t launch_sparse_w(const StepArgs& a, const Ell& ell, const float* oper
                 : launch_modes<false, true, DW>(a, nullptr, operand, ell, s);
 }
 
-cudaError_t launch_step_sparse(const StepArgs& a, const int* col, const float* val, const int* deg,
-                               const float* operand, int maxdeg, cudaStream_t s) {
-  const Ell ell{col, val, deg};
+cudaError_t launch_step_sparse(const StepArgs& a, const int2* cv, const float* operand, int maxdeg, cudaStream_t s) {
+  const Ell ell{cv};
   // the paper's 3-regular graphs: the staged Euler kernel loops over exactly
   // three entries (a fourth slot would add a zero product and cost a load)
   if (maxdeg <= 3 && a.mode == M_EULER && size_t(2) * a.Np * sizeof(float) <= kPairSmemMax)
@@ -444,10 +675,9 @@ __global__ void k_transpose_state(const float* __restrict__ x, int Np, int Cp, f
 }
 
 // One warp per row of J0 (FP32, diagonal removed, zero padding): the nonzeros
-// of row i in ascending column order go to col / val [k][Np] for k < dmax;
-// deg[i] = min(count, dmax) and *maxdeg receives the largest count.
-__global__ void k_prepare_ell(const float* __restrict__ J32, int N, int Np, int dmax, int* col, float* val, int* deg,
-                              int* maxdeg) {
+// of row i in ascending column order go to cv [k][Np] for k < dmax; *maxdeg
+// receives the largest count.
+__global__ void k_prepare_ell(const float* __restrict__ J32, int N, int Np, int dmax, int2* cv, int* maxdeg) {
   const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
   if (warp >= Np) return;
   const int i = warp;
@@ -459,17 +689,11 @@ __global__ void k_prepare_ell(const float* __restrict__ J32, int N, int Np, int 
       const float v = j < N ? row[j] : 0.0f;
       const unsigned m = __ballot_sync(0xffffffffu, v != 0.0f);
       const int k = count + __popc(m & ((1u << lane) - 1u));
-      if (v != 0.0f && k < dmax) {
-        col[size_t(k) * Np + i] = j;
-        val[size_t(k) * Np + i] = v;
-      }
+      if (v != 0.0f && k < dmax) cv[size_t(k) * Np + i] = make_int2(j, __float_as_int(v));
       count += __popc(m);
     }
   }
-  if (lane == 0) {
-    deg[i] = count < dmax ? count : dmax;
-    atomicMax(maxdeg, count);
-  }
+  if (lane == 0) atomicMax(maxdeg, count);
 }
 
 }  // namespace
@@ -479,10 +703,9 @@ cudaError_t launch_transpose_state(const float* x, int Np, int Cp, float* out, c
   return cudaGetLastError();
 }
 
-cudaError_t launch_prepare_ell(const float* J32, int N, int Np, int dmax, int* col, float* val, int* deg, int* maxdeg,
-                               cudaStream_t s) {
+cudaError_t launch_prepare_ell(const float* J32, int N, int Np, int dmax, int2* cv, int* maxdeg, cudaStream_t s) {
   const int blocks = (Np * 32 + 255) / 256;
-  k_prepare_ell<<<blocks, 256, 0, s>>>(J32, N, Np, dmax, col, val, deg, maxdeg);
+  k_prepare_ell<<<blocks, 256, 0, s>>>(J32, N, Np, dmax, cv, maxdeg);
   return cudaGetLastError();
 }
 
