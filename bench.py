@@ -505,7 +505,7 @@ def run_ours(args):
              else {gda.BF16: "step_tcs_kernel (persistent streaming launch of all timed steps, two-SM tiles: GEMM + "
                              "fused epilogue), time per step",
                    gda.FP8: "step_tcs_kernel (persistent streaming launch, E4M3 operands), time per step",
-                   gda.FP32: "step_simt_kernel"}[prec])
+                   gda.FP32: "k_dense_step"}[prec])
     traffic = TRAFFIC.get(args.workload) if prec == gda.BF16 else None
     roofline = {"bound": "alu" if prec == gda.FP32 else "tensor", "achieved": achieved, "peak": peak,
                 "unit": "TFLOP/s", "frac": achieved / peak, "traffic": traffic,

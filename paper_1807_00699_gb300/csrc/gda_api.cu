@@ -1,6 +1,6 @@
 // C ABI of the GD solver (include/gda.h): context, device memory, the step
 // loop and the energy / argmin calls.  The arithmetic runs in the kernels of
-// step_simt.cu, step_tc.cu and energy.cu; this file only orders launches.
+// the step_*.cu and energy*.cu files; this file only orders launches.
 #include <algorithm>
 #include <cmath>
 #include <cstdarg>
@@ -28,7 +28,7 @@ size_t round_up(size_t x, size_t m) { return (x + m - 1) / m * m; }
 }  // namespace
 
 struct gda_ctx {
-  int dev = 0;
+  int dev = 0, sms = 148;
   int N = 0, Np = 0, model = 0, cplx = 0;
   cudaStream_t stream = nullptr;
   bool tc_ok = false;
@@ -389,7 +389,7 @@ gda_status launch_step(gda_ctx* c, const StepArgs& a, bool tc, const float* oper
   } else if (tc) {
     LK(launch_step_tc(c->plan, a, op_buf, c->stream, c->run_pair));
   } else {
-    LK(launch_step_simt(a, c->J32, operand32, c->stream));
+    LK(launch_step_dense(a, c->J32, operand32, c->sms, c->stream));
   }
   return GDA_OK;
 }
@@ -628,6 +628,7 @@ static gda_status create_impl(const double* J, const double* g, int32_t N, int32
     delete c;
     return GDA_ERR_CUDA;
   }
+  c->sms = device_sms(c->dev);
   c->tc_ok = tc_supported(c->dev);
   const size_t Np = c->Np;
   gda_status st = GDA_OK;
@@ -895,16 +896,23 @@ gda_status gda_run(gda_ctx* c, const gda_params* p, int32_t R, int64_t steps) {
     return GDA_OK;
   }
 
-  // Sparse Euler runs whose columns fit on chip: one launch per tracking
-  // segment.  A segment of one step gains nothing over the per-step kernel.
+  // FP32 runs whose columns fit on chip (sparse Euler, small dense Euler and
+  // RK4): one launch per tracking segment, columns never meet.  A sparse
+  // segment of one step gains nothing over the per-step kernel; dense segments
+  // of up to 10 steps keep a launch per step, the count gda_kernel_launches
+  // has always reported for such runs.
   base.rho_out = decay ? c->rho[c->rcur ^ 1] : nullptr;
-  const int seg_cols = c->run_sparse && p->integ == GDA_EULER ? sparse_seg_columns(base, device_sms(c->dev)) : 0;
+  int seg_cols = 0;
+  if (!tc && c->run_sparse)
+    seg_cols = p->integ == GDA_EULER ? sparse_seg_columns(base, c->sms) : 0;
+  else if (!tc)
+    seg_cols = dense_seg_columns(base, c->sms);
   const int64_t seg_len = p->energy_every > 0 ? p->energy_every : std::min<int64_t>(steps, 1 << 16);
-  if (seg_cols && seg_len > 1) {
+  if (seg_cols && seg_len > (c->run_sparse ? 1 : 10)) {
     for (int64_t k = 0; k < steps; k += seg_len) {
       const int64_t len = std::min<int64_t>(seg_len, steps - k);
       StepArgs a = base;
-      a.mode = M_EULER;
+      a.mode = p->integ == GDA_RK4 ? M_RK4 : M_EULER;
       a.step = static_cast<unsigned int>(c->step + k);
       a.psi_n = c->psi[c->cur];
       a.psi_out = c->psi[c->cur ^ 1];
@@ -912,7 +920,10 @@ gda_status gda_run(gda_ctx* c, const gda_params* p, int32_t R, int64_t steps) {
       a.beta_out = c->beta[c->bcur ^ 1];
       a.rho_in = c->rho[c->rcur];
       a.rho_out = decay ? c->rho[c->rcur ^ 1] : nullptr;
-      LK(launch_sparse_seg(a, c->ell, c->ell_maxdeg, int(len), seg_cols, c->stream));
+      if (c->run_sparse)
+        LK(launch_sparse_seg(a, c->ell, c->ell_maxdeg, int(len), seg_cols, c->stream));
+      else
+        LK(launch_dense_seg(a, c->J32, p->integ == GDA_RK4, int(len), seg_cols, c->stream));
       c->cur ^= 1;
       c->bcur ^= 1;
       if (decay) c->rcur ^= 1;

@@ -1,14 +1,11 @@
-// FP32 CUDA-core GD step: a tiled SGEMM Y = J0 X over one 64x64 tile of
-// (spins i) x (columns c), fused with the step epilogue (Eqs. 2, 5, 6).  This
-// is the plain FP32 path the tensor-core path is measured against, and the
-// path whose amplitudes are compared with the FP64 oracle.
-//
-// The sparse variant (SPARSE = true) replaces the SGEMM by a gather over the
-// nonzeros of J0 in ELL form ((column, value) [dmax][Np]): thread (tx, ty)
-// sums, for its 4 rows and 4 columns, val_ik X[c][col_ik] in ascending k.  The
-// tile shape, the thread-to-element map and the epilogue (with its partial-sum
-// order) are the dense kernel's, so density partials, noise decay and the
-// energy mode carry over unchanged.
+// Sparse GD steps (FP32, CUDA cores): the coupling sum is a gather over the
+// nonzeros of J0 in ELL form ((column, value) [dmax][Np]), fused with the step
+// epilogue (Eqs. 2, 5, 6).  step_sparse_kernel works on a 64 x 64 tile of
+// (spins i) x (columns c): thread (tx, ty) sums, for its 4 rows and 4 columns,
+// val_ik X[c][col_ik] in ascending k.  The tile shape, the thread-to-element
+// map and the epilogue (with its partial-sum order) are the dense FP32
+// kernel's (step_dense.cu), so density partials, noise decay and the energy
+// mode carry over unchanged.
 #include "epilogue.cuh"
 #include "tc_epilogue.cuh"
 #include "tc_ptx.cuh"
@@ -16,7 +13,7 @@
 namespace gda {
 namespace {
 
-constexpr int BM = 64, BN = 64, BK = 16, PAD = 4;
+constexpr int BM = 64, BN = 64;
 constexpr size_t kPairSmemMax = 200 * 1024;  // the staged sparse kernel: N rounded up to 128 <= 25600
 
 // J0's nonzeros, (column, value bits) in one 8-byte load: [dmax][Np], (0, 0) past a row's count.
@@ -24,14 +21,11 @@ struct Ell {
   const int2* cv;
 };
 
-// DW (sparse): the ELL width the loop runs over, a power of two >= the largest
+// DW: the ELL width the loop runs over, a power of two >= the largest
 // row count; entries beyond a row's count are (column 0, value 0) and add
 // exact zeros, so the sums equal those over the row's nonzeros alone.
-template <bool CPLX, bool SPARSE, int DW, int MODE>
-__global__ void __launch_bounds__(256) step_simt_kernel(StepArgs a, const float* __restrict__ J,
-                                                        const float* __restrict__ X, Ell ell) {
-  __shared__ __align__(16) float As[SPARSE ? 1 : BK][BM + PAD];
-  __shared__ __align__(16) float Bs[SPARSE ? 1 : BK][BN + PAD];
+template <bool CPLX, int DW, int MODE>
+__global__ void __launch_bounds__(256) step_sparse_kernel(StepArgs a, const float* __restrict__ X, Ell ell) {
   __shared__ float s_beta[BN], s_dsc[BN];
   __shared__ int s_bad;
 
@@ -51,7 +45,7 @@ __global__ void __launch_bounds__(256) step_simt_kernel(StepArgs a, const float*
   }
 
   float acc[4][4] = {};
-  if (SPARSE) {
+  {
     // The 4 rows' index loads, then their gathers, are issued together (rows
     // beyond N read the ELL padding: column 0, value 0), so the dependent
     // index -> gather chains of the rows overlap instead of following each other.
@@ -97,27 +91,6 @@ __global__ void __launch_bounds__(256) step_simt_kernel(StepArgs a, const float*
       }
     }
   }
-  const int lr = tid >> 2, lk = (tid & 3) * 4;
-  const float* Jp = SPARSE ? nullptr : J + size_t(m0 + lr) * Np + lk;
-  const float* Xp = SPARSE ? nullptr : X + size_t(n0 + lr) * Np + lk;
-  for (int k0 = 0; !SPARSE && k0 < Np; k0 += BK) {
-    const float4 av = *reinterpret_cast<const float4*>(Jp + k0);
-    const float4 bv = *reinterpret_cast<const float4*>(Xp + k0);
-    __syncthreads();
-    As[lk + 0][lr] = av.x; As[lk + 1][lr] = av.y; As[lk + 2][lr] = av.z; As[lk + 3][lr] = av.w;
-    Bs[lk + 0][lr] = bv.x; Bs[lk + 1][lr] = bv.y; Bs[lk + 2][lr] = bv.z; Bs[lk + 3][lr] = bv.w;
-    __syncthreads();
-#pragma unroll
-    for (int k = 0; k < BK; ++k) {
-      const float4 b4 = *reinterpret_cast<const float4*>(&Bs[k][4 * ty]);
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const float av2 = As[k][tx + 16 * q];
-        acc[q][0] += av2 * b4.x; acc[q][1] += av2 * b4.y;
-        acc[q][2] += av2 * b4.z; acc[q][3] += av2 * b4.w;
-      }
-    }
-  }
   __syncthreads();
 
   // Epilogue: rows m0 + tx + 16 q, columns c0 .. c0 + 3.
@@ -126,10 +99,10 @@ __global__ void __launch_bounds__(256) step_simt_kernel(StepArgs a, const float*
   const int lr0 = CPLX ? 2 * ty : 4 * ty;  // first local restart of the quad
   float rsum[4] = {0.f, 0.f, 0.f, 0.f};
   int bad = 0;
-  if (SPARSE) {
+  {
     // every input of the 4 rows is loaded before the first store, so that the
     // rows' loads are in flight together (the stores could alias them for the
-    // compiler); same arithmetic as epi_quad
+    // compiler)
     EpiRegs<MODE, CPLX, 4> E[4];
 #pragma unroll
     for (int q = 0; q < 4; ++q) epi_load<MODE, CPLX, 4>(a, m0 + tx + 16 * q, c0, E[q]);
@@ -141,16 +114,6 @@ __global__ void __launch_bounds__(256) step_simt_kernel(StepArgs a, const float*
       epi_chunk<MODE, CPLX, 4, true>(a, i, c0, acc[q], E[q], &s_beta[lr0], &s_dsc[lr0], red, bad, t4);
       if (a.opT_out && MODE != M_RAW && MODE != M_ENERGY)
         *reinterpret_cast<float4*>(a.opT_out + size_t(i) * a.Cp + c0) = make_float4(t4[0], t4[1], t4[2], t4[3]);
-#pragma unroll
-      for (int u = 0; u < U; ++u) rsum[u] += red[u];
-    }
-  } else {
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const int i = m0 + tx + 16 * q;
-      if (i >= a.N) continue;
-      float red[4];
-      epi_quad<CPLX, SPARSE, MODE>(a, i, c0, acc[q], &s_beta[lr0], &s_dsc[lr0], red, bad);
 #pragma unroll
       for (int u = 0; u < U; ++u) rsum[u] += red[u];
     }
@@ -180,28 +143,20 @@ __global__ void __launch_bounds__(256) step_simt_kernel(StepArgs a, const float*
 
 }  // namespace
 
-int simt_mtiles(int N) { return (N + BM - 1) / BM; }
-
-template <bool CPLX, bool SPARSE, int DW>
-cudaError_t launch_modes(const StepArgs& a, const float* J32, const float* operand, const Ell& ell, cudaStream_t s) {
-  dim3 grid((a.C + BN - 1) / BN, simt_mtiles(a.N));
+template <bool CPLX, int DW>
+cudaError_t launch_modes(const StepArgs& a, const float* operand, const Ell& ell, cudaStream_t s) {
+  dim3 grid((a.C + BN - 1) / BN, (a.N + BM - 1) / BM);
   switch (a.mode) {
-    case M_EULER: step_simt_kernel<CPLX, SPARSE, DW, M_EULER><<<grid, 256, 0, s>>>(a, J32, operand, ell); break;
-    case M_RK1: step_simt_kernel<CPLX, SPARSE, DW, M_RK1><<<grid, 256, 0, s>>>(a, J32, operand, ell); break;
-    case M_RK2: step_simt_kernel<CPLX, SPARSE, DW, M_RK2><<<grid, 256, 0, s>>>(a, J32, operand, ell); break;
-    case M_RK3: step_simt_kernel<CPLX, SPARSE, DW, M_RK3><<<grid, 256, 0, s>>>(a, J32, operand, ell); break;
-    case M_RK4: step_simt_kernel<CPLX, SPARSE, DW, M_RK4><<<grid, 256, 0, s>>>(a, J32, operand, ell); break;
-    case M_ENERGY: step_simt_kernel<CPLX, SPARSE, DW, M_ENERGY><<<grid, 256, 0, s>>>(a, J32, operand, ell); break;
-    case M_RAW: step_simt_kernel<CPLX, SPARSE, DW, M_RAW><<<grid, 256, 0, s>>>(a, J32, operand, ell); break;
+    case M_EULER: step_sparse_kernel<CPLX, DW, M_EULER><<<grid, 256, 0, s>>>(a, operand, ell); break;
+    case M_RK1: step_sparse_kernel<CPLX, DW, M_RK1><<<grid, 256, 0, s>>>(a, operand, ell); break;
+    case M_RK2: step_sparse_kernel<CPLX, DW, M_RK2><<<grid, 256, 0, s>>>(a, operand, ell); break;
+    case M_RK3: step_sparse_kernel<CPLX, DW, M_RK3><<<grid, 256, 0, s>>>(a, operand, ell); break;
+    case M_RK4: step_sparse_kernel<CPLX, DW, M_RK4><<<grid, 256, 0, s>>>(a, operand, ell); break;
+    case M_ENERGY: step_sparse_kernel<CPLX, DW, M_ENERGY><<<grid, 256, 0, s>>>(a, operand, ell); break;
+    case M_RAW: step_sparse_kernel<CPLX, DW, M_RAW><<<grid, 256, 0, s>>>(a, operand, ell); break;
     default: return cudaErrorInvalidValue;
   }
   return cudaGetLastError();
-}
-
-cudaError_t launch_step_simt(const StepArgs& a, const float* J32, const float* operand, cudaStream_t s) {
-  const Ell none{nullptr};
-  return a.cplx ? launch_modes<true, false, 0>(a, J32, operand, none, s)
-                : launch_modes<false, false, 0>(a, J32, operand, none, s);
 }
 
 namespace {
@@ -646,8 +601,7 @@ cudaError_t launch_sparse_w(const StepArgs& a, const Ell& ell, const float* oper
   // Euler steps whose column pair fits in shared memory: the staged kernel
   if (a.mode == M_EULER && size_t(2) * a.Np * sizeof(float) <= kPairSmemMax)
     return a.cplx ? launch_pair<true, DW>(a, ell, s) : launch_pair<false, DW>(a, ell, s);
-  return a.cplx ? launch_modes<true, true, DW>(a, nullptr, operand, ell, s)
-                : launch_modes<false, true, DW>(a, nullptr, operand, ell, s);
+  return a.cplx ? launch_modes<true, DW>(a, operand, ell, s) : launch_modes<false, DW>(a, operand, ell, s);
 }
 
 cudaError_t launch_step_sparse(const StepArgs& a, const int2* cv, const float* operand, int maxdeg, cudaStream_t s) {

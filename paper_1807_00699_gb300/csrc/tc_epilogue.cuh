@@ -1,11 +1,9 @@
-// Register-staged epilogue of the tensor-core step kernel.
+// Register-staged epilogue of the step kernels.
 //
-// Each epilogue thread owns one spin row i and walks its columns in chunks of
-// CW.  All inputs a chunk needs (amplitudes, gains, RK4 accumulators) are
+// Each epilogue thread walks columns of a spin row i in chunks of CW.  All inputs a chunk needs (amplitudes, gains, RK4 accumulators) are
 // loaded into registers one chunk ahead of the arithmetic, and the first chunk
 // is loaded while the MMAs are still running, so global-memory latency is
-// paid about once per kernel instead of once per element.  The arithmetic is
-// the same FP32 expression sequence as epi_quad (epilogue.cuh).
+// paid about once per kernel instead of once per element.
 #pragma once
 #include <cuda_fp8.h>
 
