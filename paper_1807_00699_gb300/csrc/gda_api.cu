@@ -826,7 +826,7 @@ gda_status gda_run(gda_ctx* c, const gda_params* p, int32_t R, int64_t steps) {
       a.step = static_cast<unsigned int>(c->step + k);
       a.psi_n = c->psi[c->cur];
       a.xs = c->psi[c->cur];
-      a.psi_out = c->psi[c->cur ^ 1];
+      a.psi_out = c->psi[c->cur];  // in place: an amplitude is read and written by one thread only
       a.beta_in = c->beta[c->bcur];
       a.beta_out = c->beta[c->bcur ^ 1];
       a.rho_in = c->rho[c->rcur];
@@ -836,8 +836,7 @@ gda_status gda_run(gda_ctx* c, const gda_params* p, int32_t R, int64_t steps) {
       g.buf0 = c->opcur;
       g.Cp = c->Cp;
       g.flags = c->seg_flags;
-      g.psi[0] = c->psi[c->cur];
-      g.psi[1] = c->psi[c->cur ^ 1];
+      g.psi = c->psi[c->cur];
       g.beta[0] = c->beta[c->bcur];
       g.beta[1] = c->beta[c->bcur ^ 1];
       g.rho[0] = c->rho[c->rcur];
@@ -847,7 +846,6 @@ gda_status gda_run(gda_ctx* c, const gda_params* p, int32_t R, int64_t steps) {
       CK(cudaMemsetAsync(c->seg_flags, 0, nflags * sizeof(unsigned), c->stream));
       LK(f8 ? launch_step_tcs8(c->plan8, a, g, c->stream, c->run_pair)
             : launch_step_tcs(c->plan, a, g, c->stream, c->run_pair));
-      c->cur ^= flip;
       c->bcur ^= flip;
       c->opcur ^= flip;
       if (decay) c->rcur ^= flip;

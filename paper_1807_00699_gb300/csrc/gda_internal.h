@@ -119,8 +119,8 @@ struct SegArgs {
   int buf0;                 // operand buffer holding the first step's operand
   int Cp;                   // rows of one operand buffer
   unsigned* flags;          // [column blocks][128-row blocks], zero at launch
-  float* psi[2];            // psi[0]: the first step's amplitudes; alternate per step
-  float* beta[2];           // likewise the coupling scales
+  float* psi;               // the amplitudes, updated in place
+  float* beta[2];           // beta[0]: the first step's coupling scales; alternate per step
   float* rho[2];            // likewise the density partial sums (noise decay)
   __nv_bfloat16* ops;       // BF16 operand buffers [2][Cp][Np] (or nullptr)
   unsigned char* ops8;      // E4M3 operand buffers [2][Cp][Np] (FP8 path, or nullptr)

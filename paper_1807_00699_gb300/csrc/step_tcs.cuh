@@ -243,9 +243,9 @@ __global__ void __launch_bounds__(TcThreads<M_EULER>::N, 1)
       if (e == 0) {
         StepArgs sa = a0;
         sa.step = a0.step + unsigned(n);
-        sa.psi_n = g.psi[n & 1];
-        sa.xs = g.psi[n & 1];
-        sa.psi_out = g.psi[(n + 1) & 1];
+        sa.psi_n = g.psi;
+        sa.xs = g.psi;
+        sa.psi_out = g.psi;
         sa.beta_in = g.beta[n & 1];
         sa.beta_out = g.beta[(n + 1) & 1];
         sa.rho_in = g.rho[n & 1];
