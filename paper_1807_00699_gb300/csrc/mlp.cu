@@ -16,156 +16,235 @@ constexpr int DIN = GDA_MLP_IN, DH = GDA_MLP_HIDDEN, DOUT = GDA_MLP_OUT;
 constexpr int O_W1 = 0, O_B1 = O_W1 + DH * DIN, O_W2 = O_B1 + DH, O_B2 = O_W2 + DH * DH, O_W3 = O_B2 + DH,
               O_B3 = O_W3 + DOUT * DH, P_TOTAL = O_B3 + DOUT;
 static_assert(P_TOTAL == GDA_MLP_PARAMS, "parameter count");
-constexpr int ROWS = 128;  // rows (spins) per block
+constexpr int ROWS = 64;     // rows (spins) per block
+constexpr int THREADS = 256;
+constexpr int LR = ROWS + 4;  // floats per unit of an activation array [unit][row]
+constexpr int LU = DH + 4;    // floats per row of an array [row][unit], per input of W2 transposed
 
-// Shared memory of the forward / backward kernels: all weights, plus the
-// block's hidden activations stored [unit][row] so that thread t (row t)
-// reads a column without bank conflicts.
-struct MlpSmem {
-  float W1[DH * DIN], b1[DH], W2[DH * DH], b2[DH], W3[DOUT * DH], b3[DOUT];
-  float H1[DH][ROWS + 1];
-  float H2[DH][ROWS + 1];
+// Four consecutive floats.
+__device__ __forceinline__ float4 ld4(const float* p) { return *reinterpret_cast<const float4*>(p); }
+
+// The hidden layers are 128 x 128 products over a block's 64 rows, held in
+// shared memory: a thread owns 4 x 8 (backward also 8 x 8) outputs, so a step
+// of the inner dimension costs 12 loaded values for 32 FMAs.  (One thread per
+// row with a load of W and of H per FMA, and every block's threads striding
+// through W2, took 111 us forward and 193 us backward on 10 000 rows.)
+// Every output sums in the order of the plain loop: bias first, inputs ascending.
+struct FwdSmem {
+  float W1[DH * DIN], b1[DH], b2[DH], W3[DOUT * DH], b3[DOUT + 3];
+  float X[ROWS * DIN];
+  float W2t[DH * LU];  // [input k][unit j]
+  float H1[DH * LR];   // [unit][row]
+  float H2[DH * LR];
 };
-
-__device__ void load_params(MlpSmem& s, const float* __restrict__ p) {
-  for (int k = threadIdx.x; k < DH * DIN; k += blockDim.x) s.W1[k] = p[O_W1 + k];
-  for (int k = threadIdx.x; k < DH; k += blockDim.x) s.b1[k] = p[O_B1 + k];
-  for (int k = threadIdx.x; k < DH * DH; k += blockDim.x) s.W2[k] = p[O_W2 + k];
-  for (int k = threadIdx.x; k < DH; k += blockDim.x) s.b2[k] = p[O_B2 + k];
-  for (int k = threadIdx.x; k < DOUT * DH; k += blockDim.x) s.W3[k] = p[O_W3 + k];
-  for (int k = threadIdx.x; k < DOUT; k += blockDim.x) s.b3[k] = p[O_B3 + k];
-}
 
 // Forward for ROWS rows per block; H (optional) caches h1, h2 for backward as
 // [row][2*DH].
-__global__ void __launch_bounds__(ROWS) k_mlp_forward(const float* __restrict__ p, const float* __restrict__ X, int M,
-                                                      float* __restrict__ O, float* __restrict__ H) {
+__global__ void __launch_bounds__(THREADS) k_mlp_forward(const float* __restrict__ p, const float* __restrict__ X,
+                                                         int M, float* __restrict__ O, float* __restrict__ H) {
   extern __shared__ __align__(16) unsigned char raw[];
-  MlpSmem& s = *reinterpret_cast<MlpSmem*>(raw);
-  load_params(s, p);
-  __syncthreads();
+  FwdSmem& s = *reinterpret_cast<FwdSmem*>(raw);
   const int t = threadIdx.x;
-  const int m = blockIdx.x * ROWS + t;
-  float x[DIN];
-#pragma unroll
-  for (int k = 0; k < DIN; ++k) x[k] = m < M ? X[size_t(m) * DIN + k] : 0.0f;
-  for (int j = 0; j < DH; ++j) {
-    float a = s.b1[j];
-#pragma unroll
-    for (int k = 0; k < DIN; ++k) a = fmaf(s.W1[j * DIN + k], x[k], a);
-    s.H1[j][t] = fmaxf(a, 0.0f);
+  const int m0 = blockIdx.x * ROWS;
+  for (int q = t; q < DH * DH / 4; q += THREADS) {  // W2 [j][k] -> [k][j], 4 units at a time: 4-way store conflicts at most
+    const int k = q & 127, j = (q >> 7) * 4;
+    *reinterpret_cast<float4*>(&s.W2t[k * LU + j]) =
+        make_float4(p[O_W2 + j * DH + k], p[O_W2 + (j + 1) * DH + k], p[O_W2 + (j + 2) * DH + k],
+                    p[O_W2 + (j + 3) * DH + k]);
   }
-  float o[DOUT];
-#pragma unroll
-  for (int k = 0; k < DOUT; ++k) o[k] = s.b3[k];
-  for (int j = 0; j < DH; ++j) {
-    float a = s.b2[j];
-    for (int k = 0; k < DH; ++k) a = fmaf(s.W2[j * DH + k], s.H1[k][t], a);
-    a = fmaxf(a, 0.0f);
-    s.H2[j][t] = a;
-#pragma unroll
-    for (int k = 0; k < DOUT; ++k) o[k] = fmaf(s.W3[k * DH + j], a, o[k]);
+  for (int k = t; k < DH * DIN; k += THREADS) s.W1[k] = p[O_W1 + k];
+  for (int k = t; k < DH; k += THREADS) {
+    s.b1[k] = p[O_B1 + k];
+    s.b2[k] = p[O_B2 + k];
   }
-  if (m < M) {
+  for (int k = t; k < DOUT * DH; k += THREADS) s.W3[k] = p[O_W3 + k];
+  if (t < DOUT) s.b3[t] = p[O_B3 + t];
+  for (int k = t; k < ROWS * DIN; k += THREADS)
+    s.X[k] = size_t(m0) * DIN + k < size_t(M) * DIN ? X[size_t(m0) * DIN + k] : 0.0f;
+  __syncthreads();
+  {  // layer 1: thread = row r, a quarter of the units
+    const int r = t & 63;
+    float x[DIN];
 #pragma unroll
-    for (int k = 0; k < DOUT; ++k) O[size_t(m) * DOUT + k] = o[k];
-    if (H) {
-      for (int j = 0; j < DH; ++j) {
-        H[size_t(m) * 2 * DH + j] = s.H1[j][t];
-        H[size_t(m) * 2 * DH + DH + j] = s.H2[j][t];
+    for (int k = 0; k < DIN; ++k) x[k] = s.X[r * DIN + k];
+    for (int j = (t >> 6) * (DH / 4); j < (t >> 6) * (DH / 4) + DH / 4; ++j) {
+      float a = s.b1[j];
+#pragma unroll
+      for (int k = 0; k < DIN; ++k) a = fmaf(s.W1[j * DIN + k], x[k], a);
+      s.H1[j * LR + r] = fmaxf(a, 0.0f);
+    }
+  }
+  __syncthreads();
+  {  // layer 2: thread = 4 rows x 8 units
+    const int r0 = (t & 15) * 4, j0 = (t >> 4) * 8;
+    float acc[8][4];
+#pragma unroll
+    for (int v = 0; v < 8; ++v)
+#pragma unroll
+      for (int u = 0; u < 4; ++u) acc[v][u] = s.b2[j0 + v];
+#pragma unroll 4
+    for (int k = 0; k < DH; ++k) {
+      const float4 h = ld4(&s.H1[k * LR + r0]);
+      const float4 wa = ld4(&s.W2t[k * LU + j0]), wb = ld4(&s.W2t[k * LU + j0 + 4]);
+      const float w[8] = {wa.x, wa.y, wa.z, wa.w, wb.x, wb.y, wb.z, wb.w};
+#pragma unroll
+      for (int v = 0; v < 8; ++v) {
+        acc[v][0] = fmaf(w[v], h.x, acc[v][0]);
+        acc[v][1] = fmaf(w[v], h.y, acc[v][1]);
+        acc[v][2] = fmaf(w[v], h.z, acc[v][2]);
+        acc[v][3] = fmaf(w[v], h.w, acc[v][3]);
       }
     }
+#pragma unroll
+    for (int v = 0; v < 8; ++v)
+      *reinterpret_cast<float4*>(&s.H2[(j0 + v) * LR + r0]) = make_float4(
+          fmaxf(acc[v][0], 0.0f), fmaxf(acc[v][1], 0.0f), fmaxf(acc[v][2], 0.0f), fmaxf(acc[v][3], 0.0f));
+  }
+  __syncthreads();
+  for (int q = t; q < ROWS * DOUT; q += THREADS) {  // layer 3: thread = one output of one row
+    const int r = q & 63, k = q >> 6;
+    float a = s.b3[k];
+#pragma unroll 8
+    for (int j = 0; j < DH; ++j) a = fmaf(s.W3[k * DH + j], s.H2[j * LR + r], a);
+    if (m0 + r < M) O[size_t(m0 + r) * DOUT + k] = a;
+  }
+  if (H)
+    for (int q = t; q < ROWS * 2 * DH; q += THREADS) {
+      const int r = q >> 8, j = q & 255;
+      if (m0 + r < M) H[size_t(m0 + r) * 2 * DH + j] = j < DH ? s.H1[j * LR + r] : s.H2[(j - DH) * LR + r];
+    }
+}
+
+struct BwdSmem {
+  float W2[DH * DH], W3[DOUT * DH];
+  float H1[ROWS * LU];   // [row][unit]; later dh1
+  float H2[ROWS * LU];   // [row][unit]; later dh2
+  float dO[ROWS * DOUT], X[ROWS * DIN];
+};
+
+// g[0..3] += v in one 16-byte reduction (g 16-byte aligned), or one by one.
+__device__ __forceinline__ void add4(float* g, const float* v, bool aligned) {
+  if (aligned) {
+    asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(g), "f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3])
+                 : "memory");
+  } else {
+    for (int k = 0; k < 4; ++k) atomicAdd(g + k, v[k]);
   }
 }
 
 // Backward for ROWS rows per block: accumulates the parameter gradient of
 // sum_m dO[m] . O[m] into G (atomics across blocks).
-__global__ void __launch_bounds__(ROWS) k_mlp_backward(const float* __restrict__ p, const float* __restrict__ X,
-                                                       const float* __restrict__ H, const float* __restrict__ dO,
-                                                       int M, float* __restrict__ G) {
+__global__ void __launch_bounds__(THREADS) k_mlp_backward(const float* __restrict__ p, const float* __restrict__ X,
+                                                          const float* __restrict__ H, const float* __restrict__ dO,
+                                                          int M, float* __restrict__ G) {
   extern __shared__ __align__(16) unsigned char raw[];
-  MlpSmem& s = *reinterpret_cast<MlpSmem*>(raw);
-  __shared__ float sdO[DOUT][ROWS];
-  __shared__ float sX[DIN][ROWS];
-  load_params(s, p);
+  BwdSmem& s = *reinterpret_cast<BwdSmem*>(raw);
   const int t = threadIdx.x;
-  const int m = blockIdx.x * ROWS + t;
-  const bool live = m < M;
-  for (int j = 0; j < DH; ++j) {
-    s.H1[j][t] = live ? H[size_t(m) * 2 * DH + j] : 0.0f;
-    s.H2[j][t] = live ? H[size_t(m) * 2 * DH + DH + j] : 0.0f;
+  const int m0 = blockIdx.x * ROWS;
+  for (int k = t; k < DH * DH; k += THREADS) s.W2[k] = p[O_W2 + k];
+  for (int k = t; k < DOUT * DH; k += THREADS) s.W3[k] = p[O_W3 + k];
+  for (int q = t; q < ROWS * 2 * DH; q += THREADS) {
+    const int r = q >> 8, j = q & 255;
+    const float v = m0 + r < M ? H[size_t(m0 + r) * 2 * DH + j] : 0.0f;
+    (j < DH ? s.H1 : s.H2)[r * LU + (j & 127)] = v;
   }
-#pragma unroll
-  for (int k = 0; k < DOUT; ++k) sdO[k][t] = live ? dO[size_t(m) * DOUT + k] : 0.0f;
-#pragma unroll
-  for (int k = 0; k < DIN; ++k) sX[k][t] = live ? X[size_t(m) * DIN + k] : 0.0f;
+  for (int k = t; k < ROWS * DOUT; k += THREADS)
+    s.dO[k] = size_t(m0) * DOUT + k < size_t(M) * DOUT ? dO[size_t(m0) * DOUT + k] : 0.0f;
+  for (int k = t; k < ROWS * DIN; k += THREADS)
+    s.X[k] = size_t(m0) * DIN + k < size_t(M) * DIN ? X[size_t(m0) * DIN + k] : 0.0f;
   __syncthreads();
-  // layer 3: dW3[k][j] = sum_t dO[t][k] h2[t][j], db3[k] = sum_t dO[t][k]
-  {
-    const int j = t;
-    for (int k = 0; k < DOUT; ++k) {
-      float a = 0.0f;
-      for (int r = 0; r < ROWS; ++r) a = fmaf(sdO[k][r], s.H2[j][r], a);
-      atomicAdd(&G[O_W3 + k * DH + j], a);
-    }
-    if (t < DOUT) {
-      float a = 0.0f;
-      for (int r = 0; r < ROWS; ++r) a += sdO[t][r];
-      atomicAdd(&G[O_B3 + t], a);
-    }
+  // layer 3: dW3[k][j] = sum_r dO[r][k] h2[r][j], db3[k] = sum_r dO[r][k]
+  for (int q = t; q < DOUT * DH; q += THREADS) {
+    const int k = q >> 7, j = q & 127;
+    float a = 0.0f;
+#pragma unroll 8
+    for (int r = 0; r < ROWS; ++r) a = fmaf(s.dO[r * DOUT + k], s.H2[r * LU + j], a);
+    atomicAdd(&G[O_W3 + q], a);
+  }
+  if (t < DOUT) {
+    float a = 0.0f;
+    for (int r = 0; r < ROWS; ++r) a += s.dO[r * DOUT + t];
+    atomicAdd(&G[O_B3 + t], a);
   }
   __syncthreads();
-  // dh2 = (W3^T dO) * relu'(h2), in place of H2 (the h2 values are no longer needed)
-  for (int j = 0; j < DH; ++j) {
+  // dh2 = (W3^T dO) * relu'(h2), in place of h2
+  for (int q = t; q < ROWS * DH; q += THREADS) {
+    const int r = q >> 7, j = q & 127;
     float a = 0.0f;
 #pragma unroll
-    for (int k = 0; k < DOUT; ++k) a = fmaf(s.W3[k * DH + j], sdO[k][t], a);
-    s.H2[j][t] = s.H2[j][t] > 0.0f ? a : 0.0f;
+    for (int k = 0; k < DOUT; ++k) a = fmaf(s.W3[k * DH + j], s.dO[r * DOUT + k], a);
+    s.H2[r * LU + j] = s.H2[r * LU + j] > 0.0f ? a : 0.0f;
   }
   __syncthreads();
-  // layer 2: dW2[j][k] = sum_t dh2[t][j] h1[t][k], db2[j] = sum_t dh2[t][j]
+  // layer 2: dW2[j][k] = sum_r dh2[r][j] h1[r][k], thread = 8 j x 8 k (two groups of 4, 64 apart)
+  const bool al = (reinterpret_cast<uintptr_t>(G) & 15) == 0;
   {
-    const int j = t;
-    float db = 0.0f;
-    for (int r = 0; r < ROWS; ++r) db += s.H2[j][r];
-    atomicAdd(&G[O_B2 + j], db);
-    for (int k0 = 0; k0 < DH; k0 += 32) {
-      float acc[32];
-#pragma unroll
-      for (int q = 0; q < 32; ++q) acc[q] = 0.0f;
-      for (int r = 0; r < ROWS; ++r) {
-        const float d = s.H2[j][r];
-#pragma unroll
-        for (int q = 0; q < 32; ++q) acc[q] = fmaf(d, s.H1[k0 + q][r], acc[q]);
-      }
-#pragma unroll
-      for (int q = 0; q < 32; ++q) atomicAdd(&G[O_W2 + j * DH + k0 + q], acc[q]);
-    }
-  }
-  // dh1 = (W2^T dh2) * relu'(h1), row t, written over h1 (column t only)
-  __syncthreads();
-  for (int k = 0; k < DH; ++k) {
-    float a = 0.0f;
-    for (int j = 0; j < DH; ++j) a = fmaf(s.W2[j * DH + k], s.H2[j][t], a);
-    s.H1[k][t] = s.H1[k][t] > 0.0f ? a : 0.0f;
-  }
-  __syncthreads();
-  // layer 1: dW1[j][k] = sum_t dh1[t][j] x[t][k], db1[j] = sum_t dh1[t][j]
-  {
-    const int j = t;
-    float acc[DIN];
-#pragma unroll
-    for (int k = 0; k < DIN; ++k) acc[k] = 0.0f;
-    float db = 0.0f;
+    const int k0 = (t & 15) * 4, j0 = (t >> 4) * 8;
+    float acc[8][8] = {};
+#pragma unroll 2
     for (int r = 0; r < ROWS; ++r) {
-      const float d = s.H1[j][r];
-      db += d;
+      const float4 da = ld4(&s.H2[r * LU + j0]), db = ld4(&s.H2[r * LU + j0 + 4]);
+      const float4 ha = ld4(&s.H1[r * LU + k0]), hb = ld4(&s.H1[r * LU + k0 + 64]);
+      const float d[8] = {da.x, da.y, da.z, da.w, db.x, db.y, db.z, db.w};
+      const float h[8] = {ha.x, ha.y, ha.z, ha.w, hb.x, hb.y, hb.z, hb.w};
 #pragma unroll
-      for (int k = 0; k < DIN; ++k) acc[k] = fmaf(d, sX[k][r], acc[k]);
+      for (int v = 0; v < 8; ++v)
+#pragma unroll
+        for (int u = 0; u < 8; ++u) acc[v][u] = fmaf(d[v], h[u], acc[v][u]);
     }
 #pragma unroll
-    for (int k = 0; k < DIN; ++k) atomicAdd(&G[O_W1 + j * DIN + k], acc[k]);
-    atomicAdd(&G[O_B1 + j], db);
+    for (int v = 0; v < 8; ++v) {
+      add4(&G[O_W2 + (j0 + v) * DH + k0], &acc[v][0], al);
+      add4(&G[O_W2 + (j0 + v) * DH + k0 + 64], &acc[v][4], al);
+    }
+  }
+  if (t < DH) {
+    float db = 0.0f;
+#pragma unroll 8
+    for (int r = 0; r < ROWS; ++r) db += s.H2[r * LU + t];
+    atomicAdd(&G[O_B2 + t], db);
+  }
+  __syncthreads();
+  // dh1 = (W2^T dh2) * relu'(h1), in place of h1: thread = 4 rows (16 apart) x 8 units
+  {
+    const int r0 = t >> 4, k0 = (t & 15) * 4;
+    float acc[4][8] = {};
+#pragma unroll 2
+    for (int j = 0; j < DH; ++j) {
+      const float4 wa = ld4(&s.W2[j * DH + k0]), wb = ld4(&s.W2[j * DH + k0 + 64]);
+      const float w[8] = {wa.x, wa.y, wa.z, wa.w, wb.x, wb.y, wb.z, wb.w};
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const float d = s.H2[(r0 + 16 * u) * LU + j];
+#pragma unroll
+        for (int v = 0; v < 8; ++v) acc[u][v] = fmaf(w[v], d, acc[u][v]);
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+#pragma unroll
+      for (int v = 0; v < 8; ++v) {
+        float& h = s.H1[(r0 + 16 * u) * LU + k0 + (v & 3) + (v >> 2) * 64];
+        h = h > 0.0f ? acc[u][v] : 0.0f;
+      }
+  }
+  __syncthreads();
+  // layer 1: dW1[j][k] = sum_r dh1[r][j] x[r][k], db1[j] = sum_r dh1[r][j]; thread = unit j, half of the inputs
+  {
+    const int j = t & 127, k0 = (t >> 7) * 4;
+    float acc[4] = {}, db = 0.0f;
+#pragma unroll 8
+    for (int r = 0; r < ROWS; ++r) {
+      const float d = s.H1[r * LU + j];
+      const float4 x = ld4(&s.X[r * DIN + k0]);
+      db += d;
+      acc[0] = fmaf(d, x.x, acc[0]);
+      acc[1] = fmaf(d, x.y, acc[1]);
+      acc[2] = fmaf(d, x.z, acc[2]);
+      acc[3] = fmaf(d, x.w, acc[3]);
+    }
+    add4(&G[O_W1 + j * DIN + k0], acc, al);
+    if (k0 == 0) atomicAdd(&G[O_B1 + j], db);
   }
 }
 
@@ -410,14 +489,14 @@ extern "C" gda_status gda_mlp_forward(const float* params, const float* X, int32
                                       void* stream) {
   if (!params || !X || !O || M < 0) return GDA_ERR_INVALID;
   if (M == 0) return GDA_OK;
-  const size_t smem = sizeof(MlpSmem);
+  const size_t smem = sizeof(FwdSmem);
   static bool set = false;
   if (!set) {
     if (cudaFuncSetAttribute(k_mlp_forward, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)) != cudaSuccess)
       return GDA_ERR_CUDA;
     set = true;
   }
-  k_mlp_forward<<<(M + ROWS - 1) / ROWS, ROWS, smem, static_cast<cudaStream_t>(stream)>>>(params, X, M, O, H);
+  k_mlp_forward<<<(M + ROWS - 1) / ROWS, THREADS, smem, static_cast<cudaStream_t>(stream)>>>(params, X, M, O, H);
   return cudaGetLastError() == cudaSuccess ? GDA_OK : GDA_ERR_CUDA;
 }
 
@@ -425,14 +504,14 @@ extern "C" gda_status gda_mlp_backward(const float* params, const float* X, cons
                                        int32_t M, float* G, void* stream) {
   if (!params || !X || !H || !dO || !G || M < 0) return GDA_ERR_INVALID;
   if (M == 0) return GDA_OK;
-  const size_t smem = sizeof(MlpSmem);
+  const size_t smem = sizeof(BwdSmem);
   static bool set = false;
   if (!set) {
     if (cudaFuncSetAttribute(k_mlp_backward, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)) != cudaSuccess)
       return GDA_ERR_CUDA;
     set = true;
   }
-  k_mlp_backward<<<(M + ROWS - 1) / ROWS, ROWS, smem, static_cast<cudaStream_t>(stream)>>>(params, X, H, dO, M, G);
+  k_mlp_backward<<<(M + ROWS - 1) / ROWS, THREADS, smem, static_cast<cudaStream_t>(stream)>>>(params, X, H, dO, M, G);
   return cudaGetLastError() == cudaSuccess ? GDA_OK : GDA_ERR_CUDA;
 }
 
