@@ -161,6 +161,7 @@ __device__ __forceinline__ bool epi_unit(const BatchArgs& b, const BatchInst& I,
 #pragma unroll
   for (int p = 1; p <= PF && p < NCH; ++p) epi_prefetch_l2<M_EULER, CPLX, CW>(a, i, cbeg + p * CW, lane);
   EpiRegs<M_EULER, CPLX, CW> R[2];
+  const float h = epi_drive(a, i);
   epi_load<M_EULER, CPLX, CW>(a, i, cbeg, R[0]);  // own rows of psi and gamma: written by this thread
   bool fok = true;
   if (e < RPT) {
@@ -187,7 +188,7 @@ __device__ __forceinline__ bool epi_unit(const BatchArgs& b, const BatchInst& I,
     tmem_ld<CW>(taddr + ch * CW, v);
     const int lr0 = (part * PW + ch * CW) / W;
     float red[CW / W];
-    epi_chunk<M_EULER, CPLX, CW>(a, i, cbeg + ch * CW, v, cr, &s_beta[lr0], &s_dsc[lr0], red, bad);
+    epi_chunk<M_EULER, CPLX, CW>(a, i, cbeg + ch * CW, v, cr, h, &s_beta[lr0], &s_dsc[lr0], red, bad);
   };
 #pragma unroll 1
   for (int ch = 0; ch + 1 < NCH; ch += 2) {

@@ -188,7 +188,7 @@ __global__ void __launch_bounds__(128, RT == 8 ? 2 : ModeTraits<MODE>::rk_mid ? 
         float y[4];
         unpack2(acc[q0 + q][2 * g], y[0], y[1]);
         unpack2(acc[q0 + q][2 * g + 1], y[2], y[3]);
-        epi_chunk<MODE, CPLX, 4>(a, m0 + lx + LX * (q0 + q), c0, y, E[q], &s_beta[lr0], &s_dsc[lr0], red[q0 + q], bad);
+        epi_chunk<MODE, CPLX, 4>(a, m0 + lx + LX * (q0 + q), c0, y, E[q], epi_drive(a, m0 + lx + LX * (q0 + q)), &s_beta[lr0], &s_dsc[lr0], red[q0 + q], bad);
       }
     }
     if (out) {  // rows t + 16 p summed over p = 0 .. 3, then a tree over the 16 t

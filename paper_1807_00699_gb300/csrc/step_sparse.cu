@@ -111,7 +111,7 @@ __global__ void __launch_bounds__(256) step_sparse_kernel(StepArgs a, const floa
       const int i = m0 + tx + 16 * q;
       if (i >= a.N) continue;
       float red[4] = {0.f, 0.f, 0.f, 0.f}, t4[4];
-      epi_chunk<MODE, CPLX, 4, true>(a, i, c0, acc[q], E[q], &s_beta[lr0], &s_dsc[lr0], red, bad, t4);
+      epi_chunk<MODE, CPLX, 4, true>(a, i, c0, acc[q], E[q], epi_drive(a, i), &s_beta[lr0], &s_dsc[lr0], red, bad, t4);
       if (a.opT_out && MODE != M_RAW && MODE != M_ENERGY)
         *reinterpret_cast<float4*>(a.opT_out + size_t(i) * a.Cp + c0) = make_float4(t4[0], t4[1], t4[2], t4[3]);
 #pragma unroll

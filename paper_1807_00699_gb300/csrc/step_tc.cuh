@@ -256,6 +256,7 @@ __global__ void __launch_bounds__(TcThreads<MODE>::N, 1)
       // FP8: the accumulator holds (J0_ij / s_i)(psi_j / sigma); one product
       // with s_i sigma restores Y (sigma a power of two: exact).
       const float rs = F8 ? __fmul_rn(a.row_scale[i], kFp8PsiScale) : 1.0f;
+      const float h = epi_drive(a, i);
       if (lt == 0) {  // later tiles had theirs pulled in during the previous tile
 #pragma unroll
         for (int p = 0; p < PF && p < NCH; ++p) epi_prefetch_l2<MODE, CPLX, CW>(a, i, cbeg + p * CW, lane);
@@ -288,7 +289,7 @@ __global__ void __launch_bounds__(TcThreads<MODE>::N, 1)
         }
         const int lr0 = (part * PW + ch * CW) / W;
         float red[CW / W];
-        epi_chunk<MODE, CPLX, CW>(a, i, cbeg + ch * CW, v, cur, &s_beta[lr0], &s_dsc[lr0], red, bad);
+        epi_chunk<MODE, CPLX, CW>(a, i, cbeg + ch * CW, v, cur, h, &s_beta[lr0], &s_dsc[lr0], red, bad);
         if (need_red) {
 #pragma unroll
           for (int u = 0; u < CW / W; ++u) {

@@ -269,6 +269,7 @@ __global__ void __launch_bounds__(TcThreads<M_EULER>::N, 1)
         const int cbeg = n0 + part * PW;
         const unsigned* fl = g.flags + size_t(c) * MT;
         const float rs = F8 ? __fmul_rn(a.row_scale[i], kFp8PsiScale) : 1.0f;
+        const float h = epi_drive(a, i);
 #pragma unroll
         for (int p = 0; p < PF && p < NCH; ++p) epi_prefetch_l2<MODE, CPLX, CW>(a, i, cbeg + p * CW, lane);
         epi_load<MODE, CPLX, CW>(a, i, cbeg, R[0]);  // own rows of psi and gamma: written by this thread
@@ -306,7 +307,7 @@ __global__ void __launch_bounds__(TcThreads<M_EULER>::N, 1)
           }
           const int lr0 = (part * PW + ch * CW) / W;
           float red[CW / W];
-          epi_chunk<MODE, CPLX, CW>(a, i, cbeg + ch * CW, v, cur, &s_beta[lr0], &s_dsc[lr0], red, bad);
+          epi_chunk<MODE, CPLX, CW>(a, i, cbeg + ch * CW, v, cur, h, &s_beta[lr0], &s_dsc[lr0], red, bad);
           if (need_red) {
 #pragma unroll
             for (int u = 0; u < CW / W; ++u) {

@@ -114,7 +114,11 @@ __device__ __forceinline__ void epi_prefetch_l2(const StepArgs& a, int i, int c0
   }
 }
 
-// Arithmetic and stores of one chunk.  y: the CW accumulator values of row i.
+// The drive h_1i of row i (0 beyond N).
+__device__ __forceinline__ float epi_drive(const StepArgs& a, int i) { return i < a.N ? a.h1[i] : 0.0f; }
+
+// Arithmetic and stores of one chunk.  y: the CW accumulator values of row i;
+// h: the row's drive (epi_drive).
 // beta_s / dsc: per-restart stage scale and noise amplitude, indexed by the
 // chunk's local restart.  red[u]: per-restart contribution (density of the
 // new amplitude, or Eq. (1) partial energy).  nxt (NXT only): receives the
@@ -122,14 +126,21 @@ __device__ __forceinline__ void epi_prefetch_l2(const StepArgs& a, int i, int c0
 // input), 0 for restarts beyond R.
 template <int MODE, bool CPLX, int CW, bool NXT = false>
 __device__ __forceinline__ void epi_chunk(const StepArgs& a, int i, int c0, const float* y,
-                                          const EpiRegs<MODE, CPLX, CW>& R, const float* beta_s, const float* dsc,
-                                          float* red, int& bad, float* nxt = nullptr) {
+                                          const EpiRegs<MODE, CPLX, CW>& R, float h, const float* beta_s,
+                                          const float* dsc, float* red, int& bad, float* nxt = nullptr) {
   constexpr int W = CPLX ? 2 : 1;
   constexpr int NR = CW / W;
+  // the arguments as values: where they live in shared memory, every store
+  // below could otherwise change them
   const size_t Np = a.Np;
   const int r0 = CPLX ? c0 / 2 : c0;
+  const int nR = a.R, drive = CPLX ? a.q : 0, pitch = a.op_pitch;
+  const float dt = a.dt, eps = a.eps, rho_th = a.rho_th, hq = a.hq, op8_inv = a.op8_inv;
+  float *const psi_out = a.psi_out, *const gam = a.gam, *const acc = a.acc, *const gacc = a.gacc;
+  float *const xs_next = a.xs_next, *const gstg = a.gstg;
+  __nv_bfloat16* const op_out = a.op_out;
+  unsigned char* const op8_out = a.op8_out;
   const bool row_ok = i < a.N;
-  const float h = row_ok ? a.h1[i] : 0.0f;
   const float gi = (MODE == M_ENERGY && row_ok) ? a.g[i] : 0.0f;
   float z[CW];
   if (MODE == M_EULER || MODE == M_RK4) {
@@ -153,23 +164,23 @@ __device__ __forceinline__ void epi_chunk(const StepArgs& a, int i, int c0, cons
       if (CPLX) nxt[u * W + 1] = 0.0f;
     }
     const int r = r0 + u;
-    if (!row_ok || r >= a.R) continue;
+    if (!row_ok || r >= nR) continue;
     const int k0 = u * W;
     const size_t o0 = size_t(c0 + k0) * Np + i;
     const size_t o1 = o0 + Np;
     const size_t og = size_t(r) * Np + i;
     const float yr = y[k0], yi = CPLX ? y[k0 + 1] : 0.0f;
     if (MODE == M_RAW) {
-      a.psi_out[o0] = yr;
-      if (CPLX) a.psi_out[o1] = yi;
+      psi_out[o0] = yr;
+      if (CPLX) psi_out[o1] = yi;
       continue;
     }
     if (MODE == M_ENERGY) {
       const float pr = R.x[k0], pi = CPLX ? R.x[k0 + 1] : 0.0f;
       float sr, si = 0.0f;
-      if (CPLX && a.q >= 2) {  // Potts: the nearest q-th root, as the operand's projection
+      if (CPLX && drive >= 2) {  // Potts: the nearest q-th root, as the operand's projection
         double dr, di;
-        potts_project(pr, pi, a.q, dr, di);
+        potts_project(pr, pi, drive, dr, di);
         sr = float(dr);
         si = float(di);
       } else if (CPLX) {
@@ -185,49 +196,49 @@ __device__ __forceinline__ void epi_chunk(const StepArgs& a, int i, int c0, cons
     const float xr = R.x[k0], xi = CPLX ? R.x[k0 + 1] : 0.0f;
     const float gs = R.gs[u];
     float kr, ki, kg;
-    gd_rhs(xr, xi, gs, yr, yi, beta_s[u], h, a.eps, a.rho_th, kr, ki, kg);
-    if (CPLX && a.q) resonant_drive(xr, xi, a.q, a.hq, kr, ki);
+    gd_rhs(xr, xi, gs, yr, yi, beta_s[u], h, eps, rho_th, kr, ki, kg);
+    if (CPLX && drive) resonant_drive(xr, xi, drive, hq, kr, ki);
     float nr, ni, ng;
     if (MODE == M_EULER) {
-      nr = axpy(a.dt, kr, xr);
-      ni = axpy(a.dt, ki, xi);
-      ng = axpy(a.dt, kg, gs);
+      nr = axpy(dt, kr, xr);
+      ni = axpy(dt, ki, xi);
+      ng = axpy(dt, kg, gs);
     } else {
       const float pr = (MODE == M_RK1) ? xr : R.pn[ModeTraits<MODE>::rk_mid ? k0 : 0];
       const float pi = (MODE == M_RK1) ? xi : (CPLX ? R.pn[ModeTraits<MODE>::rk_mid ? k0 + 1 : 0] : 0.0f);
       const float gn = (MODE == M_RK1) ? gs : R.gn[ModeTraits<MODE>::rk_mid ? u : 0];
       if (MODE == M_RK4) {
-        const float d6 = __fdiv_rn(a.dt, 6.0f);
+        const float d6 = __fdiv_rn(dt, 6.0f);
         nr = axpy(d6, __fadd_rn(R.ac[k0], kr), pr);
         ni = CPLX ? axpy(d6, __fadd_rn(R.ac[CPLX ? k0 + 1 : 0], ki), pi) : 0.0f;
         ng = axpy(d6, __fadd_rn(R.ga[u], kg), gn);
       } else {
-        const float cf = (MODE == M_RK3) ? a.dt : __fmul_rn(0.5f, a.dt);
+        const float cf = (MODE == M_RK3) ? dt : __fmul_rn(0.5f, dt);
         if (MODE == M_RK1) {
-          st_state(a.acc + o0, kr);
-          if (CPLX) st_state(a.acc + o1, ki);
-          st_state(a.gacc + og, kg);
+          st_state(acc + o0, kr);
+          if (CPLX) st_state(acc + o1, ki);
+          st_state(gacc + og, kg);
         } else {
-          st_state(a.acc + o0, axpy(2.0f, kr, R.ac[ModeTraits<MODE>::rk_mid ? k0 : 0]));
-          if (CPLX) st_state(a.acc + o1, axpy(2.0f, ki, R.ac[ModeTraits<MODE>::rk_mid ? k0 + 1 : 0]));
-          st_state(a.gacc + og, axpy(2.0f, kg, R.ga[ModeTraits<MODE>::rk_mid ? u : 0]));
+          st_state(acc + o0, axpy(2.0f, kr, R.ac[ModeTraits<MODE>::rk_mid ? k0 : 0]));
+          if (CPLX) st_state(acc + o1, axpy(2.0f, ki, R.ac[ModeTraits<MODE>::rk_mid ? k0 + 1 : 0]));
+          st_state(gacc + og, axpy(2.0f, kg, R.ga[ModeTraits<MODE>::rk_mid ? u : 0]));
         }
         const float sr = axpy(cf, kr, pr), si = axpy(cf, ki, pi);
         if (NXT) {
           nxt[k0] = sr;
           if (CPLX) nxt[k0 + 1] = si;
         }
-        st_state(a.xs_next + o0, sr);
-        if (CPLX) st_state(a.xs_next + o1, si);
-        st_state(a.gstg + og, axpy(cf, kg, gn));
-        if (a.op_out) {
-          const size_t p0 = size_t(c0 + k0) * a.op_pitch + i;
-          a.op_out[p0] = __float2bfloat16_rn(sr);
-          if (CPLX) a.op_out[p0 + a.op_pitch] = __float2bfloat16_rn(si);
+        st_state(xs_next + o0, sr);
+        if (CPLX) st_state(xs_next + o1, si);
+        st_state(gstg + og, axpy(cf, kg, gn));
+        if (op_out) {
+          const size_t p0 = size_t(c0 + k0) * pitch + i;
+          op_out[p0] = __float2bfloat16_rn(sr);
+          if (CPLX) op_out[p0 + pitch] = __float2bfloat16_rn(si);
         }
-        if (a.op8_out) {
-          a.op8_out[o0] = __nv_cvt_float_to_fp8(sr * a.op8_inv, __NV_SATFINITE, __NV_E4M3);
-          if (CPLX) a.op8_out[o1] = __nv_cvt_float_to_fp8(si * a.op8_inv, __NV_SATFINITE, __NV_E4M3);
+        if (op8_out) {
+          op8_out[o0] = __nv_cvt_float_to_fp8(sr * op8_inv, __NV_SATFINITE, __NV_E4M3);
+          if (CPLX) op8_out[o1] = __nv_cvt_float_to_fp8(si * op8_inv, __NV_SATFINITE, __NV_E4M3);
         }
         continue;
       }
@@ -240,17 +251,17 @@ __device__ __forceinline__ void epi_chunk(const StepArgs& a, int i, int c0, cons
       nxt[k0] = nr;
       if (CPLX) nxt[k0 + 1] = ni;
     }
-    st_state(a.psi_out + o0, nr);
-    if (CPLX) st_state(a.psi_out + o1, ni);
-    st_state(a.gam + og, ng);
-    if (a.op_out) {
-      const size_t p0 = size_t(c0 + k0) * a.op_pitch + i;
-      a.op_out[p0] = __float2bfloat16_rn(nr);
-      if (CPLX) a.op_out[p0 + a.op_pitch] = __float2bfloat16_rn(ni);
+    st_state(psi_out + o0, nr);
+    if (CPLX) st_state(psi_out + o1, ni);
+    st_state(gam + og, ng);
+    if (op_out) {
+      const size_t p0 = size_t(c0 + k0) * pitch + i;
+      op_out[p0] = __float2bfloat16_rn(nr);
+      if (CPLX) op_out[p0 + pitch] = __float2bfloat16_rn(ni);
     }
-    if (a.op8_out) {
-      a.op8_out[o0] = __nv_cvt_float_to_fp8(nr * a.op8_inv, __NV_SATFINITE, __NV_E4M3);
-      if (CPLX) a.op8_out[o1] = __nv_cvt_float_to_fp8(ni * a.op8_inv, __NV_SATFINITE, __NV_E4M3);
+    if (op8_out) {
+      op8_out[o0] = __nv_cvt_float_to_fp8(nr * op8_inv, __NV_SATFINITE, __NV_E4M3);
+      if (CPLX) op8_out[o1] = __nv_cvt_float_to_fp8(ni * op8_inv, __NV_SATFINITE, __NV_E4M3);
     }
     const float rn = density(nr, ni);
     red[u] = rn;
