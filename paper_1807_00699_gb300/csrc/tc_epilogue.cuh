@@ -44,38 +44,41 @@ struct EpiRegs {
   float ga[T::rk_mid ? NR : 1];
 };
 
-// Loads the inputs of columns c0 .. c0+CW-1 at row i.  Column and restart
-// indices are clamped to the padded buffers (columns < Cp, restarts < Rp), so
-// every address is valid whatever the tile width; values of columns beyond C
-// are discarded by epi_chunk.
+// Loads the inputs of columns c0 .. c0+CW-1 at row i.  A chunk lies inside the
+// padded buffers (Cp and Rp are multiples of 256) or wholly beyond them, where
+// its first column and restart are clamped so that every address is valid
+// whatever the tile width; values of columns beyond C are discarded by
+// epi_chunk.
 template <int MODE, bool CPLX, int CW>
 __device__ __forceinline__ void epi_load(const StepArgs& a, int i, int c0, EpiRegs<MODE, CPLX, CW>& R) {
   using Tr = ModeTraits<MODE>;
   constexpr int W = CPLX ? 2 : 1;
   const size_t Np = a.Np;
-  const int r0 = CPLX ? c0 / 2 : c0;
+  const size_t o = size_t(min(c0, a.Cp - CW)) * Np + i;
+  const size_t og = size_t(min(CPLX ? c0 / 2 : c0, a.Rp - CW / W)) * Np + i;
+  const float* const x = (MODE == M_ENERGY ? a.psi_n : a.xs) + o;
 #pragma unroll
-  for (int k = 0; k < CW; ++k) {
-    const size_t o = size_t(min(c0 + k, a.Cp - 1)) * Np + i;
-    if (MODE == M_ENERGY) {
-      R.x[k] = ld_state(a.psi_n + o);
-    } else if (Tr::has_x) {
-      R.x[k] = ld_state(a.xs + o);
-      if (Tr::rk_mid) {
-        R.pn[k] = ld_state(a.psi_n + o);
-        R.ac[k] = ld_state(a.acc + o);
-      }
+  for (int k = 0; k < CW; ++k)
+    if (Tr::has_x) R.x[k] = ld_state(x + k * Np);
+  if (Tr::rk_mid) {
+    const float *const pn = a.psi_n + o, *const ac = a.acc + o;
+#pragma unroll
+    for (int k = 0; k < CW; ++k) {
+      R.pn[k] = ld_state(pn + k * Np);
+      R.ac[k] = ld_state(ac + k * Np);
     }
   }
   if (Tr::has_g) {
+    const float* const gs = ((MODE == M_EULER || MODE == M_RK1) ? a.gam : a.gstg) + og;
+#pragma unroll
+    for (int u = 0; u < CW / W; ++u) R.gs[u] = ld_state(gs + u * Np);
+  }
+  if (Tr::rk_mid) {
+    const float *const gn = a.gam + og, *const ga = a.gacc + og;
 #pragma unroll
     for (int u = 0; u < CW / W; ++u) {
-      const size_t og = size_t(min(r0 + u, a.Rp - 1)) * Np + i;
-      R.gs[u] = ld_state(((MODE == M_EULER || MODE == M_RK1) ? a.gam : a.gstg) + og);
-      if (Tr::rk_mid) {
-        R.gn[u] = ld_state(a.gam + og);
-        R.ga[u] = ld_state(a.gacc + og);
-      }
+      R.gn[u] = ld_state(gn + u * Np);
+      R.ga[u] = ld_state(ga + u * Np);
     }
   }
 }
@@ -134,48 +137,28 @@ __device__ __forceinline__ void epi_chunk(const StepArgs& a, int i, int c0, cons
   // below could otherwise change them
   const size_t Np = a.Np;
   const int r0 = CPLX ? c0 / 2 : c0;
-  const int nR = a.R, drive = CPLX ? a.q : 0, pitch = a.op_pitch;
+  const int drive = CPLX ? a.q : 0;
   const float dt = a.dt, eps = a.eps, rho_th = a.rho_th, hq = a.hq, op8_inv = a.op8_inv;
-  float *const psi_out = a.psi_out, *const gam = a.gam, *const acc = a.acc, *const gacc = a.gacc;
-  float *const xs_next = a.xs_next, *const gstg = a.gstg;
-  __nv_bfloat16* const op_out = a.op_out;
-  unsigned char* const op8_out = a.op8_out;
   const bool row_ok = i < a.N;
-  const float gi = (MODE == M_ENERGY && row_ok) ? a.g[i] : 0.0f;
-  float z[CW];
-  if (MODE == M_EULER || MODE == M_RK4) {
-    bool any = false;
+  const int live = row_ok ? a.R - r0 : 0;  // restarts u < live exist; the others' values go nowhere
+  const size_t o0 = size_t(c0) * Np + i, og = size_t(r0) * Np + i, p0 = size_t(c0) * a.op_pitch + i;
+  if (MODE == M_RAW) {
+    float* const out = a.psi_out + o0;
 #pragma unroll
-    for (int u = 0; u < NR; ++u) any |= dsc[u] != 0.0f;
+    for (int u = 0; u < NR; ++u) {
+      red[u] = 0.0f;
+      if (u < live)
 #pragma unroll
-    for (int q = 0; q < CW / 4; ++q) {
-      if (any) {
-        philox_normal4(uint32_t(i), uint32_t((c0 >> 2) + q), a.step, 0u, a.seed, &z[4 * q]);
-      } else {
-        z[4 * q] = z[4 * q + 1] = z[4 * q + 2] = z[4 * q + 3] = 0.0f;
-      }
+        for (int w = 0; w < W; ++w) out[(u * W + w) * Np] = y[u * W + w];
     }
+    return;
   }
+  if (MODE == M_ENERGY) {
+    const float gi = row_ok ? a.g[i] : 0.0f;
 #pragma unroll
-  for (int u = 0; u < NR; ++u) {
-    red[u] = 0.0f;
-    if (NXT) {
-      nxt[u * W] = 0.0f;
-      if (CPLX) nxt[u * W + 1] = 0.0f;
-    }
-    const int r = r0 + u;
-    if (!row_ok || r >= nR) continue;
-    const int k0 = u * W;
-    const size_t o0 = size_t(c0 + k0) * Np + i;
-    const size_t o1 = o0 + Np;
-    const size_t og = size_t(r) * Np + i;
-    const float yr = y[k0], yi = CPLX ? y[k0 + 1] : 0.0f;
-    if (MODE == M_RAW) {
-      psi_out[o0] = yr;
-      if (CPLX) psi_out[o1] = yi;
-      continue;
-    }
-    if (MODE == M_ENERGY) {
+    for (int u = 0; u < NR; ++u) {
+      const int k0 = u * W;
+      const float yr = y[k0], yi = CPLX ? y[k0 + 1] : 0.0f;
       const float pr = R.x[k0], pi = CPLX ? R.x[k0 + 1] : 0.0f;
       float sr, si = 0.0f;
       if (CPLX && drive >= 2) {  // Potts: the nearest q-th root, as the operand's projection
@@ -190,83 +173,119 @@ __device__ __forceinline__ void epi_chunk(const StepArgs& a, int i, int c0, cons
       } else {
         sr = pr >= 0.0f ? 1.0f : -1.0f;
       }
-      red[u] = -(sr * yr + si * yi) + gi * sr;
-      continue;
+      red[u] = u < live ? -(sr * yr + si * yi) + gi * sr : 0.0f;
     }
+    return;
+  }
+  constexpr bool COMPLETES = MODE == M_EULER || MODE == M_RK4;
+  // RK stages hold more values per element: they take one restart at a time
+  // and read its scales where they are used; Euler runs a chunk as straight code
+  constexpr bool MID = ModeTraits<MODE>::rk_mid, ONE = MODE != M_EULER;
+  float bs[ONE ? 1 : NR], ds[ONE ? 1 : NR], z[CW];
+  if (!ONE)
+#pragma unroll
+    for (int u = 0; u < NR; ++u) bs[ONE ? 0 : u] = beta_s[u];
+  const bool noisy = a.noise_D != 0.0f;
+  if (COMPLETES) {
+    bool any = false;
+    if (!ONE)
+#pragma unroll
+      for (int u = 0; u < NR; ++u) ds[ONE ? 0 : u] = 0.0f;
+    if (noisy) {
+#pragma unroll
+      for (int u = 0; u < NR; ++u) {
+        if (!ONE) ds[ONE ? 0 : u] = dsc[u];
+        any |= dsc[u] != 0.0f;
+      }
+    }
+#pragma unroll
+    for (int q = 0; q < CW / 4; ++q) {
+      if (any) {
+        philox_normal4(uint32_t(i), uint32_t((c0 >> 2) + q), a.step, 0u, a.seed, &z[4 * q]);
+      } else {
+        z[4 * q] = z[4 * q + 1] = z[4 * q + 2] = z[4 * q + 3] = 0.0f;
+      }
+    }
+  }
+  float* const xo = (COMPLETES ? a.psi_out : a.xs_next) + o0;
+  float* const go = (COMPLETES ? a.gam : a.gstg) + og;
+  float *const ao = COMPLETES ? nullptr : a.acc + o0, *const gao = COMPLETES ? nullptr : a.gacc + og;
+  __nv_bfloat16* const op = a.op_out;
+  unsigned char* const op8 = a.op8_out;
+  const size_t pitch = a.op_pitch;
+  unsigned top = 0;  // largest density as bits: finite and below 1e30 where it is small
+#pragma unroll
+  for (int u = 0; u < NR; ++u) {
+    const int k0 = u * W;
+    if (ONE) {
+      if (u >= live) {
+        red[u] = 0.0f;
+        if (NXT) nxt[k0] = nxt[k0 + W - 1] = 0.0f;
+        continue;
+      }
+      bs[0] = beta_s[u];
+      ds[0] = noisy ? dsc[u] : 0.0f;
+    }
+    const float yr = y[k0], yi = CPLX ? y[k0 + 1] : 0.0f;
     const float xr = R.x[k0], xi = CPLX ? R.x[k0 + 1] : 0.0f;
     const float gs = R.gs[u];
     float kr, ki, kg;
-    gd_rhs(xr, xi, gs, yr, yi, beta_s[u], h, eps, rho_th, kr, ki, kg);
+    gd_rhs(xr, xi, gs, yr, yi, bs[ONE ? 0 : u], h, eps, rho_th, kr, ki, kg);
     if (CPLX && drive) resonant_drive(xr, xi, drive, hq, kr, ki);
-    float nr, ni, ng;
+    float nr, ni, ng;  // the next operand values and gain
     if (MODE == M_EULER) {
       nr = axpy(dt, kr, xr);
       ni = axpy(dt, ki, xi);
       ng = axpy(dt, kg, gs);
     } else {
-      const float pr = (MODE == M_RK1) ? xr : R.pn[ModeTraits<MODE>::rk_mid ? k0 : 0];
-      const float pi = (MODE == M_RK1) ? xi : (CPLX ? R.pn[ModeTraits<MODE>::rk_mid ? k0 + 1 : 0] : 0.0f);
-      const float gn = (MODE == M_RK1) ? gs : R.gn[ModeTraits<MODE>::rk_mid ? u : 0];
+      const float pr = MID ? R.pn[MID ? k0 : 0] : xr;
+      const float pi = CPLX ? (MID ? R.pn[MID ? k0 + W - 1 : 0] : xi) : 0.0f;
+      const float gn = MID ? R.gn[MID ? u : 0] : gs;
       if (MODE == M_RK4) {
         const float d6 = __fdiv_rn(dt, 6.0f);
-        nr = axpy(d6, __fadd_rn(R.ac[k0], kr), pr);
-        ni = CPLX ? axpy(d6, __fadd_rn(R.ac[CPLX ? k0 + 1 : 0], ki), pi) : 0.0f;
-        ng = axpy(d6, __fadd_rn(R.ga[u], kg), gn);
+        nr = axpy(d6, __fadd_rn(R.ac[MID ? k0 : 0], kr), pr);
+        ni = CPLX ? axpy(d6, __fadd_rn(R.ac[MID ? k0 + W - 1 : 0], ki), pi) : 0.0f;
+        ng = axpy(d6, __fadd_rn(R.ga[MID ? u : 0], kg), gn);
       } else {
         const float cf = (MODE == M_RK3) ? dt : __fmul_rn(0.5f, dt);
-        if (MODE == M_RK1) {
-          st_state(acc + o0, kr);
-          if (CPLX) st_state(acc + o1, ki);
-          st_state(gacc + og, kg);
-        } else {
-          st_state(acc + o0, axpy(2.0f, kr, R.ac[ModeTraits<MODE>::rk_mid ? k0 : 0]));
-          if (CPLX) st_state(acc + o1, axpy(2.0f, ki, R.ac[ModeTraits<MODE>::rk_mid ? k0 + 1 : 0]));
-          st_state(gacc + og, axpy(2.0f, kg, R.ga[ModeTraits<MODE>::rk_mid ? u : 0]));
+        if (u < live) {
+          st_state(ao + k0 * Np, MID ? axpy(2.0f, kr, R.ac[MID ? k0 : 0]) : kr);
+          if (CPLX) st_state(ao + (k0 + 1) * Np, MID ? axpy(2.0f, ki, R.ac[MID ? k0 + W - 1 : 0]) : ki);
+          st_state(gao + u * Np, MID ? axpy(2.0f, kg, R.ga[MID ? u : 0]) : kg);
         }
-        const float sr = axpy(cf, kr, pr), si = axpy(cf, ki, pi);
-        if (NXT) {
-          nxt[k0] = sr;
-          if (CPLX) nxt[k0 + 1] = si;
-        }
-        st_state(xs_next + o0, sr);
-        if (CPLX) st_state(xs_next + o1, si);
-        st_state(gstg + og, axpy(cf, kg, gn));
-        if (op_out) {
-          const size_t p0 = size_t(c0 + k0) * pitch + i;
-          op_out[p0] = __float2bfloat16_rn(sr);
-          if (CPLX) op_out[p0 + pitch] = __float2bfloat16_rn(si);
-        }
-        if (op8_out) {
-          op8_out[o0] = __nv_cvt_float_to_fp8(sr * op8_inv, __NV_SATFINITE, __NV_E4M3);
-          if (CPLX) op8_out[o1] = __nv_cvt_float_to_fp8(si * op8_inv, __NV_SATFINITE, __NV_E4M3);
-        }
-        continue;
+        nr = axpy(cf, kr, pr);
+        ni = axpy(cf, ki, pi);
+        ng = axpy(cf, kg, gn);
       }
     }
-    if (MODE == M_EULER || MODE == M_RK4) {
-      nr = axpy(dsc[u], z[k0], nr);
-      if (CPLX) ni = axpy(dsc[u], z[k0 + 1], ni);
+    if (COMPLETES) {
+      nr = axpy(ds[ONE ? 0 : u], z[k0], nr);
+      if (CPLX) ni = axpy(ds[ONE ? 0 : u], z[CPLX ? k0 + 1 : 0], ni);
+      const float rn = CPLX ? density(nr, ni) : __fmul_rn(nr, nr);  // density(nr, 0)
+      red[u] = u < live ? rn : 0.0f;
+      top = max(top, u < live ? __float_as_uint(rn) & 0x7fffffffu : 0u);
+    } else {
+      red[u] = 0.0f;
     }
     if (NXT) {
-      nxt[k0] = nr;
-      if (CPLX) nxt[k0 + 1] = ni;
+      nxt[k0] = u < live ? nr : 0.0f;
+      if (CPLX) nxt[k0 + W - 1] = u < live ? ni : 0.0f;
     }
-    st_state(psi_out + o0, nr);
-    if (CPLX) st_state(psi_out + o1, ni);
-    st_state(gam + og, ng);
-    if (op_out) {
-      const size_t p0 = size_t(c0 + k0) * pitch + i;
-      op_out[p0] = __float2bfloat16_rn(nr);
-      if (CPLX) op_out[p0 + pitch] = __float2bfloat16_rn(ni);
+    if (u < live) {
+      st_state(xo + k0 * Np, nr);
+      if (CPLX) st_state(xo + (k0 + 1) * Np, ni);
+      st_state(go + u * Np, ng);
+      if (op) {
+        op[p0 + k0 * pitch] = __float2bfloat16_rn(nr);
+        if (CPLX) op[p0 + (k0 + 1) * pitch] = __float2bfloat16_rn(ni);
+      }
+      if (op8) {
+        op8[o0 + k0 * Np] = __nv_cvt_float_to_fp8(nr * op8_inv, __NV_SATFINITE, __NV_E4M3);
+        if (CPLX) op8[o0 + (k0 + 1) * Np] = __nv_cvt_float_to_fp8(ni * op8_inv, __NV_SATFINITE, __NV_E4M3);
+      }
     }
-    if (op8_out) {
-      op8_out[o0] = __nv_cvt_float_to_fp8(nr * op8_inv, __NV_SATFINITE, __NV_E4M3);
-      if (CPLX) op8_out[o1] = __nv_cvt_float_to_fp8(ni * op8_inv, __NV_SATFINITE, __NV_E4M3);
-    }
-    const float rn = density(nr, ni);
-    red[u] = rn;
-    bad |= !(rn < 1e30f);
   }
+  bad |= top >= __float_as_uint(1e30f);
 }
 
 }  // namespace gda
