@@ -256,10 +256,10 @@ __global__ void __launch_bounds__(ETHREADS, 1) k_energy_product(const __grid_con
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  const uint32_t tmem = s_tmem;
+  const uint32_t tmem = warp_uniform(s_tmem);
 
   if (warp == 0) {
-    if (lane == 0) {
+    if (elect_one()) {
       int it = 0;
       bool stop = false;
       for (int t = blockIdx.x; t < n_tile && !stop; t += gridDim.x) {
@@ -288,8 +288,9 @@ __global__ void __launch_bounds__(ETHREADS, 1) k_energy_product(const __grid_con
       }
     }
   } else if (warp == 1) {
-    if (lane == 0) {
+    if (elect_one()) {
       constexpr uint32_t idesc = idesc_bf16<TILE>();
+      const uint64_t d0 = sdesc_sw128(base);
       int it = 0, use = 0;
       bool stop = false;
       for (int t = blockIdx.x; t < n_tile && !stop; t += gridDim.x) {
@@ -312,10 +313,9 @@ __global__ void __launch_bounds__(ETHREADS, 1) k_energy_product(const __grid_con
                 break;
               }
               tc_fence_after();
-              const uint32_t sa = base + s * 2 * TBYTES;
 #pragma unroll
               for (int k = 0; k < 4; ++k)
-                mma_bf16(tmem + b * TILE, sdesc_sw128(sa + k * 32), sdesc_sw128(sa + TBYTES + k * 32), idesc,
+                mma_bf16(tmem + b * TILE, sdesc_at(d0, s * 2 * TBYTES + k * 32), sdesc_at(d0, s * 2 * TBYTES + TBYTES + k * 32), idesc,
                          (kb > k0) || k);
               mma_commit(empty_bar(s));
             }

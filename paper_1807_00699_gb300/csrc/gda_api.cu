@@ -877,10 +877,10 @@ gda_status gda_run(gda_ctx* c, const gda_params* p, int32_t R, int64_t steps) {
       ra.rho[0] = c->rho[c->rcur];
       ra.rho[1] = c->rho[c->rcur ^ 1];
       ra.ops = c->ops;
-      ra.withhold_tile = p->withhold_flag > 0 ? int((c->C + 127) / 128) * int((c->N + 127) / 128) - 1 : -1;
       ra.withhold_step = p->withhold_flag > 0 ? p->withhold_flag : -1;
       CK(cudaMemsetAsync(c->flags, 0, kMaxResidentTiles * sizeof(unsigned), c->stream));
-      LK(launch_step_res(c->plan, ra, a, c->stream, res_pair));
+      LK(res_pair ? launch_step_res_pair(c->plan, ra, a, c->stream)
+                  : launch_step_res(c->plan, ra, a, c->sms, c->stream));
       c->cur ^= flip;
       c->bcur ^= flip;
       c->opcur ^= flip;

@@ -257,11 +257,11 @@ __global__ void __launch_bounds__(NTHREADS, 1)
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  const uint32_t tmem = *s_tmem;
+  const uint32_t tmem = warp_uniform(*s_tmem);
 
   if (warp == 0) {
     // ---------------- TMA producer ----------------
-    if (lane == 0) {
+    if (elect_one()) {
       int it = 0;
       bool stop = false;
       for (int n = 0; n < b.nsteps && !stop; ++n) {
@@ -304,8 +304,9 @@ __global__ void __launch_bounds__(NTHREADS, 1)
     }
   } else if (warp == 1) {
     // ---------------- MMA issuer ----------------
-    if (lane == 0) {
+    if (elect_one()) {
       constexpr uint32_t idesc = idesc_bf16<BN>();
+      const uint64_t dA = sdesc_sw128(sA), dB = sdesc_sw128(sB);
       int it = 0, lt = 0;
       int committed = -1;  // accumulator of the last commit (lt), -1 before any
       bool stop = false;
@@ -330,7 +331,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
             tc_fence_after();
 #pragma unroll
             for (int k = 0; k < BK / 16; ++k)
-              mma_bf16(dacc, sdesc_sw128(sA + s * Cfg::A_BYTES + k * 32), sdesc_sw128(sB + s * Cfg::B_BYTES + k * 32),
+              mma_bf16(dacc, sdesc_at(dA, s * Cfg::A_BYTES + k * 32), sdesc_at(dB, s * Cfg::B_BYTES + k * 32),
                        idesc, (kb | k) != 0);
             mma_commit(empty_bar(s));
           }

@@ -98,12 +98,12 @@ __global__ void __launch_bounds__(TcThreads<M_EULER>::N, 1)
   __syncthreads();
   if (PAIR) cluster_sync();  // barriers of both CTAs initialised before any remote arrival
   tc_fence_after();
-  const uint32_t tmem = *s_tmem;
+  const uint32_t tmem = warp_uniform(*s_tmem);
   if (threadIdx.x == 0) stamp(a0, 1);
 
   if (warp == 0) {
     // ---------------- TMA producer ----------------
-    if (lane == 0) {
+    if (elect_one()) {
       const uint64_t keep = policy_evict_last();  // J and the operand are re-read by every tile row / column
       int it = 0;
       bool stop = false;
@@ -158,9 +158,10 @@ __global__ void __launch_bounds__(TcThreads<M_EULER>::N, 1)
     }
   } else if (warp == 1) {
     // ---------------- MMA issuer ----------------
-    if (lane == 0 && leader) {
+    if (leader && elect_one()) {
       constexpr uint32_t idesc = PAIR ? (F8 ? idesc_e4m3_m256<BN>() : idesc_bf16_m256<BN>())
                                       : (F8 ? idesc_e4m3<BN>() : idesc_bf16<BN>());
+      const uint64_t dA = sdesc_sw128(sA), dB = sdesc_sw128(sB);
       int it = 0, lt = 0;
       bool stop = false;
       for (int n = 0; n < g.steps && !stop; ++n) {
@@ -186,8 +187,8 @@ __global__ void __launch_bounds__(TcThreads<M_EULER>::N, 1)
             if (lt == 0 && kb == 0) stamp(a0, 2);
 #pragma unroll
             for (int k = 0; k < 4; ++k) {  // 32 bytes of K per instruction
-              const uint64_t da = sdesc_sw128(sA + s * Cfg::A_BYTES + k * 32);
-              const uint64_t db = sdesc_sw128(sB + s * Cfg::B_BYTES + k * 32);
+              const uint64_t da = sdesc_at(dA, s * Cfg::A_BYTES + k * 32);
+              const uint64_t db = sdesc_at(dB, s * Cfg::B_BYTES + k * 32);
               if (PAIR) {
                 if (F8)
                   mma_e4m3_pair(dacc, da, db, idesc, (kb | k) != 0);

@@ -20,6 +20,25 @@ static __device__ __forceinline__ uint32_t smem_u32(const void* p) {
   return static_cast<uint32_t>(__cvta_generic_to_shared(p));
 }
 
+// True in one lane of a converged warp.  A role's loop inside `if (elect_one())`
+// is known to run in one thread, so its TMA and MMA operands live in uniform
+// registers; inside `if (lane == 0)` the compiler moves every operand there for
+// each instruction: four M128 N128 K16 MMAs and a commit then take 469 SM cycles
+// to issue, elected 256, which is what the tensor core needs for them (N = 64:
+// 469 against 192).
+static __device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile(
+      "{\n\t.reg .pred q;\n\t"
+      "elect.sync _|q, 0xffffffff;\n\t"
+      "selp.u32 %0, 1, 0, q;\n\t}"
+      : "=r"(p));
+  return p != 0;
+}
+
+// A value that is the same in every lane of a converged warp, for the compiler too.
+static __device__ __forceinline__ uint32_t warp_uniform(uint32_t v) { return __reduce_max_sync(0xffffffffu, v); }
+
 static __device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
 }
@@ -140,6 +159,9 @@ static __device__ __forceinline__ uint64_t sdesc_sw128(uint32_t saddr) {
   d |= static_cast<uint64_t>(2) << 61;
   return d;
 }
+
+// The descriptor of an operand `bytes` further on.
+static __device__ __forceinline__ uint64_t sdesc_at(uint64_t d, uint32_t bytes) { return d + (bytes >> 4); }
 
 // Instruction descriptor of kind::f16: FP32 accumulator, BF16 A and B, both
 // K-major, shape M = 128 x N.
