@@ -50,7 +50,7 @@ struct BatchInst {
   int rowX;            // first row of operand buffer 0 (buffer 1 follows at rowX + Cp)
   int flag0;           // flag of unit (row block 0, column block 0); unit (m, n) at flag0 + n * mt + m
   int has_base;        // init_mode 3: per-spin base amplitudes at off_base
-  long long off_psi;   // psi [2][Cp][Np]
+  long long off_psi;   // psi [Cp][Np], updated in place
   long long off_gam;   // gamma [Rp][Np]
   long long off_h1;    // h1 [Np]
   long long off_beta;  // beta [2][Rp]
@@ -115,10 +115,9 @@ __device__ __forceinline__ StepArgs unit_args(const BatchArgs& b, const BatchIns
   a.noise_decay = 0;
   a.seed = I.seed;
   a.step = step;
-  const size_t cn = size_t(I.Cp) * I.Np;
-  a.psi_n = b.psi + I.off_psi + size_t(cur) * cn;
+  a.psi_n = b.psi + I.off_psi;
   a.xs = a.psi_n;
-  a.psi_out = b.psi + I.off_psi + size_t(cur ^ 1) * cn;
+  a.psi_out = b.psi + I.off_psi;  // an amplitude is read and written by one thread only
   a.gam = b.gam + I.off_gam;
   a.h1 = b.h1 + I.off_h1;
   a.beta_in = b.beta + I.off_beta + size_t(cur) * I.Rp;
@@ -131,11 +130,15 @@ __device__ __forceinline__ StepArgs unit_args(const BatchArgs& b, const BatchIns
 
 // Epilogue of one unit at one step (all NEPI epilogue warps): waits for the
 // unit's accumulator, runs the Euler update of its 128 x BN tile, frees the
-// accumulator and publishes the unit's flag.  Returns false on an abort.
-template <int BN, bool CPLX>
+// accumulator and publishes the unit's flag.  a: the unit's arguments in shared
+// memory (read where used, not kept in every thread's registers); next builds
+// the following unit's in the other slot, published by the barrier that ends
+// this one.  Returns false on an abort.
+template <int BN, bool CPLX, typename Next>
 __device__ __forceinline__ bool epi_unit(const BatchArgs& b, const BatchInst& I, const BatchUnit& U, unsigned step,
                                          int cur, int n, uint32_t tacc, uint32_t full, uint32_t empty, uint32_t use,
-                                         float* s_beta, float* s_dsc, int* s_flag, StepArgs* s_args, int& bad) {
+                                         float* s_beta, float* s_dsc, int* s_flag, const StepArgs& a, Next next,
+                                         int& bad) {
   constexpr int W = CPLX ? 2 : 1;
   constexpr int RPT = BN / W;
   constexpr int PW = BN / (NEPI / 4);  // columns per part
@@ -146,12 +149,6 @@ __device__ __forceinline__ bool epi_unit(const BatchArgs& b, const BatchInst& I,
   const int e = threadIdx.x - 64;
   const int q = warp & 3;
   const int part = (warp - 2) >> 2;
-  // the unit's arguments live in shared memory (read where used), not in
-  // every epilogue thread's registers
-  bar_epi();  // every thread is done with the previous unit's arguments
-  if (e == 0) *s_args = unit_args(b, I, step, cur);
-  bar_epi();
-  const StepArgs& a = *s_args;
   const int m0 = U.mt * BM, n0 = U.nt * BN;
   const int rbase = n0 / W;
   const int i = m0 + 32 * q + lane;
@@ -199,15 +196,15 @@ __device__ __forceinline__ bool epi_unit(const BatchArgs& b, const BatchInst& I,
   const bool publish = b.nsteps > 1;  // later steps of this launch read what this unit wrote
   tc_fence_before();
   if (publish) fence_proxy_async_global();  // the next operand rows are read by other CTAs' TMA loads
-  bar_epi();
-  if (e == 0) mbar_arrive(empty);
   if (e < RPT && U.mt == 0) {
     const int r = rbase + e;
     if (r < a.R) a.beta_out[r] = next_beta(a, a.beta_in[r]);
   }
-  if (publish) {
-    bar_epi();
-    if (e == 0)  // a release store: ordered after every epilogue thread's writes (seen through the barrier)
+  if (e == 32 * NEPI - 1) next();  // a thread that publishes nothing
+  bar_epi();
+  if (e == 0) {
+    mbar_arrive(empty);
+    if (publish)  // a release store: ordered after every epilogue thread's writes (seen through the barrier)
       st_release_gpu(b.flags + I.flag0 + U.nt * I.mt + U.mt, step + 1u);
   }
   return true;
@@ -228,9 +225,9 @@ __global__ void __launch_bounds__(NTHREADS, 1)
   float* s_dsc = s_beta + BN;
   uint32_t* s_tmem = reinterpret_cast<uint32_t*>(s_dsc + 5 * BN);
   int* s_flag = reinterpret_cast<int*>(s_tmem + 1);
-  __shared__ StepArgs s_args;
+  __shared__ StepArgs s_args[2];
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = threadIdx.x >> 5;
   const unsigned step0 = *b.step_base + b.step_off;
   const long long lim = b.wait_cycles;
   const int u0 = b.cta_begin[blockIdx.x], u1 = b.cta_begin[blockIdx.x + 1];
@@ -350,6 +347,8 @@ __global__ void __launch_bounds__(NTHREADS, 1)
     const int e = threadIdx.x - 64;
     int bad = 0, lt = 0;
     bool run = true;
+    if (e == 0 && u0 < u1) s_args[0] = unit_args(b, b.inst[b.units[u0].inst], step0, int(step0 & 1u));
+    bar_epi();
     for (int n = 0; n < b.nsteps && run; ++n) {
       const unsigned step = step0 + unsigned(n);
       const int cur = int(step & 1u);
@@ -359,10 +358,16 @@ __global__ void __launch_bounds__(NTHREADS, 1)
         const int k2 = lt & 1;
         const uint32_t use = lt >> 1;
         const uint32_t tacc = tmem + k2 * BN;
+        auto next = [&]() {
+          const bool wrap = u + 1 == u1;
+          const unsigned sn = step + (wrap ? 1u : 0u);
+          if (!wrap || n + 1 < b.nsteps)
+            s_args[k2 ^ 1] = unit_args(b, b.inst[b.units[wrap ? u0 : u + 1].inst], sn, int(sn & 1u));
+        };
         run = I.cplx ? epi_unit<BN, true>(b, I, U, step, cur, n, tacc, acc_full(k2), acc_empty(k2), use, s_beta,
-                                          s_dsc, s_flag, &s_args, bad)
+                                          s_dsc, s_flag, s_args[k2], next, bad)
                      : epi_unit<BN, false>(b, I, U, step, cur, n, tacc, acc_full(k2), acc_empty(k2), use, s_beta,
-                                           s_dsc, s_flag, &s_args, bad);
+                                           s_dsc, s_flag, s_args[k2], next, bad);
       }
     }
     if (bad) s_flag[1] = 1;
@@ -530,7 +535,7 @@ struct gda_batch {
   std::vector<long long> oJ, oG, oP;
   std::vector<double> jmax;       // per instance: largest |J_ij| of an integer J, else -1
   std::vector<EnergyGroup> egroups;
-  EnergyProb* eprobs[2] = {nullptr, nullptr};  // panels for either state parity
+  EnergyProb* eprobs = nullptr;
   int4* eunits = nullptr;
   int* erexp = nullptr;
   unsigned char* edigits = nullptr;
@@ -711,12 +716,12 @@ gda_status upload_settings(gda_batch* b, const gda_params* p) {
 // panels are grouped while the digits and spins of a group fit together
 // (in `bound` bytes, unless one row block against one column block needs more).
 gda_status plan_energies(gda_batch* b, size_t bound) {
-  void* stale[] = {b->erexp, b->eunits, b->eprobs[0], b->eprobs[1]};  // of an attempt that failed
+  void* stale[] = {b->erexp, b->eunits, b->eprobs};  // of an attempt that failed
   for (void* p : stale)
     if (p) cudaFree(p);
   b->erexp = nullptr;
   b->eunits = nullptr;
-  b->eprobs[0] = b->eprobs[1] = nullptr;
+  b->eprobs = nullptr;
   auto align = [](size_t x) { return (x + 1023) / 1024 * 1024; };
   struct Place {
     int inst;
@@ -792,29 +797,27 @@ gda_status plan_energies(gda_batch* b, size_t bound) {
   BCK(cudaMemcpy(b->eunits + row.size() + col.size(), tile.data(), tile.size() * sizeof(int4),
                  cudaMemcpyHostToDevice));
   BCK(balloc(&ws, top));
-  for (int cur = 0; cur < 2; ++cur) {
-    for (size_t q = 0; q < probs.size(); ++q) {
-      const int k = place[q].inst;
-      const BatchInst& I = b->host[k];
-      EnergyProb& p = probs[q];
-      p.J = b->J64 + b->oJ[k];
-      p.g = b->g64 + b->oG[k];
-      p.psi = b->psi + I.off_psi + size_t(cur) * I.Cp * I.Np;
-      p.rexp = b->erexp + orexp[k];
-      p.Jd = ws + place[q].jd;
-      p.Sd = ws + place[q].sd;
-      // the panel's spins, addressed by the instance's column numbers
-      p.S64 = I.cplx ? reinterpret_cast<double*>(ws + place[q].s64) - (long long)p.nt0 * 128 * I.Np : nullptr;
-      p.part = b->part + b->oP[k];
-      p.ldp = I.R;
-    }
-    cudaError_t e = balloc(&b->eprobs[cur], probs.size());
-    if (e == cudaSuccess)
-      e = cudaMemcpy(b->eprobs[cur], probs.data(), probs.size() * sizeof(EnergyProb), cudaMemcpyHostToDevice);
-    if (e != cudaSuccess) {
-      cudaFree(ws);
-      BCK(e);
-    }
+  for (size_t q = 0; q < probs.size(); ++q) {
+    const int k = place[q].inst;
+    const BatchInst& I = b->host[k];
+    EnergyProb& p = probs[q];
+    p.J = b->J64 + b->oJ[k];
+    p.g = b->g64 + b->oG[k];
+    p.psi = b->psi + I.off_psi;
+    p.rexp = b->erexp + orexp[k];
+    p.Jd = ws + place[q].jd;
+    p.Sd = ws + place[q].sd;
+    // the panel's spins, addressed by the instance's column numbers
+    p.S64 = I.cplx ? reinterpret_cast<double*>(ws + place[q].s64) - (long long)p.nt0 * 128 * I.Np : nullptr;
+    p.part = b->part + b->oP[k];
+    p.ldp = I.R;
+  }
+  cudaError_t pe = balloc(&b->eprobs, probs.size());
+  if (pe == cudaSuccess)
+    pe = cudaMemcpy(b->eprobs, probs.data(), probs.size() * sizeof(EnergyProb), cudaMemcpyHostToDevice);
+  if (pe != cudaSuccess) {
+    cudaFree(ws);
+    BCK(pe);
   }
   for (EnergyGroup& g : groups) {
     g.col0 += int(row.size());
@@ -838,7 +841,7 @@ gda_status batch_energies(gda_batch* b) {
   }
   for (const EnergyGroup& g : b->egroups) {
     EnergyUnits u{};
-    u.probs = b->eprobs[b->step & 1ULL];
+    u.probs = b->eprobs;
     u.row = b->eunits + g.row0;
     u.col = b->eunits + g.col0;
     u.tile = b->eunits + g.tile0;
@@ -925,7 +928,7 @@ gda_status gda_batch_create(int32_t n, const int32_t* N, const int32_t* model, c
     b->rowsJ += I.Np;
     b->rowsX += 2 * I.Cp;
     I.off_psi = off_psi;
-    off_psi += 2LL * I.Cp * I.Np;
+    off_psi += (long long)I.Cp * I.Np;
     I.off_gam = off_gam;
     off_gam += (long long)I.Rp * I.Np;
     I.off_h1 = off_h1;
@@ -1202,7 +1205,7 @@ gda_status gda_batch_get_state(gda_batch* b, int32_t k, float* psi, float* gamma
   const int cur = int(b->step & 1ULL);
   const int W = I.cplx ? 2 : 1;
   std::vector<float> blk(size_t(I.Cp) * I.Np), gb(size_t(I.Rp) * I.Np);
-  BCK(cudaMemcpy(blk.data(), b->psi + I.off_psi + size_t(cur) * I.Cp * I.Np, blk.size() * sizeof(float),
+  BCK(cudaMemcpy(blk.data(), b->psi + I.off_psi, blk.size() * sizeof(float),
                  cudaMemcpyDeviceToHost));
   BCK(cudaMemcpy(gb.data(), b->gam + I.off_gam, gb.size() * sizeof(float), cudaMemcpyDeviceToHost));
   for (int r = 0; r < I.R; ++r)
@@ -1226,7 +1229,7 @@ void gda_batch_destroy(gda_batch* b) {
       if (P.units) cudaFree(P.units);
       if (P.cta_begin) cudaFree(P.cta_begin);
     }
-  void* ptrs[] = {b->eprobs[0], b->eprobs[1], b->erexp, b->edigits, b->inst, b->J16, b->ops, b->J64, b->g64, b->off_J, b->off_g, b->psi, b->gam, b->h1, b->beta,
+  void* ptrs[] = {b->eprobs, b->erexp, b->edigits, b->inst, b->J16, b->ops, b->J64, b->g64, b->off_J, b->off_g, b->psi, b->gam, b->h1, b->beta,
                   b->part, b->off_part, b->E_all, b->off_E, b->bestE, b->bestR, b->eunits, b->step_base, b->err,
                   b->flags, b->base};
   for (void* p : ptrs)
