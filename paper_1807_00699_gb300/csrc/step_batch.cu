@@ -596,7 +596,7 @@ gda_status build_plan(gda_batch* b, int bn, bool sorted, BatchPlan* P) {
     for (int mt = 0; mt < I.mt; ++mt)
       for (int t = 0; t < nt; ++t) {
         units.push_back(BatchUnit{k, mt, t, 0});
-        cost.push_back(double((I.N + BK - 1) / BK) * (128 + bn) + 64.0);  // K-blocks x smem cycles + epilogue
+        cost.push_back((I.N + BK - 1) / BK + 16.0);  // K-blocks of ~0.25 us and an epilogue of ~4 us
       }
   }
   P->bn = bn;
