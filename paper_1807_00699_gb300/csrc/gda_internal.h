@@ -175,6 +175,7 @@ cudaError_t launch_gdmod_step(const StepArgs& a, const float* J, float* K, const
 cudaError_t launch_to_e4m3(const float* x, unsigned char* y, size_t n, cudaStream_t s);
 int tc_mtiles(int N);
 int tc_pick_bn(int N, int C);
+int tc_pick_bn_stream(int N, int C);
 int tc_pick_bn_pair(int N, int C);
 bool tc_pair_pays(int N, int C);
 bool tc_supported(int device);

@@ -39,17 +39,17 @@ int tc_pick_bn_pair(int N, int C) {
 // tiles, and a 128 x BN tile costs about (128 + BN) shared-memory cycles per
 // K-slice of 16 (MMA reads plus TMA writes of A and B at ~128 B/clk), so pick
 // the width minimising rounds x (128 + BN).
-int tc_pick_bn(int N, int C) {
+static int pick_width(int N, int C, const int* widths, int n) {
   static int sms = 0;
   if (!sms) {
     int dev = 0;
     cudaGetDevice(&dev);
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1) sms = 148;
   }
-  const int widths[3] = {128, 224, 256};
-  int best = 128;
+  int best = widths[0];
   long long best_cost = -1;
-  for (int bn : widths) {
+  for (int k = 0; k < n; ++k) {
+    const int bn = widths[k];
     const long long tiles = (long long)((C + bn - 1) / bn) * ((N + BM - 1) / BM);
     const long long cost = ((tiles + sms - 1) / sms) * (128 + bn);
     if (best_cost < 0 || cost < best_cost) {
@@ -58,6 +58,20 @@ int tc_pick_bn(int N, int C) {
     }
   }
   return best;
+}
+
+int tc_pick_bn(int N, int C) {
+  static constexpr int widths[3] = {128, 224, 256};
+  return pick_width(N, C, widths, 3);
+}
+
+// The streaming kernel's one-SM tiles: a step ends with the CTA that has the
+// most columns, so widths between 128 and 224 are worth having where they keep
+// its number of tiles (SK N = 3001, R = 2100: 192 instead of 224 columns, two
+// tiles per CTA either way).
+int tc_pick_bn_stream(int N, int C) {
+  static constexpr int widths[5] = {128, 160, 192, 224, 256};
+  return pick_width(N, C, widths, 5);
 }
 
 // AUTO's choice: two-SM tiles when the row blocks pair up and the pair tiles

@@ -463,7 +463,7 @@ struct TcPlan {  // tensor maps of one operand set (BF16 or FP8)
   CUtensorMap B224;
   CUtensorMap B256;
   CUtensorMap B64;   // halves of 128- and 224-wide tiles for two-SM pairs
-  CUtensorMap B112;
+  CUtensorMap B112, B160, B192;
   int Cp;
 };
 
@@ -475,7 +475,8 @@ bool plan_maps(TcPlan* p, const void* Jop, int Np, const void* ops, int n_op_buf
   const int rows = n_op_bufs * Cp;
   return make_map(&p->A, Jop, Np, Np, BM, F8) && make_map(&p->B128, ops, Np, rows, 128, F8) &&
          make_map(&p->B224, ops, Np, rows, 224, F8) && make_map(&p->B256, ops, Np, rows, 256, F8) &&
-         make_map(&p->B64, ops, Np, rows, 64, F8) && make_map(&p->B112, ops, Np, rows, 112, F8);
+         make_map(&p->B64, ops, Np, rows, 64, F8) && make_map(&p->B112, ops, Np, rows, 112, F8) &&
+         make_map(&p->B160, ops, Np, rows, 160, F8) && make_map(&p->B192, ops, Np, rows, 192, F8);
 }
 
 template <bool F8>

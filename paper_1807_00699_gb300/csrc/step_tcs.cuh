@@ -429,7 +429,8 @@ cudaError_t seg_dispatch(const CUtensorMap& A, const CUtensorMap& B, const StepA
 
 }  // namespace
 
-// Tile width as for the per-step kernel; one launch of g.steps steps.
+// One launch of g.steps steps.  Two-SM tiles take the per-step kernel's widths,
+// one-SM tiles two more (tc_pick_bn_stream).
 template <bool F8>
 cudaError_t launch_seg_plan(const TcPlan* plan, const StepArgs& a, const SegArgs& g, bool pair, cudaStream_t s) {
   if (pair) {
@@ -438,7 +439,9 @@ cudaError_t launch_seg_plan(const TcPlan* plan, const StepArgs& a, const SegArgs
     if (bn == 224) return seg_dispatch<224, 6, F8, true>(plan->A, plan->B112, a, g, s);
     return seg_dispatch<128, 8, F8, true>(plan->A, plan->B64, a, g, s);
   }
-  const int bn = tc_pick_bn(a.N, a.C);
+  const int bn = tc_pick_bn_stream(a.N, a.C);
+  if (bn == 160) return seg_dispatch<160, 5, F8, false>(plan->A, plan->B160, a, g, s);
+  if (bn == 192) return seg_dispatch<192, 5, F8, false>(plan->A, plan->B192, a, g, s);
   if (bn == 256) return seg_dispatch<256, 4, F8, false>(plan->A, plan->B256, a, g, s);
   if (bn == 224) return seg_dispatch<224, 4, F8, false>(plan->A, plan->B224, a, g, s);
   return seg_dispatch<128, 6, F8, false>(plan->A, plan->B128, a, g, s);
