@@ -182,13 +182,51 @@ void free_state(gda_ctx* c) {
   c->have_state = false;
 }
 
+// Grows a digit workspace to at least `blocks` blocks of `per` bytes, halving
+// the request while memory is short; *blocks receives what fits.
+gda_status ensure_digits(gda_ctx* c, unsigned char** p, size_t* cap, size_t per, int* blocks) {
+  while (*cap < size_t(*blocks) * per) {
+    dfree(*p);
+    *cap = 0;
+    const cudaError_t e = dalloc(p, size_t(*blocks) * per);
+    if (e == cudaSuccess) {
+      *cap = size_t(*blocks) * per;
+    } else if (e == cudaErrorMemoryAllocation && *blocks > 1) {
+      cudaGetLastError();
+      *blocks = (*blocks + 1) / 2;
+    } else {
+      return cuda_fail(c, e, "energy workspace");
+    }
+  }
+  return GDA_OK;
+}
+
+// The digit workspaces of the final energies of R restarts: *mp row blocks of
+// J and *np column blocks of spins fit at a time.
+gda_status reserve_digits(gda_ctx* c, const EnergyProb& p, int* mp, int* np) {
+  if (!c->erexp) CK(dalloc(&c->erexp, size_t(c->Np)));
+  const size_t perJ = energy_J_bytes(p) / p.mtn, perS = energy_S_bytes(p) / p.ntn;
+  *mp = int(std::min<size_t>(p.mtn, std::max<size_t>(1, kEnergyJBytes / perJ)));
+  *np = int(std::min<size_t>(p.ntn, std::max<size_t>(1, kEnergySBytes / perS)));
+  if (c->eJd_cap < size_t(*mp) * perJ) c->eJ_ready = false;
+  const gda_status s = ensure_digits(c, &c->eJd, &c->eJd_cap, perJ, mp);
+  return s == GDA_OK ? ensure_digits(c, &c->eSd, &c->eSd_cap, perS, np) : s;
+}
+
+// With the state, so that energy calls allocate nothing; short of memory the
+// workspaces shrink to panels.
+gda_status reserve_state_digits(gda_ctx* c) {
+  int mp = 0, np = 0;
+  return reserve_digits(c, energy_prob(c->N, c->Np, c->Np, c->R, c->C, c->cplx, c->jmax), &mp, &np);
+}
+
 // Allocates (or keeps) the state for R restarts; padding stays zero.
 gda_status ensure_state(gda_ctx* c, int R) {
   const int C = c->cplx ? 2 * R : R;
   if (c->Rcap_cols >= C && c->psi[0]) {
     c->R = R;
     c->C = C;
-    return GDA_OK;
+    return reserve_state_digits(c);
   }
   free_state(c);
   const size_t Cp = round_up(C, 256), Np = c->Np;
@@ -226,7 +264,7 @@ gda_status ensure_state(gda_ctx* c, int R) {
   c->Rp = int(Rp);
   c->MT = int(MT);
   c->Rcap_cols = int(Cp);
-  return GDA_OK;
+  return reserve_state_digits(c);
 }
 
 // Uploads J (N x N, row-major) and g into the padded FP64 copies, checks the
@@ -453,25 +491,6 @@ gda_status run_gdmod(gda_ctx* c, const gda_params* p, int R, int64_t steps) {
   return GDA_OK;
 }
 
-// Grows a digit workspace to at least `blocks` blocks of `per` bytes, halving
-// the request while memory is short; *blocks receives what fits.
-gda_status ensure_digits(gda_ctx* c, unsigned char** p, size_t* cap, size_t per, int* blocks) {
-  while (*cap < size_t(*blocks) * per) {
-    dfree(*p);
-    *cap = 0;
-    const cudaError_t e = dalloc(p, size_t(*blocks) * per);
-    if (e == cudaSuccess) {
-      *cap = size_t(*blocks) * per;
-    } else if (e == cudaErrorMemoryAllocation && *blocks > 1) {
-      cudaGetLastError();
-      *blocks = (*blocks + 1) / 2;
-    } else {
-      return cuda_fail(c, e, "energy workspace");
-    }
-  }
-  return GDA_OK;
-}
-
 // FP64 Eq. (1) energies of R restarts (C columns) of psi into E64
 // (energy_tc.cu), in panels that fit the digit workspaces.
 gda_status energies_of(gda_ctx* c, const float* psi, int R, int C) {
@@ -482,16 +501,16 @@ gda_status energies_of(gda_ctx* c, const float* psi, int R, int C) {
   p.S64 = c->S64;
   p.part = c->part64;
   p.ldp = c->Rp;
-  if (!c->erexp) CK(dalloc(&c->erexp, size_t(c->Np)));
-  p.rexp = c->erexp;
   const int MT = p.mtn, NT = p.ntn;
-  const size_t perJ = energy_J_bytes(p) / MT, perS = energy_S_bytes(p) / NT;
-  int mp = int(std::min<size_t>(MT, std::max<size_t>(1, kEnergyJBytes / perJ)));
-  int np = int(std::min<size_t>(NT, std::max<size_t>(1, kEnergySBytes / perS)));
-  if (c->eJd_cap < size_t(mp) * perJ) c->eJ_ready = false;
-  gda_status s = ensure_digits(c, &c->eJd, &c->eJd_cap, perJ, &mp);
-  if (s == GDA_OK) s = ensure_digits(c, &c->eSd, &c->eSd_cap, perS, &np);
+  int mp = 0, np = 0;
+  gda_status s = reserve_digits(c, p, &mp, &np);
   if (s != GDA_OK) return s;
+  p.rexp = c->erexp;
+  // work recorded into a graph runs later, maybe after another gda_load: it
+  // makes its own digits and leaves the flag alone
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(c->stream, &cs) != cudaSuccess) cudaGetLastError();
+  const bool recording = cs != cudaStreamCaptureStatusNone;
   p.Jd = c->eJd;
   p.Sd = c->eSd;
   for (int m = 0; m < MT; m += mp) {
@@ -500,9 +519,9 @@ gda_status energies_of(gda_ctx* c, const float* psi, int R, int C) {
     EnergyUnits u{};
     u.KBmax = p.KB;
     u.n_row = p.mtn;
-    if (!c->eJ_ready) {
+    if (!c->eJ_ready || recording) {
       LK(launch_energy_slice_J(p, u, c->stream));
-      c->eJ_ready = mp == MT;
+      if (!recording) c->eJ_ready = mp == MT;
     }
     for (int n = 0; n < NT; n += np) {
       p.nt0 = n;

@@ -115,3 +115,30 @@ def test_batch_energies_equal_single_instances(gda):
             s.close()
         b.run(gda.default_params(dt=0.01, prec=gda.BF16, init_mode=2), 12)
     b.close()
+
+
+def test_energies_recorded_into_a_graph(gda):
+    # a recorded gda_energy_dev follows the instance loaded when it is replayed
+    import torch
+    n, R = 200, 40
+    st = torch.cuda.Stream()
+    J1, J2 = synth.sk_gaussian(n, 1)[0], synth.sk_gaussian(n, 2)[0]
+    psi = synth.initial_amplitudes(n, R, 4, 1.0, True)
+    s = gda.Solver(J1, None, gda.XY, stream=st)
+    s.set_state(psi)
+    E = torch.zeros(R, dtype=torch.float64, device="cuda")
+    g = torch.cuda.CUDAGraph()
+    torch.cuda.synchronize()
+    with torch.cuda.stream(st):
+        g.capture_begin()
+        s.energy_dev(E.data_ptr())  # the first energy call of this context
+        g.capture_end()
+    for J in (J1, J2, J1):
+        s.load(J)
+        s.set_state(psi)
+        with torch.cuda.stream(st):
+            g.replay()
+        torch.cuda.synchronize()
+        got = E.cpu().numpy()
+        assert np.array_equal(got, s.energy())
+    s.close()
