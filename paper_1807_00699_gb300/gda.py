@@ -114,6 +114,18 @@ class GdaError(RuntimeError):
         self.status = status
 
 
+def _interleave(x: np.ndarray, xy: bool) -> np.ndarray:
+    """Amplitudes as the ABI's flat floats: (re, im) pairs (XY) or reals (Ising)."""
+    if xy:  # complex64 lies in memory as those pairs
+        return np.ascontiguousarray(x, dtype=np.complex64).ravel().view(np.float32)
+    return np.ascontiguousarray(x, dtype=np.float32).ravel()
+
+
+def _amplitudes(flat: np.ndarray, R: int, N: int, W: int) -> np.ndarray:
+    """The ABI's flat floats as (R, N) complex64 (W = 2) or float32 amplitudes, without a copy."""
+    return flat.view(np.complex64).reshape(R, N) if W == 2 else flat.reshape(R, N)
+
+
 def _ptr(a: np.ndarray, typ):
     return a.ctypes.data_as(ct.POINTER(typ))
 
@@ -223,18 +235,13 @@ class Solver:
         step = ct.c_int64()
         self._check(self._lib.gda_get_state(self._h, _ptr(psi, ct.c_float), _ptr(gam, ct.c_float),
                                             _ptr(beta, ct.c_float), ct.byref(step)))
-        psi = psi.reshape(R, N, W)
-        psi = psi[..., 0] + 1j * psi[..., 1] if W == 2 else psi[..., 0]
-        return psi, gam.reshape(R, N), beta, step.value
+        return _amplitudes(psi, R, N, W), gam.reshape(R, N), beta, step.value
 
     def set_state(self, psi: np.ndarray, gamma: np.ndarray | None = None, beta: np.ndarray | None = None,
                   step: int = 0):
         psi = np.asarray(psi)
         R = psi.shape[0]
-        if self.model == XY:
-            flat = np.stack([psi.real, psi.imag], axis=-1).astype(np.float32).ravel()
-        else:
-            flat = np.ascontiguousarray(psi, dtype=np.float32).ravel()
+        flat = _interleave(psi, self.model == XY)
         gp = None if gamma is None else _ptr(np.ascontiguousarray(gamma, dtype=np.float32), ct.c_float)
         bp = None if beta is None else _ptr(np.ascontiguousarray(beta, dtype=np.float32), ct.c_float)
         self._check(self._lib.gda_set_state(self._h, _ptr(flat, ct.c_float), gp, bp, R, int(step)))
@@ -263,15 +270,11 @@ class Solver:
         """Y = J0 X (the coupling product alone) for X of shape (R, N)."""
         X = np.asarray(X)
         R = X.shape[0]
-        if self.model == XY:
-            flat = np.stack([X.real, X.imag], axis=-1).astype(np.float32).ravel()
-        else:
-            flat = np.ascontiguousarray(X, dtype=np.float32).ravel()
+        flat = _interleave(X, self.model == XY)
         Y = np.empty_like(flat)
         self._check(self._lib.gda_coupling(self._h, prec, R, _ptr(flat, ct.c_float), _ptr(Y, ct.c_float)))
         self.R = R
-        Y = Y.reshape(R, self.N, self.width)
-        return Y[..., 0] + 1j * Y[..., 1] if self.model == XY else Y[..., 0]
+        return _amplitudes(Y, R, self.N, self.width)
 
     def profile(self, enable: bool = True):
         self._check(self._lib.gda_profile(self._h, 1 if enable else 0))
@@ -401,9 +404,7 @@ class Batch:
         beta = np.empty(R, dtype=np.float32)
         self._check(self._lib.gda_batch_get_state(self._h, k, _ptr(psi, ct.c_float), _ptr(gam, ct.c_float),
                                                   _ptr(beta, ct.c_float)))
-        psi = psi.reshape(R, N, W)
-        psi = psi[..., 0] + 1j * psi[..., 1] if W == 2 else psi[..., 0]
-        return psi, gam.reshape(R, N), beta
+        return _amplitudes(psi, R, N, W), gam.reshape(R, N), beta
 
     def close(self):
         if getattr(self, "_h", None):
