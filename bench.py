@@ -44,7 +44,7 @@ METRIC = "time-to-target energy (s) & spin-updates/s: BF16+learned vs plain FP32
 # DRAM bytes (read + write) per step of each workload's dominant kernel, from
 # one-launch ncu captures (profiles/): the streaming kernel's 3-step launch moved
 # 873.3 + 482.1 MB; None where no capture of the current kernel exists.
-TRAFFIC = {"sk4096": (873.272064e6 + 482.108672e6) / 3, "xy1000": None}
+TRAFFIC = {"sk4096": (841.058048e6 + 478.54464e6) / 3, "xy1000": None}
 
 
 def parse():

@@ -234,8 +234,8 @@ gda_status gda_run(gda_ctx* ctx, const gda_params* p, int32_t R, int64_t steps);
  * (GDA_ERR_DIVERGED, GDA_ERR_TIMEOUT).  The error flags are cleared. */
 gda_status gda_sync(gda_ctx* ctx);
 
-/* Eq. (1) energy of the projected spins of every restart, in FP64 (exact,
- * through an int64 reduction, for Ising runs with integer J and g = 0).
+/* Eq. (1) energy of the projected spins of every restart, in FP64 (exact for
+ * Ising runs with integer J and g = 0).
  * E: R doubles on the host.  Synchronises. */
 gda_status gda_energy(gda_ctx* ctx, double* E);
 
@@ -243,11 +243,8 @@ gda_status gda_energy(gda_ctx* ctx, double* E);
  * synchronise. */
 gda_status gda_energy_dev(gda_ctx* ctx, double* E_dev);
 
-/* Lowest Eq. (1) energy over the restarts (ties: lowest restart index), the
- * same answer and FP64 value as the argmin of gda_energy.  For non-integer
- * energies and R >= 32 it first bounds every restart's energy with
- * compensated FP32 sums (error below 48 * 2^-24 * (sum |J0| + sum |g|)) and
- * evaluates in FP64 only the restarts within twice that bound of the lowest.
+/* Lowest Eq. (1) energy over the restarts (ties: lowest restart index): the
+ * argmin of gda_energy, with its FP64 value.
  * E, r: host scalars (either may be NULL).  cfg (may be NULL): N int8 spins
  * (+1/-1) for Ising, or N doubles theta_i in (-pi, pi] for XY (on the q-th
  * roots of unity after a run with a resonant drive), host.  Synchronises. */
