@@ -23,9 +23,9 @@
 // plain 16 KB bulk copies.  Warp 0 loads, warp 1 issues MMAs into two
 // tensor-memory accumulators in turn, 16 warps drain them.  What bounds it is
 // the delivery of 32 KB of digits per 128 x 128 x 64 product from L2.
-// Measured (GB300): every restart's energy at XY N = 1000, R = 1024 takes 232
-// us here plus 84 us for the spins' digits, where the FP64 pipe took 4.10 ms;
-// the lowest of SK N = R = 4096 takes 3 ms, where ranking in compensated FP32
+// Measured (GB300): every restart's energy at XY N = 1000, R = 1024 takes 218
+// us here plus 83 us for the spins' digits, where the FP64 pipe took 4.10 ms;
+// the lowest of SK N = R = 4096 takes 1.1 ms, where ranking in compensated FP32
 // and evaluating the candidates in FP64 took 11.1 ms.  Against sums in
 // extended precision the energies are 2-5 times closer than the FP64 pipe's
 // (relative error, N = 150 / 777 / 1000: 1.4e-16 / 1.4e-16 / 1.8e-16, before
