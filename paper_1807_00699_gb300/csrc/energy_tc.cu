@@ -55,6 +55,21 @@ __device__ __forceinline__ int4 unit_of(const int4* u, int k, int rows) {
   return u ? u[k] : make_int4(0, k % rows, k / rows, 0);
 }
 
+// Digits of J, and whether they are J's own (EnergyProb::fmt).
+__device__ __forceinline__ int2 format_of(const EnergyProb& P) { return P.fmt ? *P.fmt : make_int2(P.nsJ, P.jint); }
+
+// Integers up to 2^(8 n - 1) are their own n digits; 0: J takes scaled digits.
+__host__ __device__ inline int integer_digits(double jmax) {
+  for (int n = 1; n <= 4; ++n)
+    if (jmax >= 0.0 && jmax <= double(1ll << (8 * n - 1))) return n;
+  return 0;
+}
+
+__global__ void k_energy_format(const int* flags, const unsigned long long* maxabs, int2* fmt) {
+  const int n = (*flags & 4) ? 0 : integer_digits(__longlong_as_double((long long)*maxabs));
+  *fmt = n ? make_int2(n, 1) : make_int2(kEnergySlices, 0);
+}
+
 // Byte offset of the 16-byte group k8 (8 values) of row r inside a digit tile.
 __device__ __forceinline__ uint32_t tile_off(int r, int k8) { return uint32_t(r) * 128u + uint32_t((k8 ^ (r & 7)) << 4); }
 
@@ -86,8 +101,9 @@ __global__ void __launch_bounds__(256) k_energy_rexp(EnergyProb p0, const Energy
   const int lane = threadIdx.x & 31;
   const int i = (P.mt0 + U.y) * TILE + int(blockIdx.y) * 8 + int(threadIdx.x >> 5);
   if (i >= P.N) return;
-  int e = 8 * P.nsJ - 1;
-  if (!P.jint) {
+  const int2 F = format_of(P);
+  int e = 8 * F.x - 1;
+  if (!F.y) {
     double m = 0.0;
     for (int j = lane; j < P.N; j += 32) m = fmax(m, fabs(P.J[size_t(i) * P.ld + j]));
     for (int o = 16; o; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
@@ -102,7 +118,7 @@ __global__ void __launch_bounds__(256) k_energy_slice_J(EnergyProb p0, const Ene
   const EnergyProb& P = probs ? probs[U.x] : p0;
   const int kb = blockIdx.y;
   if (kb >= P.KB) return;
-  const int ns = P.nsJ;
+  const int ns = format_of(P).x;
   unsigned char* out = P.Jd + (size_t(U.y) * ns * P.KB + kb) * TBYTES;
   for (int q = threadIdx.x; q < TILE * 8; q += 256) {
     const int r = q >> 3, k8 = q & 7;
@@ -198,8 +214,7 @@ __global__ void __launch_bounds__(256) k_energy_slice_S(EnergyProb p0, const Ene
 // The digit pairs of a problem in one order for all warp roles.
 struct PairIter {
   int nsJ, nsS, lim, i, j;
-  __device__ explicit PairIter(const EnergyProb& P)
-      : nsJ(P.nsJ), nsS(P.nsS), lim(P.nsJ > P.nsS ? P.nsJ : P.nsS), i(0), j(0) {}
+  __device__ PairIter(int J, int S) : nsJ(J), nsS(S), lim(J > S ? J : S), i(0), j(0) {}
   __device__ bool done() const { return i >= nsJ; }
   __device__ void next() {
     ++j;
@@ -240,6 +255,7 @@ __global__ void __launch_bounds__(ETHREADS, 1) k_energy_product(const __grid_con
   auto acc_full = [&](int b) { return smem_u32(bars + 2 * STAGES + b); };
   auto acc_empty = [&](int b) { return smem_u32(bars + 2 * STAGES + 2 + b); };
   auto aborted = [&]() { return *(volatile int*)&s_abort != 0; };
+  const int ns0 = probs ? 0 : format_of(p0).x;  // problems of a list carry their own
   if (threadIdx.x == 0) {
     for (int s = 0; s < STAGES; ++s) {
       mbar_init(full_bar(s), 1);
@@ -265,8 +281,9 @@ __global__ void __launch_bounds__(ETHREADS, 1) k_energy_product(const __grid_con
       for (int t = blockIdx.x; t < n_tile && !stop; t += gridDim.x) {
         const int4 U = unit_of(units, t, p0.mtn);
         const EnergyProb& P = probs ? probs[U.x] : p0;
-        for (PairIter q(P); !q.done() && !stop; q.next()) {
-          const unsigned char* A = P.Jd + (size_t(U.y) * P.nsJ + q.i) * P.KB * TBYTES;
+        const int nsJ = probs ? P.nsJ : ns0;
+        for (PairIter q(nsJ, P.nsS); !q.done() && !stop; q.next()) {
+          const unsigned char* A = P.Jd + (size_t(U.y) * nsJ + q.i) * P.KB * TBYTES;
           const unsigned char* B = P.Sd + (size_t(U.z) * P.nsS + q.j) * P.KB * TBYTES;
           for (int kb = 0; kb < P.KB; ++kb, ++it) {
             const int s = it % STAGES;
@@ -296,8 +313,9 @@ __global__ void __launch_bounds__(ETHREADS, 1) k_energy_product(const __grid_con
       for (int t = blockIdx.x; t < n_tile && !stop; t += gridDim.x) {
         const int4 U = unit_of(units, t, p0.mtn);
         const EnergyProb& P = probs ? probs[U.x] : p0;
+        const int nsJ = probs ? P.nsJ : ns0;
         const int ck = chunk_kb(P);
-        for (PairIter q(P); !q.done() && !stop; q.next()) {
+        for (PairIter q(nsJ, P.nsS); !q.done() && !stop; q.next()) {
           for (int k0 = 0; k0 < P.KB && !stop; k0 += ck, ++use) {
             const int b = use & 1;
             if (!mbar_wait(acc_empty(b), ((use >> 1) & 1) ^ 1, lim) || aborted()) {
@@ -337,16 +355,17 @@ __global__ void __launch_bounds__(ETHREADS, 1) k_energy_product(const __grid_con
     for (int t = blockIdx.x; t < n_tile; t += gridDim.x) {
       const int4 U = unit_of(units, t, p0.mtn);
       const EnergyProb& P = probs ? probs[U.x] : p0;
+      const int nsJ = probs ? P.nsJ : ns0;
       const int ck = chunk_kb(P);
       // unit of the int64 sums: 2^unit of digit weight one, so that |sum| < 2^62
-      const int fb = 8 * P.nsJ - 1 + (P.nsS > 1 ? 8 * P.nsS - 1 : 0);
+      const int fb = 8 * nsJ - 1 + (P.nsS > 1 ? 8 * P.nsS - 1 : 0);
       const int lg = P.N > 1 ? 32 - __clz(P.N - 1) : 0;
       const int unit = fb + lg + 1 > 62 ? fb + lg + 1 - 62 : 0;
       long long acc[32];
 #pragma unroll
       for (int k = 0; k < 32; ++k) acc[k] = 0;
       bool ok = true;
-      for (PairIter q(P); !q.done() && ok; q.next()) {
+      for (PairIter q(nsJ, P.nsS); !q.done() && ok; q.next()) {
         const int sh = q.weight() - unit;
         for (int k0 = 0; k0 < P.KB; k0 += ck, ++use) {
           const int b = use & 1;
@@ -462,12 +481,10 @@ EnergyProb energy_prob(int N, int Np, int ld, int R, int C, int pmode, double jm
   p.KB = (N + 63) / 64;
   p.nsJ = kEnergySlices;
   p.nsS = pmode ? kEnergySlices : 1;
-  // integers up to 2^(8 n - 1) are their own digits
-  for (int n = 1; n <= 4 && !p.jint; ++n)
-    if (jmax >= 0.0 && jmax <= std::ldexp(1.0, 8 * n - 1)) {
-      p.nsJ = n;
-      p.jint = 1;
-    }
+  if (const int n = integer_digits(jmax)) {
+    p.nsJ = n;
+    p.jint = 1;
+  }
   p.mtn = (N + TILE - 1) / TILE;
   p.ntn = (C + TILE - 1) / TILE;
   return p;
@@ -475,6 +492,11 @@ EnergyProb energy_prob(int N, int Np, int ld, int R, int C, int pmode, double jm
 
 size_t energy_J_bytes(const EnergyProb& p) { return size_t(p.mtn) * p.nsJ * p.KB * kEnergyTileBytes; }
 size_t energy_S_bytes(const EnergyProb& p) { return size_t(p.ntn) * p.nsS * p.KB * kEnergyTileBytes; }
+
+cudaError_t launch_energy_format(const int* flags, const unsigned long long* maxabs, int2* fmt, cudaStream_t s) {
+  k_energy_format<<<1, 1, 0, s>>>(flags, maxabs, fmt);
+  return cudaGetLastError();
+}
 
 cudaError_t launch_energy_slice_J(const EnergyProb& p0, const EnergyUnits& u, cudaStream_t s) {
   k_energy_rexp<<<dim3(u.n_row, TILE / 8), 256, 0, s>>>(p0, u.probs, u.row);

@@ -29,14 +29,22 @@ struct EnergyProb {
   int nsJ, nsS, KB;     // digits of J and of s; K blocks of 64 spins
   int jint;             // J holds integers with |J_ij| <= 2^(8 nsJ - 1): digits of J itself
   int mt0, mtn, nt0, ntn;
+  // nsJ and jint of the J loaded when the kernels run, on the device, or
+  // nullptr: those above.  Work recorded into a graph outlives the J it was
+  // recorded with.
+  const int2* fmt;
 };
 
 // Digits, K blocks and tile counts of an N-spin instance with C columns
 // (pointers and panel ranges are the caller's; the panel covers everything).
 // jmax: the largest |J_ij| when every J_ij is an integer, else a negative value.
+// (A caller with fmt passes -1 and gets sizes that hold any J.)
 EnergyProb energy_prob(int N, int Np, int ld, int R, int C, int pmode, double jmax);
 size_t energy_J_bytes(const EnergyProb& p);  // digit bytes of the panel's rows
 size_t energy_S_bytes(const EnergyProb& p);  // digit bytes of the panel's columns
+
+// *fmt = (nsJ, jint) of the checked J: flags and maxabs of launch_check_instance.
+cudaError_t launch_energy_format(const int* flags, const unsigned long long* maxabs, int2* fmt, cudaStream_t s);
 
 // units (device, or nullptr with probs = nullptr: the one problem p0): n_row
 // entries (problem, row block), n_col entries (problem, column block) and

@@ -42,7 +42,6 @@ struct gda_ctx {
   double* g64 = nullptr;  // [Np]
   float* g32 = nullptr;   // [Np]
   float* h1 = nullptr;    // [Np]
-  double jmax = -1.0;     // largest |J_ij| when every J_ij is an integer, else -1
   double diag = 0.0;      // -sum_i J_ii
   // instance checks
   int* d_flags = nullptr;
@@ -76,10 +75,15 @@ struct gda_ctx {
   int K_R = 0;         // restarts K was initialised for (0: none)
   double* S64 = nullptr;      // complex spins of the final energies
   double* part64 = nullptr;
-  int* erexp = nullptr;       // final energies: row exponents and digit tiles of J, digit tiles of the spins
+  // Final energies: row exponents and digit tiles of J, digit tiles of the
+  // spins.  Recorded energy calls keep their addresses: what belongs to J is
+  // sized for any J and stays with the context, what belongs to the spins is
+  // sized for the state's capacity and stays with the state.
+  int* erexp = nullptr;       // [Np]
+  int2* efmt = nullptr;       // (digits of J, whether J's own) of the current J
   unsigned char* eJd = nullptr;
   unsigned char* eSd = nullptr;
-  size_t eJd_cap = 0, eSd_cap = 0;
+  int eJ_blocks = 0, eS_blocks = 0;  // row / column blocks they hold
   bool eJ_ready = false;      // eJd holds the whole current J
   double* E64 = nullptr;
   double* bestE = nullptr;
@@ -172,7 +176,7 @@ void free_state(gda_ctx* c) {
     dfree(c->rho[k]);
   }
   dfree(c->acc); dfree(c->S32); dfree(c->gam); dfree(c->gstg); dfree(c->gacc); dfree(c->epart);
-  dfree(c->ops); dfree(c->S64); dfree(c->part64); dfree(c->E64);
+  dfree(c->ops); dfree(c->S64); dfree(c->eSd); dfree(c->part64); dfree(c->E64);
   if (c->plan) tc_plan_destroy(c->plan);
   c->plan = nullptr;
   dfree(c->ops8);
@@ -182,18 +186,16 @@ void free_state(gda_ctx* c) {
   c->have_state = false;
 }
 
-// Grows a digit workspace to at least `blocks` blocks of `per` bytes, halving
-// the request while memory is short; *blocks receives what fits.
-gda_status ensure_digits(gda_ctx* c, unsigned char** p, size_t* cap, size_t per, int* blocks) {
-  while (*cap < size_t(*blocks) * per) {
-    dfree(*p);
-    *cap = 0;
-    const cudaError_t e = dalloc(p, size_t(*blocks) * per);
+// A digit workspace of up to `want` blocks of `per` bytes, halving the request
+// while memory is short.
+gda_status alloc_digits(gda_ctx* c, unsigned char** p, int* blocks, size_t per, int want) {
+  while (!*p) {
+    const cudaError_t e = dalloc(p, size_t(want) * per);
     if (e == cudaSuccess) {
-      *cap = size_t(*blocks) * per;
-    } else if (e == cudaErrorMemoryAllocation && *blocks > 1) {
+      *blocks = want;
+    } else if (e == cudaErrorMemoryAllocation && want > 1) {
       cudaGetLastError();
-      *blocks = (*blocks + 1) / 2;
+      want = (want + 1) / 2;
     } else {
       return cuda_fail(c, e, "energy workspace");
     }
@@ -201,23 +203,17 @@ gda_status ensure_digits(gda_ctx* c, unsigned char** p, size_t* cap, size_t per,
   return GDA_OK;
 }
 
-// The digit workspaces of the final energies of R restarts: *mp row blocks of
-// J and *np column blocks of spins fit at a time.
-gda_status reserve_digits(gda_ctx* c, const EnergyProb& p, int* mp, int* np) {
-  if (!c->erexp) CK(dalloc(&c->erexp, size_t(c->Np)));
+// The digit workspaces of the final energies, with the state, so that energy
+// calls allocate nothing; short of memory they hold panels.
+gda_status reserve_digits(gda_ctx* c) {
+  const EnergyProb p = energy_prob(c->N, c->Np, c->Np, c->cplx ? c->Rcap_cols / 2 : c->Rcap_cols, c->Rcap_cols,
+                                   c->cplx, -1.0);
   const size_t perJ = energy_J_bytes(p) / p.mtn, perS = energy_S_bytes(p) / p.ntn;
-  *mp = int(std::min<size_t>(p.mtn, std::max<size_t>(1, kEnergyJBytes / perJ)));
-  *np = int(std::min<size_t>(p.ntn, std::max<size_t>(1, kEnergySBytes / perS)));
-  if (c->eJd_cap < size_t(*mp) * perJ) c->eJ_ready = false;
-  const gda_status s = ensure_digits(c, &c->eJd, &c->eJd_cap, perJ, mp);
-  return s == GDA_OK ? ensure_digits(c, &c->eSd, &c->eSd_cap, perS, np) : s;
-}
-
-// With the state, so that energy calls allocate nothing; short of memory the
-// workspaces shrink to panels.
-gda_status reserve_state_digits(gda_ctx* c) {
-  int mp = 0, np = 0;
-  return reserve_digits(c, energy_prob(c->N, c->Np, c->Np, c->R, c->C, c->cplx, c->jmax), &mp, &np);
+  const gda_status s = alloc_digits(c, &c->eJd, &c->eJ_blocks, perJ,
+                                    int(std::min<size_t>(p.mtn, std::max<size_t>(1, kEnergyJBytes / perJ))));
+  if (s != GDA_OK) return s;
+  return alloc_digits(c, &c->eSd, &c->eS_blocks, perS,
+                      int(std::min<size_t>(p.ntn, std::max<size_t>(1, kEnergySBytes / perS))));
 }
 
 // Allocates (or keeps) the state for R restarts; padding stays zero.
@@ -226,7 +222,7 @@ gda_status ensure_state(gda_ctx* c, int R) {
   if (c->Rcap_cols >= C && c->psi[0]) {
     c->R = R;
     c->C = C;
-    return reserve_state_digits(c);
+    return reserve_digits(c);
   }
   free_state(c);
   const size_t Cp = round_up(C, 256), Np = c->Np;
@@ -264,7 +260,7 @@ gda_status ensure_state(gda_ctx* c, int R) {
   c->Rp = int(Rp);
   c->MT = int(MT);
   c->Rcap_cols = int(Cp);
-  return reserve_state_digits(c);
+  return reserve_digits(c);
 }
 
 // Uploads J (N x N, row-major) and g into the padded FP64 copies, checks the
@@ -276,24 +272,20 @@ gda_status load_instance(gda_ctx* c, const double* J, const double* g, cudaMemcp
   CK(cudaMemsetAsync(c->g64, 0, Np * sizeof(double), c->stream));
   if (g) CK(cudaMemcpyAsync(c->g64, g, N * sizeof(double), kind, c->stream));
   c->K_R = 0;  // a GD-mod coupling state belongs to the previous J
+  c->eJ_ready = false;
   LK(launch_snapshot_reset(c->snapE, c->snapR, c->snapStep, c->stream));
   c->ell_maxdeg = -1;
   CK(cudaMemsetAsync(c->d_flags, 0, sizeof(int), c->stream));
   CK(cudaMemsetAsync(c->d_maxabs, 0, sizeof(unsigned long long), c->stream));
   LK(launch_check_instance(c->J64, c->g64, c->N, c->Np, c->d_flags, c->d_maxabs, c->d_diag, c->stream));
+  LK(launch_energy_format(c->d_flags, c->d_maxabs, c->efmt, c->stream));
   int flags = 0;
-  unsigned long long mbits = 0;
   CK(cudaMemcpyAsync(&flags, c->d_flags, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
-  CK(cudaMemcpyAsync(&mbits, c->d_maxabs, sizeof(mbits), cudaMemcpyDeviceToHost, c->stream));
   CK(cudaMemcpyAsync(&c->diag, c->d_diag, sizeof(double), cudaMemcpyDeviceToHost, c->stream));
   CK(cudaStreamSynchronize(c->stream));
   if (flags & 1) return fail(c, GDA_ERR_INVALID, "J has a non-finite entry");
   if (flags & 2) return fail(c, GDA_ERR_INVALID, "J is not symmetric");
   if (flags & 8) return fail(c, GDA_ERR_INVALID, "g has a non-finite entry");
-  double maxabs;
-  std::memcpy(&maxabs, &mbits, sizeof(maxabs));
-  c->jmax = (flags & 4) ? -1.0 : maxabs;
-  c->eJ_ready = false;
   LK(launch_prepare_J(c->J64, c->Np, c->J32, c->J16, c->stream));
   c->j8_ready = false;
   return GDA_OK;
@@ -494,25 +486,23 @@ gda_status run_gdmod(gda_ctx* c, const gda_params* p, int R, int64_t steps) {
 // FP64 Eq. (1) energies of R restarts (C columns) of psi into E64
 // (energy_tc.cu), in panels that fit the digit workspaces.
 gda_status energies_of(gda_ctx* c, const float* psi, int R, int C) {
-  EnergyProb p = energy_prob(c->N, c->Np, c->Np, R, C, pmode(c), c->jmax);
+  EnergyProb p = energy_prob(c->N, c->Np, c->Np, R, C, pmode(c), -1.0);
   p.J = c->J64;
   p.g = c->g64;
   p.psi = psi;
   p.S64 = c->S64;
   p.part = c->part64;
   p.ldp = c->Rp;
-  const int MT = p.mtn, NT = p.ntn;
-  int mp = 0, np = 0;
-  gda_status s = reserve_digits(c, p, &mp, &np);
-  if (s != GDA_OK) return s;
   p.rexp = c->erexp;
+  p.fmt = c->efmt;
+  p.Jd = c->eJd;
+  p.Sd = c->eSd;
+  const int MT = p.mtn, NT = p.ntn, mp = c->eJ_blocks, np = c->eS_blocks;
   // work recorded into a graph runs later, maybe after another gda_load: it
-  // makes its own digits and leaves the flag alone
+  // makes the digits of the J it finds, in the form direct calls expect
   cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
   if (cudaStreamIsCapturing(c->stream, &cs) != cudaSuccess) cudaGetLastError();
   const bool recording = cs != cudaStreamCaptureStatusNone;
-  p.Jd = c->eJd;
-  p.Sd = c->eSd;
   for (int m = 0; m < MT; m += mp) {
     p.mt0 = m;
     p.mtn = std::min(mp, MT - m);
@@ -521,7 +511,7 @@ gda_status energies_of(gda_ctx* c, const float* psi, int R, int C) {
     u.n_row = p.mtn;
     if (!c->eJ_ready || recording) {
       LK(launch_energy_slice_J(p, u, c->stream));
-      if (!recording) c->eJ_ready = mp == MT;
+      if (!recording) c->eJ_ready = mp >= MT;
     }
     for (int n = 0; n < NT; n += np) {
       p.nt0 = n;
@@ -605,7 +595,7 @@ void gda_destroy(gda_ctx* c) {
   dfree(c->J64); dfree(c->J32); dfree(c->J16); dfree(c->J8); dfree(c->jscale); dfree(c->g64); dfree(c->g32); dfree(c->h1);
   dfree(c->d_flags); dfree(c->d_maxabs); dfree(c->d_diag);
   dfree(c->bestE); dfree(c->bestR); dfree(c->cfg8); dfree(c->cfgth);
-  dfree(c->erexp); dfree(c->eJd); dfree(c->eSd);
+  dfree(c->erexp); dfree(c->efmt); dfree(c->eJd);
   dfree(c->t_step); dfree(c->t_E); dfree(c->t_r); dfree(c->t_count); dfree(c->err); dfree(c->flags);
   dfree(c->seg_flags);
   dfree(c->lastE); dfree(c->lastR); dfree(c->snapE); dfree(c->snapR); dfree(c->snapStep); dfree(c->snap);
@@ -678,6 +668,8 @@ static gda_status create_impl(const double* J, const double* g, int32_t N, int32
   step(dalloc(&c->snapStep, 1));
   step(dalloc(&c->snap, 2 * Np));
   step(dalloc(&c->d_zero, 1));
+  step(dalloc(&c->erexp, Np));
+  step(dalloc(&c->efmt, 1));
   step(dalloc(&c->err, 1));
   step(dalloc(&c->flags, kMaxResidentTiles));
   if (st == GDA_OK) step(cudaMemset(c->err, 0, sizeof(int)));
