@@ -11,10 +11,12 @@
 // -x the negated digits of x.  A digit is a BF16 number; a product of digits
 // is an integer <= 2^14, so FP32 accumulation over at most 512 of them (sums
 // <= 2^23) is exact.  Each accumulator is added, shifted to its weight, into
-// an int64 whose unit is 2^-(61 - ceil(log2 N)) of the row's largest |J_ij|:
-// the sum over j cannot overflow, and its error (the digit pairs below the
-// unit, k + l > 6, are left out) stays below the rounding errors of the same
-// sum in FP64.  Real spins are +-1: one digit, 7 products.  Integer J takes
+// an int64 whose unit is 2^-61 of sum_j |J_ij| (the largest of 32 rows), or
+// the weight of the last digit where that is coarser: the sum over j cannot
+// overflow, and its error (the digit pairs below the unit, k + l > 6, are left
+// out) stays below the rounding errors of the same sum in FP64, for rows of a
+// few nonzeros as well (a bound of N times the largest |J_ij| in place of the
+// sum loses 6 bits on 3-regular rows at N = 4096).  Real spins are +-1: one digit, 7 products.  Integer J takes
 // as many digits as its largest entry needs and no scaling, so those energies
 // are exact integers.
 //
@@ -94,7 +96,9 @@ __device__ __forceinline__ void digits(long long x, int ns, unsigned short (&d)[
   }
 }
 
-// e_i with |J_ij| <= 2^e_i for every j (one warp per row; integers: the scale of the digits of J itself).
+// (e_i, l_i) with |J_ij| <= 2^e_i for every j and sum_j |J_ij| < 2^(e_i + l_i), a
+// factor 2 of rounding aside (one warp per row; integers: e_i the scale of the
+// digits of J itself).
 __global__ void __launch_bounds__(256) k_energy_rexp(EnergyProb p0, const EnergyProb* probs, const int4* units) {
   const int4 U = unit_of(units, blockIdx.x, p0.mtn);
   const EnergyProb& P = probs ? probs[U.x] : p0;
@@ -102,14 +106,20 @@ __global__ void __launch_bounds__(256) k_energy_rexp(EnergyProb p0, const Energy
   const int i = (P.mt0 + U.y) * TILE + int(blockIdx.y) * 8 + int(threadIdx.x >> 5);
   if (i >= P.N) return;
   const int2 F = format_of(P);
-  int e = 8 * F.x - 1;
-  if (!F.y) {
-    double m = 0.0;
-    for (int j = lane; j < P.N; j += 32) m = fmax(m, fabs(P.J[size_t(i) * P.ld + j]));
-    for (int o = 16; o; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
-    e = m > 0.0 ? ilogb(m) + 1 : 0;
+  double m = 0.0, a = 0.0;
+  for (int j = lane; j < P.N; j += 32) {
+    const double v = fabs(P.J[size_t(i) * P.ld + j]);
+    m = fmax(m, v);
+    a += v;
   }
-  if (lane == 0) P.rexp[i] = e;
+  for (int o = 16; o; o >>= 1) {
+    m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
+    a += __shfl_xor_sync(0xffffffffu, a, o);
+  }
+  const int e = F.y ? 8 * F.x - 1 : m > 0.0 ? ilogb(m) + 1 : 0;
+  const int lgN = P.N > 1 ? 32 - __clz(P.N - 1) : 0;
+  const int l = !(m > 0.0) ? 0 : isfinite(a) ? ilogb(a) + 1 - e : lgN;
+  if (lane == 0) P.rexp[i] = make_int2(e, l);
 }
 
 // Digit tiles of J: one CTA per (row block, K block).
@@ -125,7 +135,7 @@ __global__ void __launch_bounds__(256) k_energy_slice_J(EnergyProb p0, const Ene
     const int i = (P.mt0 + U.y) * TILE + r, j0 = kb * 64 + k8 * 8;
     unsigned short d[8][kEnergySlices] = {};
     if (i < P.N) {
-      const int sh = 8 * ns - 1 - P.rexp[i];
+      const int sh = 8 * ns - 1 - P.rexp[i].x;
 #pragma unroll
       for (int t = 0; t < 8; ++t) {
         const double v = j0 + t < P.N ? P.J[size_t(i) * P.ld + j0 + t] : 0.0;
@@ -357,10 +367,11 @@ __global__ void __launch_bounds__(ETHREADS, 1) k_energy_product(const __grid_con
       const EnergyProb& P = probs ? probs[U.x] : p0;
       const int nsJ = probs ? P.nsJ : ns0;
       const int ck = chunk_kb(P);
-      // unit of the int64 sums: 2^unit of digit weight one, so that |sum| < 2^62
+      const int i = (P.mt0 + U.y) * TILE + 32 * q4 + lane;
+      const int2 re = i < P.N ? P.rexp[i] : make_int2(0, -(1 << 20));
+      // unit of the int64 sums of the warp's rows: 2^unit of digit weight one, so that |sum| < 2^62
       const int fb = 8 * nsJ - 1 + (P.nsS > 1 ? 8 * P.nsS - 1 : 0);
-      const int lg = P.N > 1 ? 32 - __clz(P.N - 1) : 0;
-      const int unit = fb + lg + 1 > 62 ? fb + lg + 1 - 62 : 0;
+      const int unit = max(0, fb + __reduce_max_sync(0xffffffffu, re.y) + 1 - 62);
       long long acc[32];
 #pragma unroll
       for (int k = 0; k < 32; ++k) acc[k] = 0;
@@ -390,11 +401,10 @@ __global__ void __launch_bounds__(ETHREADS, 1) k_energy_product(const __grid_con
       }
       // Eq. (1) terms of row i and their sum over the rows, per restart; one
       // tree over the rows for every column, whatever its place
-      const int i = (P.mt0 + U.y) * TILE + 32 * q4 + lane;
       const int c0 = (P.nt0 + U.z) * TILE + cpart * 32;
       const bool row = ok && i < P.N;
       const double gi = row && P.g ? P.g[i] : 0.0;
-      const int ex = row ? unit - fb + P.rexp[i] : 0;
+      const int ex = row ? unit - fb + re.x : 0;
       const bool wide = ex < -1000 || ex > 900;  // couplings near the ends of the double range
       const double f = __longlong_as_double((long long)((wide ? 0 : ex) + 1023) << 52);
       double v[32];

@@ -20,7 +20,7 @@ struct EnergyProb {
   const double* g;      // [N] or nullptr
   const float* psi;     // amplitudes [C][Np], column-major
   double* S64;          // complex spins s in double [C][Np]; nullptr for real spins
-  int* rexp;            // [N] exponent of every row: |J_ij| <= 2^rexp[i]
+  int2* rexp;           // [N] (e, l) of every row: |J_ij| <= 2^e, sum_j |J_ij| < 2^(e + l)
   unsigned char* Jd;    // digit tiles [mtn][nsJ][KB]
   unsigned char* Sd;    // digit tiles [ntn][nsS][KB]
   double* part;         // [row blocks of 128][ldp] partial energies

@@ -79,7 +79,7 @@ struct gda_ctx {
   // spins.  Recorded energy calls keep their addresses: what belongs to J is
   // sized for any J and stays with the context, what belongs to the spins is
   // sized for the state's capacity and stays with the state.
-  int* erexp = nullptr;       // [Np]
+  int2* erexp = nullptr;      // [Np]
   int2* efmt = nullptr;       // (digits of J, whether J's own) of the current J
   unsigned char* eJd = nullptr;
   unsigned char* eSd = nullptr;

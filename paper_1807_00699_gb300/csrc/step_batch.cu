@@ -537,7 +537,7 @@ struct gda_batch {
   std::vector<EnergyGroup> egroups;
   EnergyProb* eprobs = nullptr;
   int4* eunits = nullptr;
-  int* erexp = nullptr;
+  int2* erexp = nullptr;
   unsigned char* edigits = nullptr;
   bool eJ_ready = false;          // one group: its J digits are kept between calls
   unsigned* step_base = nullptr;
