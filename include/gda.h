@@ -243,6 +243,16 @@ gda_status gda_energy(gda_ctx* ctx, double* E);
  * synchronise. */
 gda_status gda_energy_dev(gda_ctx* ctx, double* E_dev);
 
+/* Bound, in bytes, on the device memory the context keeps for the energies'
+ * form of J between calls (14 N'^2 bytes are needed, N' = N rounded up to 128;
+ * default and most: 2 GiB, and never more than a quarter of what is free when
+ * the state is allocated).  It only saves time: with less, or 0, energy calls
+ * rebuild J's form, in pieces, in the state's scratch memory, and give the same
+ * numbers.  Memory a call cannot do without is taken from it.  Frees what is
+ * kept now.  GDA_ERR_STATE once an energy call that uses it was recorded into
+ * a CUDA graph; GDA_ERR_INVALID for bytes < 0. */
+gda_status gda_set_energy_workspace(gda_ctx* ctx, int64_t bytes);
+
 /* Lowest Eq. (1) energy over the restarts (ties: lowest restart index): the
  * argmin of gda_energy, with its FP64 value.
  * E, r: host scalars (either may be NULL).  cfg (may be NULL): N int8 spins

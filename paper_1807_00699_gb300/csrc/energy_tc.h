@@ -9,7 +9,8 @@ namespace gda {
 
 constexpr int kEnergySlices = 7;                     // 8-bit digits of a 55-bit fixed-point value
 constexpr size_t kEnergyTileBytes = 128 * 64 * 2;    // one digit tile: 128 rows x 64 BF16, swizzled
-// Bounds on the digit workspaces: larger products are cut into panels.
+// Bounds on the digit workspaces (a batch puts both kinds into their sum):
+// larger products are cut into panels.
 constexpr size_t kEnergyJBytes = size_t(2) << 30;
 constexpr size_t kEnergySBytes = size_t(512) << 20;
 

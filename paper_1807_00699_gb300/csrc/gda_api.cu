@@ -50,6 +50,10 @@ struct gda_ctx {
   // state
   int R = 0, C = 0, Cp = 0, Rp = 0, Rcap_cols = 0, MT = 0;
   float* psi[2] = {nullptr, nullptr};
+  // One block of 4 [Cp][Np] arrays that nothing reads across calls: RK stages
+  // and sums, projected spins; get_state stages in it, final energies put
+  // their digits there.
+  float* scratch = nullptr;
   float* stg[2] = {nullptr, nullptr};
   float* acc = nullptr;
   float* S32 = nullptr;
@@ -75,16 +79,16 @@ struct gda_ctx {
   int K_R = 0;         // restarts K was initialised for (0: none)
   double* S64 = nullptr;      // complex spins of the final energies
   double* part64 = nullptr;
-  // Final energies: row exponents and digit tiles of J, digit tiles of the
-  // spins.  Recorded energy calls keep their addresses: what belongs to J is
-  // sized for any J and stays with the context, what belongs to the spins is
-  // sized for the state's capacity and stays with the state.
+  // Final energies: row exponents and digit tiles of J, kept between calls (the
+  // spins' digits lie in scratch).  Sized for any J and not moved once an
+  // energy call that uses them was recorded into a graph.
   int2* erexp = nullptr;      // [Np]
   int2* efmt = nullptr;       // (digits of J, whether J's own) of the current J
-  unsigned char* eJd = nullptr;
-  unsigned char* eSd = nullptr;
-  int eJ_blocks = 0, eS_blocks = 0;  // row / column blocks they hold
-  bool eJ_ready = false;      // eJd holds the whole current J
+  unsigned char* eJd = nullptr;  // nullptr: none kept, energy calls use scratch
+  int eJ_blocks = 0;          // row blocks it holds
+  bool eJ_ready = false;      // it holds the whole current J
+  bool eJ_recorded = false;
+  size_t eJ_bound = kEnergyJBytes;
   double* E64 = nullptr;
   double* bestE = nullptr;
   int* bestR = nullptr;
@@ -168,15 +172,35 @@ void dfree(T*& p) {
   p = nullptr;
 }
 
+// Gives up the kept digits of J.
+void drop_digits(gda_ctx* c) {
+  dfree(c->eJd);
+  c->eJ_blocks = 0;
+  c->eJ_ready = false;
+}
+
+// Memory a call cannot do without: the kept digits of J make room for it.
+template <typename T>
+cudaError_t alloc_required(gda_ctx* c, T** p, size_t n) {
+  cudaError_t e = dalloc(p, n);
+  if (e == cudaErrorMemoryAllocation && c->eJd && !c->eJ_recorded) {
+    cudaGetLastError();
+    drop_digits(c);
+    e = dalloc(p, n);
+  }
+  return e;
+}
+
 void free_state(gda_ctx* c) {
   for (int k = 0; k < 2; ++k) {
     dfree(c->psi[k]);
-    dfree(c->stg[k]);
     dfree(c->beta[k]);
     dfree(c->rho[k]);
   }
-  dfree(c->acc); dfree(c->S32); dfree(c->gam); dfree(c->gstg); dfree(c->gacc); dfree(c->epart);
-  dfree(c->ops); dfree(c->S64); dfree(c->eSd); dfree(c->part64); dfree(c->E64);
+  dfree(c->scratch);
+  c->stg[0] = c->stg[1] = c->acc = c->S32 = nullptr;
+  dfree(c->gam); dfree(c->gstg); dfree(c->gacc); dfree(c->epart);
+  dfree(c->ops); dfree(c->S64); dfree(c->part64); dfree(c->E64);
   if (c->plan) tc_plan_destroy(c->plan);
   c->plan = nullptr;
   dfree(c->ops8);
@@ -186,34 +210,18 @@ void free_state(gda_ctx* c) {
   c->have_state = false;
 }
 
-// A digit workspace of up to `want` blocks of `per` bytes, halving the request
-// while memory is short.
-gda_status alloc_digits(gda_ctx* c, unsigned char** p, int* blocks, size_t per, int want) {
-  while (!*p) {
-    const cudaError_t e = dalloc(p, size_t(want) * per);
-    if (e == cudaSuccess) {
-      *blocks = want;
-    } else if (e == cudaErrorMemoryAllocation && want > 1) {
-      cudaGetLastError();
-      want = (want + 1) / 2;
-    } else {
-      return cuda_fail(c, e, "energy workspace");
-    }
-  }
-  return GDA_OK;
-}
-
-// The digit workspaces of the final energies, with the state, so that energy
-// calls allocate nothing; short of memory they hold panels.
-gda_status reserve_digits(gda_ctx* c) {
-  const EnergyProb p = energy_prob(c->N, c->Np, c->Np, c->cplx ? c->Rcap_cols / 2 : c->Rcap_cols, c->Rcap_cols,
-                                   c->cplx, -1.0);
-  const size_t perJ = energy_J_bytes(p) / p.mtn, perS = energy_S_bytes(p) / p.ntn;
-  const gda_status s = alloc_digits(c, &c->eJd, &c->eJ_blocks, perJ,
-                                    int(std::min<size_t>(p.mtn, std::max<size_t>(1, kEnergyJBytes / perJ))));
-  if (s != GDA_OK) return s;
-  return alloc_digits(c, &c->eSd, &c->eS_blocks, perS,
-                      int(std::min<size_t>(p.ntn, std::max<size_t>(1, kEnergySBytes / perS))));
+// J's digits for the final energies, out of at most a quarter of the memory that
+// is free after the state: without them energy calls work in scratch.
+void reserve_digits(gda_ctx* c) {
+  size_t free_b = 0, total = 0;
+  if (c->eJd || cudaMemGetInfo(&free_b, &total) != cudaSuccess) return;
+  const EnergyProb p = energy_prob(c->N, c->Np, c->Np, 1, 1, c->cplx, -1.0);
+  const size_t perJ = energy_J_bytes(p) / p.mtn;
+  const int blocks = int(std::min<size_t>(p.mtn, std::min(c->eJ_bound, free_b / 4) / perJ));
+  if (dalloc(&c->eJd, size_t(blocks) * perJ) == cudaSuccess)
+    c->eJ_blocks = blocks;
+  else
+    cudaGetLastError();
 }
 
 // Allocates (or keeps) the state for R restarts; padding stays zero.
@@ -222,7 +230,7 @@ gda_status ensure_state(gda_ctx* c, int R) {
   if (c->Rcap_cols >= C && c->psi[0]) {
     c->R = R;
     c->C = C;
-    return reserve_digits(c);
+    return GDA_OK;
   }
   free_state(c);
   const size_t Cp = round_up(C, 256), Np = c->Np;
@@ -230,27 +238,29 @@ gda_status ensure_state(gda_ctx* c, int R) {
   const size_t MT = (c->N + 63) / 64;
   const size_t cn = Cp * Np, rn = Rp * Np;
   for (int k = 0; k < 2; ++k) {
-    CK(dalloc(&c->psi[k], cn));
-    CK(dalloc(&c->stg[k], cn));
-    CK(dalloc(&c->beta[k], Rp));
-    CK(dalloc(&c->rho[k], MT * Rp));
+    CK(alloc_required(c, &c->psi[k], cn));
+    CK(alloc_required(c, &c->beta[k], Rp));
+    CK(alloc_required(c, &c->rho[k], MT * Rp));
   }
-  CK(dalloc(&c->acc, cn));
-  CK(dalloc(&c->S32, cn));
-  CK(dalloc(&c->gam, rn));
-  CK(dalloc(&c->gstg, rn));
-  CK(dalloc(&c->gacc, rn));
-  CK(dalloc(&c->epart, MT * Rp));
-  if (c->cplx) CK(dalloc(&c->S64, cn));
-  CK(dalloc(&c->part64, MT * Rp));
-  CK(dalloc(&c->E64, Rp));
-  float* zf[] = {c->psi[0], c->psi[1], c->stg[0], c->stg[1], c->acc, c->S32};
-  for (float* p : zf) CK(cudaMemsetAsync(p, 0, cn * sizeof(float), c->stream));
+  CK(alloc_required(c, &c->scratch, 4 * cn));
+  c->stg[0] = c->scratch;
+  c->stg[1] = c->scratch + cn;
+  c->acc = c->scratch + 2 * cn;
+  c->S32 = c->scratch + 3 * cn;
+  CK(alloc_required(c, &c->gam, rn));
+  CK(alloc_required(c, &c->gstg, rn));
+  CK(alloc_required(c, &c->gacc, rn));
+  CK(alloc_required(c, &c->epart, MT * Rp));
+  if (c->cplx) CK(alloc_required(c, &c->S64, cn));
+  CK(alloc_required(c, &c->part64, MT * Rp));
+  CK(alloc_required(c, &c->E64, Rp));
+  for (float* p : c->psi) CK(cudaMemsetAsync(p, 0, cn * sizeof(float), c->stream));
+  CK(cudaMemsetAsync(c->scratch, 0, 4 * cn * sizeof(float), c->stream));
   CK(cudaMemsetAsync(c->gam, 0, rn * sizeof(float), c->stream));
   CK(cudaMemsetAsync(c->gstg, 0, rn * sizeof(float), c->stream));
   CK(cudaMemsetAsync(c->gacc, 0, rn * sizeof(float), c->stream));
   if (c->tc_ok) {
-    CK(dalloc(&c->ops, 3 * cn));
+    CK(alloc_required(c, &c->ops, 3 * cn));
     CK(cudaMemsetAsync(c->ops, 0, 3 * cn * sizeof(__nv_bfloat16), c->stream));
     CK(tc_plan_create(&c->plan, c->J16, int(Np), c->ops, 3, int(Cp)));
   }
@@ -260,7 +270,8 @@ gda_status ensure_state(gda_ctx* c, int R) {
   c->Rp = int(Rp);
   c->MT = int(MT);
   c->Rcap_cols = int(Cp);
-  return reserve_digits(c);
+  reserve_digits(c);
+  return GDA_OK;
 }
 
 // Uploads J (N x N, row-major) and g into the padded FP64 copies, checks the
@@ -296,8 +307,8 @@ gda_status load_instance(gda_ctx* c, const double* J, const double* g, cudaMemcp
 gda_status ensure_ell(gda_ctx* c) {
   const size_t Np = c->Np;
   if (!c->ell) {
-    CK(dalloc(&c->ell, size_t(GDA_SPARSE_MAX_DEG) * Np));
-    CK(dalloc(&c->d_maxdeg, 1));
+    CK(alloc_required(c, &c->ell, size_t(GDA_SPARSE_MAX_DEG) * Np));
+    CK(alloc_required(c, &c->d_maxdeg, 1));
   }
   if (c->ell_maxdeg < 0) {
     CK(cudaMemsetAsync(c->ell, 0, size_t(GDA_SPARSE_MAX_DEG) * Np * sizeof(int2), c->stream));
@@ -319,8 +330,8 @@ gda_status ensure_ell(gda_ctx* c) {
 gda_status ensure_fp8(gda_ctx* c) {
   const size_t Np = c->Np;
   if (!c->J8) {
-    CK(dalloc(&c->J8, Np * Np));
-    CK(dalloc(&c->jscale, Np));
+    CK(alloc_required(c, &c->J8, Np * Np));
+    CK(alloc_required(c, &c->jscale, Np));
   }
   if (!c->j8_ready) {
     LK(launch_prepare_J8(c->J32, int(Np), c->J8, c->jscale, c->stream));
@@ -328,7 +339,7 @@ gda_status ensure_fp8(gda_ctx* c) {
   }
   if (!c->ops8) {
     const size_t cn = size_t(c->Cp) * Np;
-    CK(dalloc(&c->ops8, 2 * cn));
+    CK(alloc_required(c, &c->ops8, 2 * cn));
     CK(cudaMemsetAsync(c->ops8, 0, 2 * cn, c->stream));
     CK(tc_plan8_create(&c->plan8, c->J8, int(Np), c->ops8, 2, c->Cp));
   }
@@ -456,7 +467,7 @@ gda_status run_gdmod(gda_ctx* c, const gda_params* p, int R, int64_t steps) {
     if (c->K_cap < need) {
       dfree(c->K);
       c->K_cap = 0;
-      CK(dalloc(&c->K, need));
+      CK(alloc_required(c, &c->K, need));
       c->K_cap = need;
     }
     LK(launch_gdmod_init(c->K, c->J32, float(p->beta0), c->N, c->Np, R, c->stream));
@@ -484,7 +495,9 @@ gda_status run_gdmod(gda_ctx* c, const gda_params* p, int R, int64_t steps) {
 }
 
 // FP64 Eq. (1) energies of R restarts (C columns) of psi into E64
-// (energy_tc.cu), in panels that fit the digit workspaces.
+// (energy_tc.cu).  The spins' digits take at most 14 of the 16 bytes an
+// amplitude has in scratch; where no digits of J are kept, panels of both share
+// it (a block of each needs 3584 of its >= 4096 Np bytes).
 gda_status energies_of(gda_ctx* c, const float* psi, int R, int C) {
   EnergyProb p = energy_prob(c->N, c->Np, c->Np, R, C, pmode(c), -1.0);
   p.J = c->J64;
@@ -495,14 +508,23 @@ gda_status energies_of(gda_ctx* c, const float* psi, int R, int C) {
   p.ldp = c->Rp;
   p.rexp = c->erexp;
   p.fmt = c->efmt;
+  const int MT = p.mtn, NT = p.ntn;
+  int mp = c->eJ_blocks, np = NT;
   p.Jd = c->eJd;
-  p.Sd = c->eSd;
-  const int MT = p.mtn, NT = p.ntn, mp = c->eJ_blocks, np = c->eS_blocks;
+  p.Sd = reinterpret_cast<unsigned char*>(c->scratch);
+  if (!c->eJd) {
+    const size_t perJ = energy_J_bytes(p) / MT, perS = energy_S_bytes(p) / NT;
+    const size_t room = size_t(4) * c->Cp * c->Np * sizeof(float);
+    if (NT * perS + perJ > room) np = int((room - perJ) / perS);
+    mp = int(std::min<size_t>(MT, (room - np * perS) / perJ));
+    p.Jd = p.Sd + np * perS;
+  }
   // work recorded into a graph runs later, maybe after another gda_load: it
   // makes the digits of the J it finds, in the form direct calls expect
   cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
   if (cudaStreamIsCapturing(c->stream, &cs) != cudaSuccess) cudaGetLastError();
   const bool recording = cs != cudaStreamCaptureStatusNone;
+  if (recording && c->eJd) c->eJ_recorded = true;
   for (int m = 0; m < MT; m += mp) {
     p.mt0 = m;
     p.mtn = std::min(mp, MT - m);
@@ -511,7 +533,7 @@ gda_status energies_of(gda_ctx* c, const float* psi, int R, int C) {
     u.n_row = p.mtn;
     if (!c->eJ_ready || recording) {
       LK(launch_energy_slice_J(p, u, c->stream));
-      if (!recording) c->eJ_ready = mp >= MT;
+      if (!recording) c->eJ_ready = c->eJd && mp >= MT;
     }
     for (int n = 0; n < NT; n += np) {
       p.nt0 = n;
@@ -707,6 +729,16 @@ gda_status gda_load_dev(gda_ctx* c, const double* J_dev, const double* g_dev) {
   return load_common(c, J_dev, g_dev, cudaMemcpyDeviceToDevice);
 }
 
+gda_status gda_set_energy_workspace(gda_ctx* c, int64_t bytes) {
+  if (!c) return GDA_ERR_INVALID;
+  if (bytes < 0) return fail(c, GDA_ERR_INVALID, "bytes must be >= 0");
+  if (c->eJ_recorded) return fail(c, GDA_ERR_STATE, "a recorded energy call uses the workspace");
+  c->eJ_bound = std::min(size_t(bytes), kEnergyJBytes);
+  drop_digits(c);
+  if (c->scratch) reserve_digits(c);
+  return GDA_OK;
+}
+
 gda_status gda_set_stream(gda_ctx* c, void* stream) {
   if (!c) return GDA_ERR_INVALID;
   c->stream = static_cast<cudaStream_t>(stream);
@@ -753,7 +785,7 @@ gda_status gda_run(gda_ctx* c, const gda_params* p, int32_t R, int64_t steps) {
     if (c->hist_bytes < n * row) {
       dfree(c->hist);
       c->hist_bytes = 0;
-      CK(dalloc(reinterpret_cast<unsigned char**>(&c->hist), n * row));
+      CK(alloc_required(c, reinterpret_cast<unsigned char**>(&c->hist), n * row));
       c->hist_bytes = n * row;
     }
     c->hist_run = int(n);
@@ -785,7 +817,7 @@ gda_status gda_run(gda_ctx* c, const gda_params* p, int32_t R, int64_t steps) {
     if (c->opT_cap < tn) {
       for (float*& t : c->opT) dfree(t);
       c->opT_cap = 0;
-      for (float*& t : c->opT) CK(dalloc(&t, tn));
+      for (float*& t : c->opT) CK(alloc_required(c, &t, tn));
       c->opT_cap = tn;
     }
     LK(launch_transpose_state(c->psi[c->cur], c->Np, c->Cp, c->opT[0], c->stream));
@@ -825,7 +857,7 @@ gda_status gda_run(gda_ctx* c, const gda_params* p, int32_t R, int64_t steps) {
     if (c->seg_flags_cap < nflags) {
       dfree(c->seg_flags);
       c->seg_flags_cap = 0;
-      CK(dalloc(&c->seg_flags, nflags));
+      CK(alloc_required(c, &c->seg_flags, nflags));
       c->seg_flags_cap = nflags;
     }
     const int64_t seg = p->energy_every > 0 ? p->energy_every : steps;
@@ -1167,7 +1199,7 @@ gda_status gda_profile(gda_ctx* c, int32_t enable) {
   }
   if (!c->stamps) {
     const int ctas = (c->Np / 64) * 4096;  // bound on the CTAs of any step launch
-    CK(dalloc(&c->stamps, size_t(ctas) * 8));
+    CK(alloc_required(c, &c->stamps, size_t(ctas) * 8));
     CK(cudaMemsetAsync(c->stamps, 0, size_t(ctas) * 8 * sizeof(unsigned long long), c->stream));
     c->stamp_cap = ctas;
   }
@@ -1189,7 +1221,7 @@ gda_status gda_set_init_base(gda_ctx* c, const float* base, int32_t on_device) {
   if (!c) return GDA_ERR_INVALID;
   if (!base) return fail(c, GDA_ERR_INVALID, "base is NULL");
   if (!c->base) {
-    CK(dalloc(&c->base, size_t(2) * c->N));
+    CK(alloc_required(c, &c->base, size_t(2) * c->N));
   }
   const size_t W = c->cplx ? 2 : 1;
   const cudaMemcpyKind kind = on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
@@ -1208,7 +1240,7 @@ gda_status gda_features(gda_ctx* c, float* F) {
   if (!c) return GDA_ERR_INVALID;
   if (!F) return fail(c, GDA_ERR_INVALID, "F is NULL");
   for (int k = 0; k < 2; ++k)
-    if (!c->fw[k]) CK(dalloc(&c->fw[k], size_t(c->Np)));
+    if (!c->fw[k]) CK(alloc_required(c, &c->fw[k], size_t(c->Np)));
   LK(launch_features(c->J64, c->g64, c->N, c->Np, c->cplx, c->fw[0], c->fw[1], F, c->stream));
   return GDA_OK;
 }

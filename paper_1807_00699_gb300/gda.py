@@ -45,6 +45,7 @@ SIGNATURES = {
     "gda_create": (ct.c_int, [_D, _D, ct.c_int32, ct.c_int32, ct.POINTER(_VP)]),
     "gda_load": (ct.c_int, [_VP, _D, _D]),
     "gda_load_dev": (ct.c_int, [_VP, _VP, _VP]),
+    "gda_set_energy_workspace": (ct.c_int, [_VP, ct.c_int64]),
     "gda_set_stream": (ct.c_int, [_VP, _VP]),
     "gda_run": (ct.c_int, [_VP, ct.POINTER(Params), ct.c_int32, ct.c_int64]),
     "gda_sync": (ct.c_int, [_VP]),
@@ -177,6 +178,10 @@ class Solver:
         """stream: a torch.cuda.Stream, a raw cudaStream_t integer, or None."""
         handle = getattr(stream, "cuda_stream", stream)
         self._check(self._lib.gda_set_stream(self._h, _VP(handle or 0)))
+
+    def set_energy_workspace(self, bytes: int):
+        """Bound on the memory kept for the energies' form of J (gda_set_energy_workspace)."""
+        self._check(self._lib.gda_set_energy_workspace(self._h, int(bytes)))
 
     def load(self, J: np.ndarray, g: np.ndarray | None = None):
         J = np.ascontiguousarray(J, dtype=np.float64)
