@@ -487,6 +487,13 @@ int32_t gda_batch_launch_mode(const gda_batch* b);
  * reports device errors of earlier runs. */
 gda_status gda_batch_best(gda_batch* b, double* E, int32_t* r);
 
+/* Bound, in bytes, on the device memory of the energies' workspace (allocated
+ * with the batch; default and most: 2.5 GiB, and never more than a quarter of
+ * what is free then, unless a single 128 x 128 block of an energy needs more).
+ * A smaller one costs time, not accuracy: instances are evaluated in pieces.
+ * GDA_ERR_INVALID for bytes < 0. */
+gda_status gda_batch_set_energy_workspace(gda_batch* b, int64_t bytes);
+
 /* State of instance k in the gda_get_state layout (host).  Synchronises. */
 gda_status gda_batch_get_state(gda_batch* b, int32_t k, float* psi, float* gamma, float* beta);
 const char* gda_batch_last_error(const gda_batch* b);

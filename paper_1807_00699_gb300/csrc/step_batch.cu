@@ -503,7 +503,7 @@ struct BatchPlan {
   int n_units = 0;
 };
 
-// Panels [prob0, ...) of one group: offsets of its unit lists in eunits.
+// One group of panels: its unit lists in eunits.
 struct EnergyGroup {
   int row0 = 0, n_row = 0, col0 = 0, n_col = 0, tile0 = 0, n_tile = 0, KBmax = 0;
 };
@@ -711,17 +711,19 @@ gda_status upload_settings(gda_batch* b, const gda_params* p) {
   return GDA_OK;
 }
 
-// Plans the final energies on first use: every instance is cut into panels
-// (row blocks x column blocks) whose digits fit the workspace bounds, and
-// panels are grouped while the digits and spins of a group fit together
-// (in `bound` bytes, unless one row block against one column block needs more).
+// Plans the final energies: every instance is cut into panels (row blocks x
+// column blocks) whose digits fit the workspace bounds, and panels are grouped
+// while the digits and spins of a group fit together (in `bound` bytes, unless
+// one row block against one column block needs more).
 gda_status plan_energies(gda_batch* b, size_t bound) {
-  void* stale[] = {b->erexp, b->eunits, b->eprobs};  // of an attempt that failed
+  void* stale[] = {b->erexp, b->eunits, b->eprobs, b->edigits};  // of another bound
   for (void* p : stale)
     if (p) cudaFree(p);
   b->erexp = nullptr;
   b->eunits = nullptr;
   b->eprobs = nullptr;
+  b->edigits = nullptr;
+  b->eJ_ready = false;
   auto align = [](size_t x) { return (x + 1023) / 1024 * 1024; };
   struct Place {
     int inst;
@@ -828,15 +830,20 @@ gda_status plan_energies(gda_batch* b, size_t bound) {
   return GDA_OK;
 }
 
+// The plan in at most `bytes`, a quarter of them while memory is short.
+gda_status reserve_energies(gda_batch* b, size_t bytes) {
+  size_t free_b = 0, total = 0;
+  BCK(cudaMemGetInfo(&free_b, &total));
+  for (size_t bound = std::min({bytes, kEnergyJBytes + kEnergySBytes, free_b / 4});; bound /= 4) {
+    const gda_status s = plan_energies(b, bound);
+    if (s != GDA_ERR_OOM || bound == 0) return s;
+  }
+}
+
 // FP64 Eq. (1) energies of every restart: partial sums per 128-row block in part.
 gda_status batch_energies(gda_batch* b) {
-  size_t bound = kEnergyJBytes + kEnergySBytes;
-  while (!b->edigits) {
-    const gda_status s = plan_energies(b, bound);
-    if (s == GDA_ERR_OOM && bound > (size_t(64) << 20)) {
-      bound /= 4;
-      continue;
-    }
+  if (!b->edigits) {  // gda_batch_set_energy_workspace found no room
+    const gda_status s = reserve_energies(b, 0);
     if (s != GDA_OK) return s;
   }
   for (const EnergyGroup& g : b->egroups) {
@@ -1017,6 +1024,9 @@ gda_status gda_batch_create(int32_t n, const int32_t* N, const int32_t* model, c
         if (s != GDA_OK) return s;
       }
     BCK(set_batch_attrs());
+    // with the batch: a batch that could be created and run can be judged
+    const gda_status es = reserve_energies(b, SIZE_MAX);
+    if (es != GDA_OK) return es;
     BCK(cudaDeviceSynchronize());
     return GDA_OK;
   }();
@@ -1195,6 +1205,12 @@ gda_status gda_batch_best(gda_batch* b, double* E, int32_t* r) {
     return bfail(b, (e & E_TIMEOUT) ? GDA_ERR_TIMEOUT : GDA_ERR_DIVERGED, "device error during the batched run");
   }
   return GDA_OK;
+}
+
+gda_status gda_batch_set_energy_workspace(gda_batch* b, int64_t bytes) {
+  if (!b) return GDA_ERR_INVALID;
+  if (bytes < 0) return bfail(b, GDA_ERR_INVALID, "bytes must be >= 0");
+  return reserve_energies(b, size_t(bytes));
 }
 
 gda_status gda_batch_get_state(gda_batch* b, int32_t k, float* psi, float* gamma, float* beta) {

@@ -80,6 +80,7 @@ SIGNATURES = {
     "gda_batch_set_init_base": (ct.c_int, [_VP, ct.c_int32, _VP, ct.c_int32]),
     "gda_batch_launch_mode": (ct.c_int32, [_VP]),
     "gda_batch_best": (ct.c_int, [_VP, _D, ct.POINTER(ct.c_int32)]),
+    "gda_batch_set_energy_workspace": (ct.c_int, [_VP, ct.c_int64]),
     "gda_batch_get_state": (ct.c_int, [_VP, ct.c_int32, _F, _F, _F]),
     "gda_batch_last_error": (ct.c_char_p, [_VP]),
     "gda_batch_destroy": (None, [_VP]),
@@ -395,6 +396,10 @@ class Batch:
     def launch_mode(self) -> int:
         """1: chunks replay a captured CUDA graph; 0: direct launches."""
         return int(self._lib.gda_batch_launch_mode(self._h))
+
+    def set_energy_workspace(self, bytes: int):
+        """Bound on the memory of the energies' workspace (gda_batch_set_energy_workspace)."""
+        self._check(self._lib.gda_batch_set_energy_workspace(self._h, int(bytes)))
 
     def best(self):
         E = np.empty(self.n, dtype=np.float64)

@@ -105,3 +105,30 @@ def test_recorded_energies_in_scratch(gda):
     with pytest.raises(gda.GdaError):
         s.set_energy_workspace(-1)
     s.close()
+
+
+def test_batch_groups_give_the_same_bits(gda):
+    # instances in one group, in several, and cut into panels of rows and columns down to single blocks
+    inst = []
+    for k, (n, R, xy) in enumerate([(129, 40, True), (300, 300, False), (50, 130, True), (700, 70, True),
+                                    (257, 129, False)]):
+        J = (synth.ising_pm1 if k % 2 else synth.sk_gaussian)(n, n)[0]
+        inst.append((J / np.sqrt(n) if k % 2 == 0 else J, 0.1 * synth.normal(k, n), gda.XY if xy else gda.ISING, R))
+    b = gda.Batch(inst, seed=3)
+    p = dict(dt=0.002, init_amp=0.1, prec=gda.BF16)
+    b.run(gda.default_params(**p), 20)
+    for bytes in (0, 1 << 20, 3 << 20, 8 << 20, 1 << 40):
+        ref = [b.best() for _ in range(2)]
+        b.set_energy_workspace(bytes)
+        for E, r in [b.best(), b.best(), *ref]:
+            assert np.array_equal(E, ref[0][0]) and np.array_equal(r, ref[0][1])
+        b.run(gda.default_params(**p, init_mode=2), 10)
+    for k, (J, g, model, R) in enumerate(inst):
+        s = gda.Solver(J, g, model)
+        s.set_state(b.get_state(k)[0])
+        E = s.energy()
+        assert b.best()[0][k] == E.min() and b.best()[1][k] == np.argmin(E)
+        s.close()
+    with pytest.raises(gda.GdaError):
+        b.set_energy_workspace(-1)
+    b.close()
