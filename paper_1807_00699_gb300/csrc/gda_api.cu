@@ -952,22 +952,27 @@ gda_status gda_run(gda_ctx* c, const gda_params* p, int32_t R, int64_t steps) {
   if (seg_cols && seg_len > (c->run_sparse ? 1 : 10)) {
     for (int64_t k = 0; k < steps; k += seg_len) {
       const int64_t len = std::min<int64_t>(seg_len, steps - k);
+      // the state ends in the buffers where a launch per step leaves it (which
+      // may be those it starts in: a CTA reads its columns before it writes
+      // them), so that a recorded run of an even number of steps continues
+      // its own result
+      const int flip = int(len & 1), pflip = p->integ == GDA_RK4 ? 0 : flip;
       StepArgs a = base;
       a.mode = p->integ == GDA_RK4 ? M_RK4 : M_EULER;
       a.step = static_cast<unsigned int>(c->step + k);
       a.psi_n = c->psi[c->cur];
-      a.psi_out = c->psi[c->cur ^ 1];
+      a.psi_out = c->psi[c->cur ^ pflip];
       a.beta_in = c->beta[c->bcur];
-      a.beta_out = c->beta[c->bcur ^ 1];
+      a.beta_out = c->beta[c->bcur ^ flip];
       a.rho_in = c->rho[c->rcur];
-      a.rho_out = decay ? c->rho[c->rcur ^ 1] : nullptr;
+      a.rho_out = decay ? c->rho[c->rcur ^ flip] : nullptr;
       if (c->run_sparse)
         LK(launch_sparse_seg(a, c->ell, c->ell_maxdeg, int(len), seg_cols, c->stream));
       else
         LK(launch_dense_seg(a, c->J32, p->integ == GDA_RK4, int(len), seg_cols, c->stream));
-      c->cur ^= 1;
-      c->bcur ^= 1;
-      if (decay) c->rcur ^= 1;
+      c->cur ^= pflip;
+      c->bcur ^= flip;
+      if (decay) c->rcur ^= flip;
       if (p->energy_every > 0 && len == seg_len) {
         s = track(c, p, tc, c->step + k + len);
         if (s != GDA_OK) return s;

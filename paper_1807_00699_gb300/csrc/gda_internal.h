@@ -93,7 +93,8 @@ double ptx_cycles_per_second();
 // Launchers (return cudaGetLastError() of the launch).
 cudaError_t launch_step_dense(const StepArgs& a, const float* J32, const float* operand, int sms, cudaStream_t s);
 // A segment of Euler or RK4 steps of a small dense instance in one launch
-// (psi_n -> psi_out, beta_in -> beta_out, rho_in -> rho_out, gam in place);
+// (psi_n -> psi_out, beta_in -> beta_out, rho_in -> rho_out, which may be the
+// same buffers, gam in place);
 // columns per CTA from dense_seg_columns (0: a launch per step is better).
 int dense_seg_columns(const StepArgs& a, int sms);
 cudaError_t launch_dense_seg(const StepArgs& a, const float* J32, bool rk4, int steps, int columns, cudaStream_t s);
@@ -104,7 +105,7 @@ int simt_mtiles(int N);
 cudaError_t launch_step_sparse(const StepArgs& a, const int2* cv, const float* operand, int maxdeg, cudaStream_t s);
 cudaError_t launch_prepare_ell(const float* J32, int N, int Np, int dmax, int2* cv, int* maxdeg, cudaStream_t s);
 // A segment of forward-Euler steps in one launch (psi_n -> psi_out, beta_in ->
-// beta_out, rho_in -> rho_out, gam in place); columns per CTA from
+// beta_out, rho_in -> rho_out, which may be the same buffers, gam in place); columns per CTA from
 // sparse_seg_columns (0: not applicable).
 int sparse_seg_columns(const StepArgs& a, int sms);
 cudaError_t launch_sparse_seg(const StepArgs& a, const int2* cv, int maxdeg, int steps, int columns, cudaStream_t s);
