@@ -113,7 +113,7 @@ typedef struct {
   int32_t init_mode;    /* 0: psi = 0; 1: seeded U(-a, a) per real component;
                            2: continue from the current state (resume);
                            3: as 1 plus the per-spin base of gda_set_init_base */
-  int32_t schedule;     /* gda_schedule: how BF16 steps are launched           */
+  int32_t schedule;     /* gda_schedule: how steps are launched                */
   double init_amp;      /* a for init_mode 1                                   */
   int32_t coupling;     /* gda_coupling_mode: GD (K = beta J) or GD-mod        */
   int32_t withhold_flag; /* testing only, 0 otherwise: k >= 1 makes the last
@@ -154,13 +154,16 @@ typedef struct {
  *   gda_get_state does not return it. */
 typedef enum { GDA_COUPLING_GD = 0, GDA_COUPLING_GDMOD = 1 } gda_coupling_mode;
 
-/* Launch schedule of the tensor-core path.  AUTO picks the resident kernel
+/* Launch schedule.  PER_STEP launches every step (RK4 stage) by itself, in any
+ * precision.  For the tensor-core path AUTO picks the resident kernel
  * for Euler runs whose 128 x 128 tiles all fit on the device at once (every
  * CTA keeps its tile's FP32 state in tensor memory for a whole segment of
  * steps, with per-tile flags between steps); else, for Euler runs whose
  * coupling operand (N'^2 BF16 or E4M3 values) fits in 48 MiB, the persistent
  * streaming launch (GDA_SCHEDULE_STREAM); else one launch per step (RK4
- * stage), with two-SM tiles where they pay.  All give the same numbers. */
+ * stage), with two-SM tiles where they pay.  For GDA_SPARSE Euler runs and
+ * GDA_FP32 runs of small N it launches a tracking segment at a time where the
+ * state fits in shared memory, else a step.  All give the same numbers. */
 typedef enum {
   GDA_SCHEDULE_AUTO = 0,
   GDA_SCHEDULE_PER_STEP = 1,

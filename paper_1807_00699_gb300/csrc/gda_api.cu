@@ -373,7 +373,7 @@ gda_status check_params(gda_ctx* c, const gda_params* p) {
     return fail(c, GDA_ERR_UNSUPPORTED, "tensor-core path needs an sm_103 device");
   const bool res_sched = p->schedule == GDA_SCHEDULE_RESIDENT || p->schedule == GDA_SCHEDULE_RESIDENT_PAIR;
   if (p->prec == GDA_SPARSE && res_sched)
-    return fail(c, GDA_ERR_UNSUPPORTED, "the sparse product runs per step");
+    return fail(c, GDA_ERR_UNSUPPORTED, "the sparse product has no resident schedule");
   if ((p->schedule == GDA_SCHEDULE_PAIR || p->schedule == GDA_SCHEDULE_STREAM_PAIR) &&
       (!(p->prec == GDA_BF16 || p->prec == GDA_FP8) || (c->Np / 128) % 2 != 0 || p->coupling != GDA_COUPLING_GD))
     return fail(c, GDA_ERR_UNSUPPORTED, "two-SM tiles need BF16 or FP8 and an even number of 128-row blocks");
@@ -938,7 +938,8 @@ gda_status gda_run(gda_ctx* c, const gda_params* p, int32_t R, int64_t steps) {
   }
 
   // FP32 runs whose columns fit on chip (sparse Euler, small dense Euler and
-  // RK4): one launch per tracking segment, columns never meet.  A sparse
+  // RK4): one launch per tracking segment, columns never meet, unless a launch
+  // per step is asked for.  A sparse
   // segment of one step gains nothing over the per-step kernel; dense segments
   // of up to 10 steps keep a launch per step, the count gda_kernel_launches
   // has always reported for such runs.
@@ -949,7 +950,7 @@ gda_status gda_run(gda_ctx* c, const gda_params* p, int32_t R, int64_t steps) {
   else if (!tc)
     seg_cols = dense_seg_columns(base, c->sms);
   const int64_t seg_len = p->energy_every > 0 ? p->energy_every : std::min<int64_t>(steps, 1 << 16);
-  if (seg_cols && seg_len > (c->run_sparse ? 1 : 10)) {
+  if (p->schedule == GDA_SCHEDULE_AUTO && seg_cols && seg_len > (c->run_sparse ? 1 : 10)) {
     for (int64_t k = 0; k < steps; k += seg_len) {
       const int64_t len = std::min<int64_t>(seg_len, steps - k);
       // the state ends in the buffers where a launch per step leaves it (which
