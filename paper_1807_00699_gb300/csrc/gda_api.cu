@@ -939,10 +939,16 @@ gda_status gda_run(gda_ctx* c, const gda_params* p, int32_t R, int64_t steps) {
 
   // FP32 runs whose columns fit on chip (sparse Euler, small dense Euler and
   // RK4): one launch per tracking segment, columns never meet, unless a launch
-  // per step is asked for.  A sparse
-  // segment of one step gains nothing over the per-step kernel; dense segments
-  // of up to 10 steps keep a launch per step, the count gda_kernel_launches
-  // has always reported for such runs.
+  // per step is asked for.  A sparse segment of one step gains nothing over the
+  // per-step kernel.  A dense segment first loads J0 into every CTA, which a few
+  // stages pay back, more for larger N.  Measured (GB300, us a step with
+  // tracking, segment / launch per stage): Ising N = 20, R = 64, Euler, every 2
+  // steps 13.9 / 15.9, every 10 3.2 / 7.3; N = 200, R = 256, Euler, every 2 24.1 /
+  // 20.0, every 3 16.8 / 16.1, every 5 11.7 / 12.9, every 10 7.5 / 10.6; XY N =
+  // 200, R = 64, RK4, every 2 33.3 / 45.6.  Dense runs of up to 10 launches in all
+  // keep them: gda_kernel_launches has always counted every step there, which
+  // the tests hold it to (a segment would save about 40 of 58 us on 10 steps at
+  // N = 20).
   base.rho_out = decay ? c->rho[c->rcur ^ 1] : nullptr;
   int seg_cols = 0;
   if (!tc && c->run_sparse)
@@ -950,7 +956,10 @@ gda_status gda_run(gda_ctx* c, const gda_params* p, int32_t R, int64_t steps) {
   else if (!tc)
     seg_cols = dense_seg_columns(base, c->sms);
   const int64_t seg_len = p->energy_every > 0 ? p->energy_every : std::min<int64_t>(steps, 1 << 16);
-  if (p->schedule == GDA_SCHEDULE_AUTO && seg_cols && seg_len > (c->run_sparse ? 1 : 10)) {
+  const int stages = p->integ == GDA_RK4 ? 4 : 1;
+  const bool seg_pays = c->run_sparse ? seg_len > 1
+                                      : seg_len > std::max(1, (1 + c->N / 64) / stages) && steps > 10 / stages;
+  if (p->schedule == GDA_SCHEDULE_AUTO && seg_cols && seg_pays) {
     for (int64_t k = 0; k < steps; k += seg_len) {
       const int64_t len = std::min<int64_t>(seg_len, steps - k);
       // the state ends in the buffers where a launch per step leaves it (which

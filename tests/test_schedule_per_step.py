@@ -19,7 +19,7 @@ def gda():
     return mod
 
 
-@pytest.mark.parametrize("every", [0])
+@pytest.mark.parametrize("every", [0, 7])
 @pytest.mark.parametrize("model,n,prec,integ", [("ising", 20, "FP32", "EULER"), ("xy", 130, "FP32", "RK4"),
                                                 ("ising", 800, "SPARSE", "EULER"), ("xy", 130, "SPARSE", "EULER")])
 def test_per_step_is_honoured(gda, model, n, prec, integ, every):
