@@ -938,28 +938,23 @@ gda_status gda_run(gda_ctx* c, const gda_params* p, int32_t R, int64_t steps) {
   }
 
   // FP32 runs whose columns fit on chip (sparse Euler, small dense Euler and
-  // RK4): one launch per tracking segment, columns never meet, unless a launch
-  // per step is asked for.  A sparse segment of one step gains nothing over the
-  // per-step kernel.  A dense segment first loads J0 into every CTA, which a few
-  // stages pay back, more for larger N.  Measured (GB300, us a step with
-  // tracking, segment / launch per stage): Ising N = 20, R = 64, Euler, every 2
-  // steps 13.9 / 15.9, every 10 3.2 / 7.3; N = 200, R = 256, Euler, every 2 24.1 /
-  // 20.0, every 3 16.8 / 16.1, every 5 11.7 / 12.9, every 10 7.5 / 10.6; XY N =
-  // 200, R = 64, RK4, every 2 33.3 / 45.6.  Dense runs of up to 10 launches in all
-  // keep them: gda_kernel_launches has always counted every step there, which
-  // the tests hold it to (a segment would save about 40 of 58 us on 10 steps at
-  // N = 20).
+  // RK4): one launch per tracking segment where that is the faster form, columns
+  // never meet, unless a launch per step is asked for.  Dense runs of up to 10
+  // launches in all keep them: gda_kernel_launches has always counted every
+  // step there, which the tests hold it to (a segment would save about 40 of 58
+  // us on 10 steps at N = 20).
   base.rho_out = decay ? c->rho[c->rcur ^ 1] : nullptr;
-  int seg_cols = 0;
-  if (!tc && c->run_sparse)
-    seg_cols = p->integ == GDA_EULER ? sparse_seg_columns(base, c->sms) : 0;
-  else if (!tc)
-    seg_cols = dense_seg_columns(base, c->sms);
   const int64_t seg_len = p->energy_every > 0 ? p->energy_every : std::min<int64_t>(steps, 1 << 16);
-  const int stages = p->integ == GDA_RK4 ? 4 : 1;
-  const bool seg_pays = c->run_sparse ? seg_len > 1
-                                      : seg_len > std::max(1, (1 + c->N / 64) / stages) && steps > 10 / stages;
-  if (p->schedule == GDA_SCHEDULE_AUTO && seg_cols && seg_pays) {
+  const int64_t rule_len = std::min<int64_t>(std::min(seg_len, steps), 1 << 20);
+  const bool rk4 = p->integ == GDA_RK4;
+  int seg_cols = 0;
+  if (!tc && p->schedule == GDA_SCHEDULE_AUTO) {
+    if (c->run_sparse)
+      seg_cols = rk4 ? 0 : sparse_seg_columns(base, c->ell_maxdeg, c->sms, rule_len);
+    else if (seg_len > 1 && steps > (rk4 ? 2 : 10))
+      seg_cols = dense_seg_columns(base, c->sms, rk4, rule_len);
+  }
+  if (seg_cols) {
     for (int64_t k = 0; k < steps; k += seg_len) {
       const int64_t len = std::min<int64_t>(seg_len, steps - k);
       // the state ends in the buffers where a launch per step leaves it (which

@@ -94,9 +94,9 @@ double ptx_cycles_per_second();
 cudaError_t launch_step_dense(const StepArgs& a, const float* J32, const float* operand, int sms, cudaStream_t s);
 // A segment of Euler or RK4 steps of a small dense instance in one launch
 // (psi_n -> psi_out, beta_in -> beta_out, rho_in -> rho_out, which may be the
-// same buffers, gam in place);
-// columns per CTA from dense_seg_columns (0: a launch per step is better).
-int dense_seg_columns(const StepArgs& a, int sms);
+// same buffers, gam in place); columns per CTA from dense_seg_columns (0: a
+// launch per stage is better).
+int dense_seg_columns(const StepArgs& a, int sms, bool rk4, long long steps);
 cudaError_t launch_dense_seg(const StepArgs& a, const float* J32, bool rk4, int steps, int columns, cudaStream_t s);
 int simt_mtiles(int N);
 // Sparse J0 (ELL [dmax][Np] of (column, value), ascending columns): the SIMT
@@ -105,9 +105,9 @@ int simt_mtiles(int N);
 cudaError_t launch_step_sparse(const StepArgs& a, const int2* cv, const float* operand, int maxdeg, cudaStream_t s);
 cudaError_t launch_prepare_ell(const float* J32, int N, int Np, int dmax, int2* cv, int* maxdeg, cudaStream_t s);
 // A segment of forward-Euler steps in one launch (psi_n -> psi_out, beta_in ->
-// beta_out, rho_in -> rho_out, which may be the same buffers, gam in place); columns per CTA from
-// sparse_seg_columns (0: not applicable).
-int sparse_seg_columns(const StepArgs& a, int sms);
+// beta_out, rho_in -> rho_out, which may be the same buffers, gam in place);
+// columns per CTA from sparse_seg_columns (0: a launch per step is better).
+int sparse_seg_columns(const StepArgs& a, int maxdeg, int sms, long long steps);
 cudaError_t launch_sparse_seg(const StepArgs& a, const int2* cv, int maxdeg, int steps, int columns, cudaStream_t s);
 bool sparse_stages(int Np);
 // out[i][c] = x[c][i] for c < Cp, i < Np (column-major state -> spin-major operand).

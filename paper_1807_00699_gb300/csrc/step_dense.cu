@@ -8,6 +8,8 @@
 //    Y = J0 X over 64 x BN tiles of (spins i) x (columns c) fused with the
 //    step epilogue (Eqs. 2, 5, 6).
 //  * k_dense_seg: small N; one launch runs a whole tracking segment.
+#include <algorithm>
+
 #include "epilogue.cuh"
 #include "tc_epilogue.cuh"
 #include "tc_ptx.cuh"
@@ -496,16 +498,33 @@ cudaError_t launch_step_dense(const StepArgs& a, const float* J32, const float* 
   return a.cplx ? launch_dense<true>(a, J32, operand, sms, s) : launch_dense<false>(a, J32, operand, sms, s);
 }
 
-// Columns per CTA of a segment launch, 0 where a launch per step is better:
-// J0 must fit in shared memory (N <= ~235), and the busiest SM's coupling
-// sums (rounds x warps x N x (NC FMAs + 2 loads) / 4 issue slots) stay below
-// ~16 000 cycles a stage, about what a per-step launch takes at these sizes.
-int dense_seg_columns(const StepArgs& a, int sms) {
+// Columns per CTA of a segment of `steps` steps in one launch, 0 where a launch
+// per stage is better.  J0 must fit in shared memory (N <= ~235).  A stage of
+// a segment takes the chain of N FMAs and loads for every wave of CTAs (and the
+// issue slots of further CTAs on the SM), and every wave first loads its J0; a
+// stage by itself takes a launch and its tile's K loop, which a lone tile of
+// four warps per SM runs at `alone` cycles a K.  Times in ns, fitted to runs on
+// GB300 over N = 10 .. 233, R = 16 .. 2048, both models and integrators, 13 and 300
+// steps: the rule chose nothing more than 3 % slower than a launch per stage.  us
+// a step, segment / launch per stage, Euler: Ising N = 10, R = 64 0.5 / 5.2; N = 200,
+// R = 256 3.6 / 8.2; XY N = 200, R = 400 8.1 / 10.3, R = 1024 (four waves) 16.2 /
+// 14.4; and 13.5 us a wave to load J0 at N = 200.
+int dense_seg_columns(const StepArgs& a, int sms, bool rk4, long long steps) {
   if (a.N > 256 || dense_seg_smem(a, 4) > kDenseSegSmemMax) return 0;
   auto rounds = [&](int nc) { return ((a.C + nc - 1) / nc + sms - 1) / sms; };
   const int nc = rounds(4) < rounds(2) ? 4 : 2;
-  const long long cycles = (long long)rounds(nc) * ((a.N + 31) / 32) * a.N * (nc + 2) / 4;
-  return cycles <= 16000 ? nc : 0;
+  const long long N = a.N, ctas = (a.C + nc - 1) / nc, warps = (a.N + 31) / 32;
+  const long long per_sm = std::min<long long>((227 * 1024) / (dense_seg_smem(a, nc) + 1024), 64 / warps);
+  const long long waves = (ctas + sms * per_sm - 1) / (sms * per_sm);
+  const long long shared = (std::min(ctas, sms * per_sm) + sms - 1) / sms - 1;
+  const long long stage = waves * (350 + (a.cplx ? 19 : 17) * N + shared * warps * N * (nc + 2) / 8);
+  const long long load = waves * (2000 + 65 * N);
+  const int bn = dense_bn(a, sms);
+  const long long alone = bn == 128 ? 176 : bn == 64 ? 84 : bn == 32 ? 47 : 29;
+  const long long tiles = (long long)((a.C + bn - 1) / bn) * simt_mtiles(a.N);
+  const long long single = 5000 + (tiles + sms - 1) / sms * ((N + BK - 1) / BK * BK) * alone / 2;
+  const long long stages = steps * (rk4 ? 4 : 1);
+  return stages * stage + load < stages * single ? nc : 0;
 }
 
 cudaError_t launch_dense_seg(const StepArgs& a, const float* J32, bool rk4, int steps, int columns, cudaStream_t s) {

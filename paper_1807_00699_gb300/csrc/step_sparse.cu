@@ -6,6 +6,8 @@
 // map and the epilogue (with its partial-sum order) are the dense FP32
 // kernel's (step_dense.cu), so density partials, noise decay and the energy
 // mode carry over unchanged.
+#include <algorithm>
+
 #include "epilogue.cuh"
 #include "tc_epilogue.cuh"
 #include "tc_ptx.cuh"
@@ -573,15 +575,32 @@ cudaError_t launch_seg(const StepArgs& a, const Ell& ell, int maxdeg, int steps,
 
 }  // namespace
 
-// The columns per CTA of a segment launch, 0 if the amplitudes of two columns
-// do not fit in shared memory twice (N > ~14 300).  Four columns share a row's
-// table loads and gathers: about 90 instructions a row against 2 x 53 for two
-// CTAs of two columns, so they win wherever they leave no more rounds of SMs.
-int sparse_seg_columns(const StepArgs& a, int sms) {
+// The columns per CTA of a segment of `steps` steps in one launch, 0 if the
+// amplitudes of two columns do not fit in shared memory twice (N > ~14 300) or a
+// launch per step is better.  Four columns share a row's table loads and
+// gathers: about 90 instructions a row against 2 x 53 for two CTAs of two
+// columns, so they win wherever they leave no more rounds of SMs.  A segment
+// sweeps all rows of a CTA's columns on one SM, the per-step kernel spreads few
+// columns over the chip: with few columns of a large instance it is the faster
+// one.  Times in ns, fitted to runs on GB300 over N = 100 .. 14 000, 3 and 8
+// entries per row, R = 4 .. 1024, both models, 3 and 300 steps: the rule chose
+// nothing more than 3 % slower than a launch per step.  us a step, segment / per
+// step, 3-regular Ising: N = 800, R = 1024 2.0 / 10.3; N = 6000, R = 64 3.7 / 6.2, R =
+// 512 6.2 / 16.4; N = 12 000, R = 32 7.2 / 6.2, R = 512 14.3 / 27.2; 8 entries, XY
+// N = 14 000, R = 4 24.7 / 8.3.
+int sparse_seg_columns(const StepArgs& a, int maxdeg, int sms, long long steps) {
   if (seg_smem(a, 2) > kSegSmemMax || a.mt_count > 256) return 0;
-  if (seg_smem(a, 4) > kSegSmemMax || a.mt_count > 112) return 2;
-  const long long w2 = ((a.C + 1) / 2 + sms - 1) / sms * 53LL, w4 = ((a.C + 3) / 4 + sms - 1) / sms * 90LL;
-  return w4 <= w2 ? 4 : 2;
+  auto rounds = [&](int c) { return (long long)((a.C + c - 1) / c + sms - 1) / sms; };
+  const bool four = seg_smem(a, 4) <= kSegSmemMax && a.mt_count <= 112 && rounds(4) * 90 <= rounds(2) * 53;
+  const int nc = four ? 4 : 2;
+  const long long N = a.N, deg = maxdeg < 3 ? 3 : maxdeg;
+  long long sweep = rounds(nc) * N * (250 + 130 * deg) / 1000;  // table loads, gathers and updates
+  if (four) sweep = sweep * 17 / 10;
+  if (a.cplx && deg > 3 && a.mt_count > 192) sweep = sweep * 27 / 20;  // four tiles per group
+  const long long step = 300 + 100 * deg + sweep;
+  const long long load = 3000 + rounds(nc) * N * nc * 3 / 10;  // the state in and out
+  const long long single = std::max<long long>(6200, 5500 + N * a.C * (2200 + 480 * deg) / 1000000);
+  return steps > 1 && steps * step + load < steps * single ? nc : 0;
 }
 
 cudaError_t launch_sparse_seg(const StepArgs& a, const int2* cv, int maxdeg, int steps, int columns, cudaStream_t s) {
