@@ -151,6 +151,48 @@ __global__ void k_track_reduce(const float* e_part, int mt, int R, int Rp, doubl
   }
 }
 
+// ---------------------------------------------------------------- final energy
+// Energies of real spins, g = 0 and a small instance of integer couplings whose
+// sums all stay below 2^24: exact in FP32.  One CTA per restart, a warp per
+// row of J.  A tile of the digit products costs a single small instance its
+// fixed 19 us (prologue, pipeline, tile-wide sums); this kernel takes 8 for N =
+// 100, R = 256 and reads N^2 doubles per restart from L2, so it is used up to
+// 2^25 of them.
+constexpr int ES_MAXN = 256, ES_WARPS = 16;
+
+// An integer of at most 24 bits from double to float by its bits (the
+// conversion instruction runs at the FP64 pipe's rate: 16 us instead of 8).
+__device__ __forceinline__ float small_float(double v) {
+  const unsigned hi = unsigned(__double2hiint(v)), lo = unsigned(__double2loint(v));
+  if (!(hi & 0x7fffffffu)) return 0.0f;
+  return __uint_as_float((hi & 0x80000000u) | (((hi & 0x7fffffffu) - (896u << 20)) << 3) | (lo >> 29));
+}
+
+__global__ void __launch_bounds__(32 * ES_WARPS) k_energy_small(const double* __restrict__ J,
+                                                                const float* __restrict__ psi, int N, int Np,
+                                                                double* __restrict__ E) {
+  __shared__ float s[ES_MAXN], part[ES_WARPS];
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  if (tid < ES_MAXN) s[tid] = tid >= N ? 0.0f : psi[size_t(blockIdx.x) * Np + tid] >= 0.0f ? 1.0f : -1.0f;
+  __syncthreads();
+  float t = 0.0f;
+#pragma unroll 2
+  for (int i = warp; i < N; i += ES_WARPS) {
+    float y = 0.0f;
+#pragma unroll
+    for (int k = 0; k < ES_MAXN / 32; ++k)
+      if (k * 32 + lane < N) y = fmaf(small_float(J[size_t(i) * Np + k * 32 + lane]), s[k * 32 + lane], y);
+    t = fmaf(s[i], y, t);
+  }
+  for (int o = 16; o; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+  if (lane == 0) part[warp] = t;
+  __syncthreads();
+  if (tid == 0) {
+    for (int w = 1; w < ES_WARPS; ++w) t += part[w];
+    E[blockIdx.x] = -double(t);
+  }
+}
+
 // Lowest energy over restarts (ties: lowest index) -> best[0] = E, best_r.
 __global__ void k_argmin(const double* E, int R, double* bestE, int* bestR) {
   __shared__ double sE[32];
@@ -292,6 +334,14 @@ cudaError_t launch_snapshot(const float* psi, int Np, int W, const double* lastE
 
 cudaError_t launch_snapshot_reset(double* snapE, int* snapR, long long* snapStep, cudaStream_t s) {
   k_snapshot_reset<<<1, 1, 0, s>>>(snapE, snapR, snapStep);
+  return cudaGetLastError();
+}
+
+bool energy_small_fits(int N, double jmax) { return N <= ES_MAXN && double(N) * N * jmax <= double(1 << 24); }
+
+cudaError_t launch_energy_small(const double* J64, const float* psi, int N, int Np, int R, double* E,
+                                cudaStream_t s) {
+  k_energy_small<<<R, 32 * ES_WARPS, 0, s>>>(J64, psi, N, Np, E);
   return cudaGetLastError();
 }
 

@@ -50,6 +50,9 @@ constexpr int EWARPS = 16;
 constexpr int ETHREADS = 64 + 32 * EWARPS;
 constexpr uint32_t TBYTES = uint32_t(kEnergyTileBytes);
 constexpr uint32_t ESMEM = 1024 + STAGES * 2 * TBYTES;
+// A complex spin is a square root and two divisions in FP64: one CTA takes 47 us
+// for the 64 x 64 spins of a block, four take 13 (XY N = 100, R = 64).
+constexpr int SPLIT = 4;
 constexpr int KCHUNK = 8;  // K blocks of 64 per accumulation of digit products up to 2^14
 
 // Unit k of a list (problem, row or column block, column block of a tile).
@@ -155,8 +158,8 @@ __global__ void __launch_bounds__(256) k_energy_slice_J(EnergyProb p0, const Ene
   }
 }
 
-// Projected spins of one column block and K block: digit tiles, and (complex
-// spins) s itself in double for the reduction.  A row of a tile is a column
+// Projected spins of one column block and K block, SPLIT CTAs to each: digit
+// tiles, and (complex spins) s itself in double for the reduction.  A row of a tile is a column
 // of the state; complex spins are handled as the pair of columns 2r, 2r + 1.
 __global__ void __launch_bounds__(256) k_energy_slice_S(EnergyProb p0, const EnergyProb* probs, const int4* units) {
   const int4 U = unit_of(units, blockIdx.x, p0.ntn);
@@ -167,7 +170,7 @@ __global__ void __launch_bounds__(256) k_energy_slice_S(EnergyProb p0, const Ene
   unsigned char* out = P.Sd + (size_t(U.y) * ns * P.KB + kb) * TBYTES;
   const size_t slice = size_t(P.KB) * TBYTES;
   if (!P.pmode) {
-    for (int q = threadIdx.x; q < TILE * 8; q += 256) {
+    for (int q = blockIdx.z * 256 + threadIdx.x; q < TILE * 8; q += SPLIT * 256) {
       const int cr = q >> 3, k8 = q & 7;
       const int c = (P.nt0 + U.y) * TILE + cr, i0 = kb * 64 + k8 * 8;
       uint32_t w[4] = {0u, 0u, 0u, 0u};
@@ -182,7 +185,7 @@ __global__ void __launch_bounds__(256) k_energy_slice_S(EnergyProb p0, const Ene
     return;
   }
   // complex: a thread takes 4 spins of a restart (half a 16-byte group of both of its rows)
-  for (int q = threadIdx.x; q < (TILE / 2) * 16; q += 256) {
+  for (int q = blockIdx.z * 256 + threadIdx.x; q < (TILE / 2) * 16; q += SPLIT * 256) {
     const int rr = q >> 4, k4 = q & 15;
     const int c = (P.nt0 + U.y) * TILE + 2 * rr, i0 = kb * 64 + k4 * 4;
     unsigned short d[2][4][kEnergySlices] = {};
@@ -265,7 +268,7 @@ __global__ void __launch_bounds__(ETHREADS, 1) k_energy_product(const __grid_con
   auto acc_full = [&](int b) { return smem_u32(bars + 2 * STAGES + b); };
   auto acc_empty = [&](int b) { return smem_u32(bars + 2 * STAGES + 2 + b); };
   auto aborted = [&]() { return *(volatile int*)&s_abort != 0; };
-  const int ns0 = probs ? 0 : format_of(p0).x;  // problems of a list carry their own
+  const int2 f0 = probs ? make_int2(0, 0) : format_of(p0);  // problems of a list carry their own
   if (threadIdx.x == 0) {
     for (int s = 0; s < STAGES; ++s) {
       mbar_init(full_bar(s), 1);
@@ -291,7 +294,7 @@ __global__ void __launch_bounds__(ETHREADS, 1) k_energy_product(const __grid_con
       for (int t = blockIdx.x; t < n_tile && !stop; t += gridDim.x) {
         const int4 U = unit_of(units, t, p0.mtn);
         const EnergyProb& P = probs ? probs[U.x] : p0;
-        const int nsJ = probs ? P.nsJ : ns0;
+        const int nsJ = probs ? P.nsJ : f0.x;
         for (PairIter q(nsJ, P.nsS); !q.done() && !stop; q.next()) {
           const unsigned char* A = P.Jd + (size_t(U.y) * nsJ + q.i) * P.KB * TBYTES;
           const unsigned char* B = P.Sd + (size_t(U.z) * P.nsS + q.j) * P.KB * TBYTES;
@@ -323,7 +326,7 @@ __global__ void __launch_bounds__(ETHREADS, 1) k_energy_product(const __grid_con
       for (int t = blockIdx.x; t < n_tile && !stop; t += gridDim.x) {
         const int4 U = unit_of(units, t, p0.mtn);
         const EnergyProb& P = probs ? probs[U.x] : p0;
-        const int nsJ = probs ? P.nsJ : ns0;
+        const int nsJ = probs ? P.nsJ : f0.x;
         const int ck = chunk_kb(P);
         for (PairIter q(nsJ, P.nsS); !q.done() && !stop; q.next()) {
           for (int k0 = 0; k0 < P.KB && !stop; k0 += ck, ++use) {
@@ -365,7 +368,7 @@ __global__ void __launch_bounds__(ETHREADS, 1) k_energy_product(const __grid_con
     for (int t = blockIdx.x; t < n_tile; t += gridDim.x) {
       const int4 U = unit_of(units, t, p0.mtn);
       const EnergyProb& P = probs ? probs[U.x] : p0;
-      const int nsJ = probs ? P.nsJ : ns0;
+      const int nsJ = probs ? P.nsJ : f0.x;
       const int ck = chunk_kb(P);
       const int i = (P.mt0 + U.y) * TILE + 32 * q4 + lane;
       const int2 re = i < P.N ? P.rexp[i] : make_int2(0, -(1 << 20));
@@ -430,6 +433,42 @@ __global__ void __launch_bounds__(ETHREADS, 1) k_energy_product(const __grid_con
         v[0] += __shfl_xor_sync(0xffffffffu, v[0], 1);
         if (!(lane & 1))  // lane bits 4..1 are the restart's bits 3..0
           s_red[q4][cpart * 16 + (lane >> 1)] = v[0];
+      } else if (probs ? P.jint : f0.y) {
+        // integers: acc is (J s)_i itself (unit 0); 32 rows of them stay below
+        // 2^52, summed as integers (in FP64, at a 64th of the rate, a tile's
+        // sums took 30 of the kernel's 49 us at N = 100, R = 256)
+        unsigned neg = 0;  // columns of spin -1
+#pragma unroll 4
+        for (int u = 0; u < 32; ++u)
+          if (row && c0 + u < P.C && !(P.psi[size_t(c0 + u) * P.Np + i] >= 0.0f)) neg |= 1u << u;
+#pragma unroll
+        for (int u = 0; u < 32; ++u) acc[u] = !row || c0 + u >= P.C ? 0 : (neg >> u & 1) ? -acc[u] : acc[u];
+#pragma unroll
+        for (int o = 16, n = 16; n; o >>= 1, n >>= 1)
+#pragma unroll
+          for (int u = 0; u < n; ++u) {
+            const bool up = lane & o;
+            const long long give = up ? acc[u] : acc[u + n];
+            acc[u] = (up ? acc[u + n] : acc[u]) + __shfl_xor_sync(0xffffffffu, give, o);
+          }
+        double e0 = -double(acc[0]);
+        if (__any_sync(0xffffffffu, gi != 0.0)) {
+          double v[32];
+#pragma unroll
+          for (int u = 0; u < 32; ++u) {
+            v[u] = !row || c0 + u >= P.C ? 0.0 : (neg >> u & 1) ? -gi : gi;
+          }
+#pragma unroll
+          for (int o = 16, n = 16; n; o >>= 1, n >>= 1)
+#pragma unroll
+            for (int u = 0; u < n; ++u) {
+              const bool up = lane & o;
+              const double give = up ? v[u] : v[u + n];
+              v[u] = (up ? v[u + n] : v[u]) + __shfl_xor_sync(0xffffffffu, give, o);
+            }
+          e0 += v[0];
+        }
+        s_red[q4][cpart * 32 + lane] = e0;
       } else {
 #pragma unroll
         for (int u = 0; u < 32; ++u) {
@@ -515,16 +554,15 @@ cudaError_t launch_energy_slice_J(const EnergyProb& p0, const EnergyUnits& u, cu
 }
 
 cudaError_t launch_energy_slice_S(const EnergyProb& p0, const EnergyUnits& u, cudaStream_t s) {
-  k_energy_slice_S<<<dim3(u.n_col, u.KBmax), 256, 0, s>>>(p0, u.probs, u.col);
+  k_energy_slice_S<<<dim3(u.n_col, u.KBmax, SPLIT), 256, 0, s>>>(p0, u.probs, u.col);
   return cudaGetLastError();
 }
 
-cudaError_t launch_energy_product(const EnergyProb& p0, const EnergyUnits& u, int* err, cudaStream_t s) {
-  int dev = 0, sms = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_energy_product, cudaFuncAttributeMaxDynamicSharedMemorySize, ESMEM);
-  if (e != cudaSuccess) return e;
+cudaError_t energy_init() {
+  return cudaFuncSetAttribute(k_energy_product, cudaFuncAttributeMaxDynamicSharedMemorySize, ESMEM);
+}
+
+cudaError_t launch_energy_product(const EnergyProb& p0, const EnergyUnits& u, int sms, int* err, cudaStream_t s) {
   k_energy_product<<<std::min(u.n_tile, sms), ETHREADS, ESMEM, s>>>(p0, u.probs, u.tile, u.n_tile, err, kWaitCycles);
   return cudaGetLastError();
 }

@@ -60,7 +60,8 @@ struct EnergyUnits {
 };
 cudaError_t launch_energy_slice_J(const EnergyProb& p0, const EnergyUnits& u, cudaStream_t s);
 cudaError_t launch_energy_slice_S(const EnergyProb& p0, const EnergyUnits& u, cudaStream_t s);
-cudaError_t launch_energy_product(const EnergyProb& p0, const EnergyUnits& u, int* err, cudaStream_t s);
+cudaError_t energy_init();  // once per device, before its first product
+cudaError_t launch_energy_product(const EnergyProb& p0, const EnergyUnits& u, int sms, int* err, cudaStream_t s);
 
 // E[r] = sum over the row blocks of part (mt rows of ldp), r < R.
 cudaError_t launch_energy_sum(const double* part, int mt, int R, int ldp, double* E, cudaStream_t s);

@@ -43,6 +43,7 @@ struct gda_ctx {
   float* g32 = nullptr;   // [Np]
   float* h1 = nullptr;    // [Np]
   double diag = 0.0;      // -sum_i J_ii
+  bool small_int = false; // Ising, g = 0, J of few small integers (launch_energy_small)
   // instance checks
   int* d_flags = nullptr;
   unsigned long long* d_maxabs = nullptr;
@@ -283,7 +284,7 @@ gda_status load_instance(gda_ctx* c, const double* J, const double* g, cudaMemcp
   CK(cudaMemsetAsync(c->g64, 0, Np * sizeof(double), c->stream));
   if (g) CK(cudaMemcpyAsync(c->g64, g, N * sizeof(double), kind, c->stream));
   c->K_R = 0;  // a GD-mod coupling state belongs to the previous J
-  c->eJ_ready = false;
+  c->eJ_ready = c->small_int = false;
   LK(launch_snapshot_reset(c->snapE, c->snapR, c->snapStep, c->stream));
   c->ell_maxdeg = -1;
   CK(cudaMemsetAsync(c->d_flags, 0, sizeof(int), c->stream));
@@ -291,12 +292,15 @@ gda_status load_instance(gda_ctx* c, const double* J, const double* g, cudaMemcp
   LK(launch_check_instance(c->J64, c->g64, c->N, c->Np, c->d_flags, c->d_maxabs, c->d_diag, c->stream));
   LK(launch_energy_format(c->d_flags, c->d_maxabs, c->efmt, c->stream));
   int flags = 0;
+  double jmax = 0.0;
   CK(cudaMemcpyAsync(&flags, c->d_flags, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
+  CK(cudaMemcpyAsync(&jmax, c->d_maxabs, sizeof(double), cudaMemcpyDeviceToHost, c->stream));  // a double's bits
   CK(cudaMemcpyAsync(&c->diag, c->d_diag, sizeof(double), cudaMemcpyDeviceToHost, c->stream));
   CK(cudaStreamSynchronize(c->stream));
   if (flags & 1) return fail(c, GDA_ERR_INVALID, "J has a non-finite entry");
   if (flags & 2) return fail(c, GDA_ERR_INVALID, "J is not symmetric");
   if (flags & 8) return fail(c, GDA_ERR_INVALID, "g has a non-finite entry");
+  c->small_int = !c->cplx && !(flags & (4 | 16)) && energy_small_fits(c->N, jmax);
   LK(launch_prepare_J(c->J64, c->Np, c->J32, c->J16, c->stream));
   c->j8_ready = false;
   return GDA_OK;
@@ -524,6 +528,11 @@ gda_status energies_of(gda_ctx* c, const float* psi, int R, int C) {
   cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
   if (cudaStreamIsCapturing(c->stream, &cs) != cudaSuccess) cudaGetLastError();
   const bool recording = cs != cudaStreamCaptureStatusNone;
+  // (not into a graph: a replay may find another kind of J)
+  if (c->small_int && !recording && size_t(c->N) * c->N * R <= size_t(1) << 25) {
+    LK(launch_energy_small(c->J64, psi, c->N, c->Np, R, c->E64, c->stream));
+    return GDA_OK;
+  }
   if (recording && c->eJd) c->eJ_recorded = true;
   for (int m = 0; m < MT; m += mp) {
     p.mt0 = m;
@@ -541,7 +550,7 @@ gda_status energies_of(gda_ctx* c, const float* psi, int R, int C) {
       u.n_col = p.ntn;
       u.n_tile = p.mtn * p.ntn;
       if (m == 0 || np < NT) LK(launch_energy_slice_S(p, u, c->stream));
-      LK(launch_energy_product(p, u, c->err, c->stream));
+      LK(launch_energy_product(p, u, c->sms, c->err, c->stream));
     }
   }
   LK(launch_energy_sum(c->part64, MT, R, c->Rp, c->E64, c->stream));
@@ -666,6 +675,7 @@ static gda_status create_impl(const double* J, const double* g, int32_t N, int32
   auto step = [&](cudaError_t e) {
     if (st == GDA_OK && e != cudaSuccess) st = cuda_fail(c, e, "gda_create allocation");
   };
+  step(energy_init());
   step(dalloc(&c->J64, Np * Np));
   step(dalloc(&c->J32, Np * Np));
   if (c->tc_ok) step(dalloc(&c->J16, Np * Np));

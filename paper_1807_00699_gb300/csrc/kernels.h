@@ -27,6 +27,11 @@ cudaError_t launch_snapshot(const float* psi, int Np, int W, const double* lastE
                             double* snapE, int* snapR, long long* snapStep, float* snap, float* hist, int hist_cap,
                             const int* count, cudaStream_t s);
 cudaError_t launch_snapshot_reset(double* snapE, int* snapR, long long* snapStep, cudaStream_t s);
+// Energies of R restarts of real spins with g = 0 and integer J, |J_ij| <= jmax,
+// if energy_small_fits.
+bool energy_small_fits(int N, double jmax);
+cudaError_t launch_energy_small(const double* J64, const float* psi, int N, int Np, int R, double* E,
+                                cudaStream_t s);
 cudaError_t launch_argmin(const double* E, int R, double* bestE, int* bestR, cudaStream_t s);
 cudaError_t launch_best_cfg(const float* psi, const int* bestR, int N, int Np, int cplx, signed char* s8, double* th,
                             cudaStream_t s);

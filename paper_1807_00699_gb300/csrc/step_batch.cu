@@ -859,7 +859,7 @@ gda_status batch_energies(gda_batch* b) {
     const EnergyProb none{};
     if (!b->eJ_ready) BCK(launch_energy_slice_J(none, u, b->stream));
     BCK(launch_energy_slice_S(none, u, b->stream));
-    BCK(launch_energy_product(none, u, b->err, b->stream));
+    BCK(launch_energy_product(none, u, b->sms, b->err, b->stream));
   }
   b->eJ_ready = b->egroups.size() == 1;
   return GDA_OK;
@@ -1024,6 +1024,7 @@ gda_status gda_batch_create(int32_t n, const int32_t* N, const int32_t* model, c
         if (s != GDA_OK) return s;
       }
     BCK(set_batch_attrs());
+    BCK(energy_init());
     // with the batch: a batch that could be created and run can be judged
     const gda_status es = reserve_energies(b, SIZE_MAX);
     if (es != GDA_OK) return es;
