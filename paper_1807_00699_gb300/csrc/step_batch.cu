@@ -711,6 +711,27 @@ gda_status upload_settings(gda_batch* b, const gda_params* p) {
   return GDA_OK;
 }
 
+// True if J (n x n, host) is finite and symmetric; *jmax receives its largest
+// |J_ij| when every entry is an integer, else -1.  By pairs of mirrored 32 x 32
+// tiles: reading the mirrored entry down whole columns, a cache line each, took
+// half of the creation of 96 instances of up to 2000 spins.
+bool check_couplings(const double* J, int64_t n, double* jmax) {
+  constexpr int64_t T = 32;
+  bool integer = true;
+  double m = 0.0;
+  for (int64_t i0 = 0; i0 < n; i0 += T)
+    for (int64_t j0 = i0; j0 < n; j0 += T)
+      for (int64_t i = i0; i < std::min(n, i0 + T); ++i)
+        for (int64_t j = j0; j < std::min(n, j0 + T); ++j) {
+          const double v = J[i * n + j];
+          if (!std::isfinite(v) || v != J[j * n + i]) return false;
+          integer = integer && v == std::rint(v);
+          m = std::max(m, std::fabs(v));
+        }
+  *jmax = integer ? m : -1.0;
+  return true;
+}
+
 // Plans the final energies: every instance is cut into panels (row blocks x
 // column blocks) whose digits fit the workspace bounds, and panels are grouped
 // while the digits and spins of a group fit together (in `bound` bytes, unless
@@ -878,19 +899,9 @@ gda_status gda_batch_create(int32_t n, const int32_t* N, const int32_t* model, c
   for (int k = 0; k < n; ++k) {
     if (N[k] < 1 || N[k] > 65536 || R[k] < 1 || (model[k] != GDA_ISING && model[k] != GDA_XY) || !J[k])
       return GDA_ERR_INVALID;
-    const int64_t nn = N[k];
-    bool integer = true;
-    double m = 0.0;
-    for (int64_t i = 0; i < nn; ++i)
-      for (int64_t j = 0; j < nn; ++j) {
-        const double v = J[k][i * nn + j];
-        if (!std::isfinite(v) || v != J[k][j * nn + i]) return GDA_ERR_INVALID;
-        integer = integer && v == std::rint(v);
-        m = std::max(m, std::fabs(v));
-      }
-    jmax[k] = integer ? m : -1.0;
+    if (!check_couplings(J[k], N[k], &jmax[k])) return GDA_ERR_INVALID;
     if (g && g[k])
-      for (int64_t i = 0; i < nn; ++i)
+      for (int32_t i = 0; i < N[k]; ++i)
         if (!std::isfinite(g[k][i])) return GDA_ERR_INVALID;
   }
   gda_batch* b = new gda_batch();
