@@ -44,7 +44,10 @@ constexpr uint32_t T_GAM = 256;  // tensor-memory column of gamma
 // Measured (us a step, two 64-column blocks / one of 128 columns): Ising N =
 // 300, R = 4000 6.8 / 8.0; XY N = 1000, R = 1024 11.7 / 9.0; XY N = 2000, R =
 // 500 21.3 / 13.5: where tiles are not kept, the two blocks load them twice.
-constexpr int kResPairedMaxN = 576;
+// With noise decay each block also waits for the density sums of its column
+// block: Ising N = 130, R = 6000 10.5 / 9.2; N = 300, R = 4096 10.6 / 10.3, R =
+// 6000 10.9 / 11.6; N = 450, R = 4096 10.4 / 11.8, so one block up to N = 256.
+constexpr int kResPairedMaxN = 576, kResPairedMinNDecay = 257;
 // Rings of a CTA whose blocks have BN columns.
 template <int BN>
 struct ResCfg {
@@ -310,8 +313,11 @@ __global__ void __launch_bounds__(RES_THREADS, 1)
         if (e < RPT) {
           const int r = rbase + e;
           s_bstage[h * BN + e] = s_beta[h * BN + e];
-          if (need_red && n > 0)  // partial sums of step n-1 from every row block of this column block
-            for (int mb = 0; mb < MT && flags_ok; ++mb) flags_ok = flag_wait(fl + mb, unsigned(n), lim);
+          if (need_red && n > 0) {  // partial sums of step n-1 from every row block of this column block, a lane per flag
+            for (int mb = lane; mb < MT && flags_ok; mb += 32) flags_ok = flag_wait(fl + mb, unsigned(n), lim);
+            flags_ok = __all_sync(0xffffffffu, flags_ok);
+            __syncwarp();
+          }
           s_dsc[h * BN + e] = r < a.R ? noise_scale(sa, r) : 0.0f;
         }
         // one decision for all epilogue warps (the vote is also the barrier that
@@ -491,7 +497,9 @@ cudaError_t launch_res(const TcPlan* plan, const ResArgs& ra, const StepArgs& a,
   // while the chain they hide outweighs the coupling tiles they load twice, and
   // one 128-column block for larger N
   if ((a.C + 63) / 64 * mt <= sms) return launch_res_impl<CPLX, 64, 1>(A, *tc_plan_B64(plan), ra, a, s);
-  if (a.N <= kResPairedMaxN) return launch_res_impl<CPLX, 64, 2>(A, *tc_plan_B64(plan), ra, a, s);
+  const bool decay = a.noise_decay && a.noise_D != 0.0f;
+  if (a.N <= kResPairedMaxN && !(decay && a.N < kResPairedMinNDecay))
+    return launch_res_impl<CPLX, 64, 2>(A, *tc_plan_B64(plan), ra, a, s);
   return launch_res_impl<CPLX, 128, 1>(A, *tc_plan_B(plan), ra, a, s);
 }
 
