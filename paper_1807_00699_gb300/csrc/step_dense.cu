@@ -50,8 +50,8 @@ __device__ __forceinline__ void unpack2(unsigned long long v, float& lo, float& 
 // one K block ahead.  Shared memory returns one 4-byte value per thread and
 // cycle, so a K costs an SM 4 (RT + CPT) cycles of loads against RT CPT of
 // FMAs per scheduler: 64 / 64 for the 8 x 8 form (64 x 128 tiles), 48 / 32 for
-// 4 x 8, 32 / 16 for 4 x 4, 24 / 8 for 2 x 4; dense_bn weighs them.  On one
-// tile per SM a single warp per scheduler leaves latency exposed as well.
+// 4 x 8, 32 / 16 for 4 x 4, 24 / 8 for 2 x 4.  On one tile per SM a single
+// warp per scheduler leaves latency exposed as well; dense_bn weighs both.
 // Measured (GB300, us a step, against the 64 x 64 tile with 4 x 4 outputs per
 // thread and a transposing copy that this replaced): XY N = 1000, R = 256, RK4
 // 147 / 218; XY N = 1000, R = 1024, Euler 114 / 148; SK N = R = 4096, Euler
@@ -237,20 +237,26 @@ cudaError_t launch_dense_cfg(const StepArgs& a, const float* J32, const float* o
   return cudaGetLastError();
 }
 
-// Tile width: the busiest SM's tiles times a tile's cycles per K (the larger of
-// its shared-memory and FMA cycles, DenseCfg).
-int dense_bn(const StepArgs& a, int sms) {
-  static constexpr int width[4] = {128, 64, 32, 16}, cycles[4] = {64, 48, 32, 24};
+// Tile width with the smallest time per K of the busiest SM: a tile alone on it
+// runs one warp per scheduler, at the latency of its loads and FMA chains; tiles
+// that share it run at the rate of its shared-memory loads and FMAs (DenseCfg:
+// 64, 48, 32, 24 cycles at best).  Cycles fitted to every width on GB300 over N =
+// 20 .. 2200 and 8 .. 6000 columns, both models, Euler and RK4: on average 1 % above
+// the best width (XY N = 500, 3000 columns, Euler, us a step for 128 / 64 / 32 / 16 columns
+// 65 / 48 / 51 / 61; SK N = R = 4096 keeps 128).  *cycles: that time.
+int dense_bn(const StepArgs& a, int sms, long long* cycles = nullptr) {
+  static constexpr int width[4] = {128, 64, 32, 16}, lone[4] = {150, 76, 42, 29}, shared[4] = {90, 48, 28, 24};
   int best = 0;
   long long cost = -1;
   for (int k = 0; k < 4; ++k) {
     const long long tiles = (long long)((a.C + width[k] - 1) / width[k]) * simt_mtiles(a.N);
-    const long long c = (tiles + sms - 1) / sms * cycles[k];
+    const long long c = std::max<long long>(lone[k], (tiles + sms - 1) / sms * shared[k]);
     if (cost < 0 || c < cost) {
       cost = c;
       best = width[k];
     }
   }
+  if (cycles) *cycles = cost;
   return best;
 }
 
@@ -502,13 +508,12 @@ cudaError_t launch_step_dense(const StepArgs& a, const float* J32, const float* 
 // per stage is better.  J0 must fit in shared memory (N <= ~235).  A stage of
 // a segment takes the chain of N FMAs and loads for every wave of CTAs (and the
 // issue slots of further CTAs on the SM), and every wave first loads its J0; a
-// stage by itself takes a launch and its tile's K loop, which a lone tile of
-// four warps per SM runs at `alone` cycles a K.  Times in ns, fitted to runs on
-// GB300 over N = 10 .. 233, R = 16 .. 2048, both models and integrators, 13 and 300
-// steps: the rule chose nothing more than 3 % slower than a launch per stage.  us
-// a step, segment / launch per stage, Euler: Ising N = 10, R = 64 0.5 / 5.2; N = 200,
-// R = 256 3.6 / 8.2; XY N = 200, R = 400 8.1 / 10.3, R = 1024 (four waves) 16.2 /
-// 14.4; and 13.5 us a wave to load J0 at N = 200.
+// stage by itself takes a launch and its tiles' K loops (dense_bn).  Times in
+// ns, fitted to runs on GB300 over N = 10 .. 233, R = 16 .. 2048, both models and
+// integrators, 13 and 300 steps: the rule chose nothing more than 3 % slower than
+// a launch per stage.  us a step, segment / launch per stage, Euler: Ising N = 10,
+// R = 64 0.5 / 5.2; N = 200, R = 256 3.6 / 8.2; XY N = 200, R = 400 8.1 / 10.3, R =
+// 1024 (four waves) 16.2 / 14.4; and 13.5 us a wave to load J0 at N = 200.
 int dense_seg_columns(const StepArgs& a, int sms, bool rk4, long long steps) {
   if (a.N > 256 || dense_seg_smem(a, 4) > kDenseSegSmemMax) return 0;
   auto rounds = [&](int nc) { return ((a.C + nc - 1) / nc + sms - 1) / sms; };
@@ -519,10 +524,9 @@ int dense_seg_columns(const StepArgs& a, int sms, bool rk4, long long steps) {
   const long long shared = (std::min(ctas, sms * per_sm) + sms - 1) / sms - 1;
   const long long stage = waves * (350 + (a.cplx ? 19 : 17) * N + shared * warps * N * (nc + 2) / 8);
   const long long load = waves * (2000 + 65 * N);
-  const int bn = dense_bn(a, sms);
-  const long long alone = bn == 128 ? 176 : bn == 64 ? 84 : bn == 32 ? 47 : 29;
-  const long long tiles = (long long)((a.C + bn - 1) / bn) * simt_mtiles(a.N);
-  const long long single = 5000 + (tiles + sms - 1) / sms * ((N + BK - 1) / BK * BK) * alone / 2;
+  long long cycles = 0;
+  (void)dense_bn(a, sms, &cycles);
+  const long long single = 5000 + ((N + BK - 1) / BK * BK) * cycles / 2;
   const long long stages = steps * (rk4 ? 4 : 1);
   return stages * stage + load < stages * single ? nc : 0;
 }
