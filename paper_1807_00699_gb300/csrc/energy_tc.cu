@@ -60,6 +60,13 @@ __device__ __forceinline__ int4 unit_of(const int4* u, int k, int rows) {
   return u ? u[k] : make_int4(0, k % rows, k / rows, 0);
 }
 
+// Exponent of a row with a non-finite entry (a J that gda_load_dev refused): its
+// energies are NaN.
+constexpr int kRowBad = 1 << 24;
+__device__ __forceinline__ double scaled(double a, int ex) {  // a 2^ex for any ex
+  return ex > kRowBad / 2 ? __longlong_as_double(0x7ff8000000000000ll) : scalbn(a, ex);
+}
+
 // Digits of J, and whether they are J's own (EnergyProb::fmt).
 __device__ __forceinline__ int2 format_of(const EnergyProb& P) { return P.fmt ? *P.fmt : make_int2(P.nsJ, P.jint); }
 
@@ -71,7 +78,7 @@ __host__ __device__ inline int integer_digits(double jmax) {
 }
 
 __global__ void k_energy_format(const int* flags, const unsigned long long* maxabs, int2* fmt) {
-  const int n = (*flags & 4) ? 0 : integer_digits(__longlong_as_double((long long)*maxabs));
+  const int n = (*flags & 5) ? 0 : integer_digits(__longlong_as_double((long long)*maxabs));
   *fmt = n ? make_int2(n, 1) : make_int2(kEnergySlices, 0);
 }
 
@@ -110,18 +117,21 @@ __global__ void __launch_bounds__(256) k_energy_rexp(EnergyProb p0, const Energy
   if (i >= P.N) return;
   const int2 F = format_of(P);
   double m = 0.0, a = 0.0;
+  bool bad = false;
   for (int j = lane; j < P.N; j += 32) {
     const double v = fabs(P.J[size_t(i) * P.ld + j]);
+    bad |= !isfinite(v);
     m = fmax(m, v);
     a += v;
   }
+  bad = __any_sync(0xffffffffu, bad);
   for (int o = 16; o; o >>= 1) {
     m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
     a += __shfl_xor_sync(0xffffffffu, a, o);
   }
-  const int e = F.y ? 8 * F.x - 1 : m > 0.0 ? ilogb(m) + 1 : 0;
+  const int e = bad ? kRowBad : F.y ? 8 * F.x - 1 : m > 0.0 ? ilogb(m) + 1 : 0;
   const int lgN = P.N > 1 ? 32 - __clz(P.N - 1) : 0;
-  const int l = !(m > 0.0) ? 0 : isfinite(a) ? ilogb(a) + 1 - e : lgN;
+  const int l = bad || !(m > 0.0) ? 0 : isfinite(a) ? ilogb(a) + 1 - e : lgN;
   if (lane == 0) P.rexp[i] = make_int2(e, l);
 }
 
@@ -419,7 +429,7 @@ __global__ void __launch_bounds__(ETHREADS, 1) k_energy_product(const __grid_con
           if (row && c < P.C) {
             const double sr = P.S64[size_t(c) * P.Np + i], si = P.S64[size_t(c + 1) * P.Np + i];
             const double a = fma(sr, double(acc[2 * u]), si * double(acc[2 * u + 1]));
-            v[u] = fma(gi, sr, -(wide ? scalbn(a, ex) : a * f));
+            v[u] = fma(gi, sr, -(wide ? scaled(a, ex) : a * f));
           }
         }
 #pragma unroll
@@ -477,7 +487,7 @@ __global__ void __launch_bounds__(ETHREADS, 1) k_energy_product(const __grid_con
           if (row && c < P.C) {
             const double s = P.psi[size_t(c) * P.Np + i] >= 0.0f ? 1.0 : -1.0;
             const double a = double(acc[u]);
-            v[u] = s * (gi - (wide ? scalbn(a, ex) : a * f));
+            v[u] = s * (gi - (wide ? scaled(a, ex) : a * f));
           }
         }
 #pragma unroll
