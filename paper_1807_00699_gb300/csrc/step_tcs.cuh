@@ -319,7 +319,6 @@ __global__ void __launch_bounds__(TcThreads<M_EULER>::N, 1)
             }
           }
         };
-        if (cbeg < a.C)  // the warp's columns hold a restart (FP8, XY N = 130, 8 columns: 7.4 us a step without this, 6.7 with)
 #pragma unroll
         for (int ch = 0; ch < NCH; ++ch) {
           if (PF > 0 && ch + PF < NCH) epi_prefetch_l2<MODE, CPLX, CW>(a, i, cbeg + (ch + PF) * CW, lane);
