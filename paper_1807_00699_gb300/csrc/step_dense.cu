@@ -55,7 +55,7 @@ __device__ __forceinline__ void unpack2(unsigned long long v, float& lo, float& 
 // Measured (GB300, us a step, against the 64 x 64 tile with 4 x 4 outputs per
 // thread and a transposing copy that this replaced): XY N = 1000, R = 256, RK4
 // 147 / 218; XY N = 1000, R = 1024, Euler 114 / 148; SK N = R = 4096, Euler
-// 2745 / 3678 (50 TFLOP/s); XY N = 300, R = 64, RK4 36 / 102.
+// 2556 / 3678 (54 TFLOP/s); XY N = 300, R = 64, RK4 36 / 102.
 template <int RT, int CPT>
 struct DenseCfg {
   static constexpr int LX = BM / RT, LY = 32 / LX;
@@ -238,19 +238,19 @@ cudaError_t launch_dense_cfg(const StepArgs& a, const float* J32, const float* o
 }
 
 // Tile width with the smallest time per K of the busiest SM: a tile alone on it
-// runs one warp per scheduler, at the latency of its loads and FMA chains; tiles
-// that share it run at the rate of its shared-memory loads and FMAs (DenseCfg:
-// 64, 48, 32, 24 cycles at best).  Cycles fitted to every width on GB300 over N =
-// 20 .. 2200 and 8 .. 6000 columns, both models, Euler and RK4: on average 1 % above
-// the best width (XY N = 500, 3000 columns, Euler, us a step for 128 / 64 / 32 / 16 columns
-// 65 / 48 / 51 / 61; SK N = R = 4096 keeps 128).  *cycles: that time.
+// runs one warp per scheduler, at the latency of its loads and FMA chains (`lone`
+// cycles); each further tile on the SM adds the cycles of its shared-memory
+// loads and FMAs (`more`; DenseCfg: 64, 48, 32, 24).  Averages over every width on
+// GB300, N = 250 .. 2200, 8 .. 6000 columns, both models, Euler and RK4; the choice is
+// on average 1.2 % above the best width.  (us a step for 128 / 64 / 32 / 16 columns:
+// XY N = 500, 3000 columns, Euler 65 / 48 / 51 / 61.)  *cycles: that time.
 int dense_bn(const StepArgs& a, int sms, long long* cycles = nullptr) {
-  static constexpr int width[4] = {128, 64, 32, 16}, lone[4] = {150, 76, 42, 29}, shared[4] = {90, 48, 28, 24};
+  static constexpr int width[4] = {128, 64, 32, 16}, lone[4] = {142, 73, 47, 32}, more[4] = {93, 46, 31, 21};
   int best = 0;
   long long cost = -1;
   for (int k = 0; k < 4; ++k) {
     const long long tiles = (long long)((a.C + width[k] - 1) / width[k]) * simt_mtiles(a.N);
-    const long long c = std::max<long long>(lone[k], (tiles + sms - 1) / sms * shared[k]);
+    const long long c = lone[k] + ((tiles + sms - 1) / sms - 1) * more[k];
     if (cost < 0 || c < cost) {
       cost = c;
       best = width[k];
