@@ -7,6 +7,7 @@
 #include <cstdio>
 #include <cstring>
 #include <string>
+#include <type_traits>
 #include <vector>
 
 #include "../../include/gda.h"
@@ -28,6 +29,7 @@ size_t round_up(size_t x, size_t m) { return (x + m - 1) / m * m; }
 }  // namespace
 
 struct gda_ctx {
+  unsigned char* small = nullptr;  // one allocation of 16-byte slots for the single values below
   int dev = 0, sms = 148;
   int N = 0, Np = 0, model = 0, cplx = 0;
   cudaStream_t stream = nullptr;
@@ -624,14 +626,13 @@ void gda_destroy(gda_ctx* c) {
   if (!c) return;
   free_state(c);
   dfree(c->J64); dfree(c->J32); dfree(c->J16); dfree(c->J8); dfree(c->jscale); dfree(c->g64); dfree(c->g32); dfree(c->h1);
-  dfree(c->d_flags); dfree(c->d_maxabs); dfree(c->d_diag);
-  dfree(c->bestE); dfree(c->bestR); dfree(c->cfg8); dfree(c->cfgth);
-  dfree(c->erexp); dfree(c->efmt); dfree(c->eJd);
-  dfree(c->t_step); dfree(c->t_E); dfree(c->t_r); dfree(c->t_count); dfree(c->err); dfree(c->flags);
+  dfree(c->small);
+  dfree(c->cfg8); dfree(c->cfgth);
+  dfree(c->erexp); dfree(c->eJd);
+  dfree(c->t_step); dfree(c->t_E); dfree(c->t_r); dfree(c->flags);
   dfree(c->seg_flags);
-  dfree(c->lastE); dfree(c->lastR); dfree(c->snapE); dfree(c->snapR); dfree(c->snapStep); dfree(c->snap);
+  dfree(c->snap);
   dfree(c->hist);
-  dfree(c->d_zero);
   dfree(c->stamps);
   dfree(c->K);
   dfree(c->ell); dfree(c->d_maxdeg);
@@ -682,31 +683,23 @@ static gda_status create_impl(const double* J, const double* g, int32_t N, int32
   step(dalloc(&c->g64, Np));
   step(dalloc(&c->g32, Np));
   step(dalloc(&c->h1, Np));
-  step(dalloc(&c->d_flags, 1));
-  step(dalloc(&c->d_maxabs, 1));
-  step(dalloc(&c->d_diag, 1));
-  step(dalloc(&c->bestE, 1));
-  step(dalloc(&c->bestR, 1));
   step(dalloc(&c->cfg8, Np));
   step(dalloc(&c->cfgth, Np));
   step(dalloc(&c->t_step, kTraceCap));
   step(dalloc(&c->t_E, kTraceCap));
   step(dalloc(&c->t_r, kTraceCap));
-  step(dalloc(&c->t_count, 1));
-  step(dalloc(&c->lastE, 1));
-  step(dalloc(&c->lastR, 1));
-  step(dalloc(&c->snapE, 1));
-  step(dalloc(&c->snapR, 1));
-  step(dalloc(&c->snapStep, 1));
   step(dalloc(&c->snap, 2 * Np));
-  step(dalloc(&c->d_zero, 1));
   step(dalloc(&c->erexp, Np));
-  step(dalloc(&c->efmt, 1));
-  step(dalloc(&c->err, 1));
   step(dalloc(&c->flags, kMaxResidentTiles));
-  if (st == GDA_OK) step(cudaMemset(c->err, 0, sizeof(int)));
-  if (st == GDA_OK) step(cudaMemset(c->t_count, 0, sizeof(int)));
-  if (st == GDA_OK) step(cudaMemset(c->d_zero, 0, sizeof(int)));
+  step(dalloc(&c->small, 16 * 16));
+  if (st == GDA_OK) {
+    step(cudaMemset(c->small, 0, 16 * 16));
+    int slot = 0;
+    auto place = [&](auto*& p) { p = reinterpret_cast<std::remove_reference_t<decltype(p)>>(c->small + 16 * slot++); };
+    place(c->d_flags); place(c->d_maxabs); place(c->d_diag); place(c->bestE); place(c->bestR); place(c->t_count);
+    place(c->lastE); place(c->lastR); place(c->snapE); place(c->snapR); place(c->snapStep); place(c->d_zero);
+    place(c->efmt); place(c->err);
+  }
   if (st == GDA_OK) step(cudaMemset(c->snap, 0, 2 * Np * sizeof(float)));
   if (st == GDA_OK) step(cudaMemset(c->h1, 0, Np * sizeof(float)));
   if (st == GDA_OK) step(cudaMemset(c->g32, 0, Np * sizeof(float)));
