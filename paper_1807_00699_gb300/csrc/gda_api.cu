@@ -92,6 +92,10 @@ struct gda_ctx {
   bool eJ_ready = false;      // it holds the whole current J
   bool eJ_recorded = false;
   size_t eJ_bound = kEnergyJBytes;
+  // The latest energies' work, which uses scratch and eJd: another stream's
+  // calls come after it (gda_set_stream).
+  cudaEvent_t e_done = nullptr;
+  bool e_pending = false;
   double* E64 = nullptr;
   double* bestE = nullptr;
   int* bestR = nullptr;
@@ -556,6 +560,10 @@ gda_status energies_of(gda_ctx* c, const float* psi, int R, int C) {
     }
   }
   LK(launch_energy_sum(c->part64, MT, R, c->Rp, c->E64, c->stream));
+  if (!recording) {
+    CK(cudaEventRecord(c->e_done, c->stream));
+    c->e_pending = true;
+  }
   return GDA_OK;
 }
 
@@ -626,6 +634,7 @@ void gda_destroy(gda_ctx* c) {
   if (!c) return;
   free_state(c);
   dfree(c->J64); dfree(c->J32); dfree(c->J16); dfree(c->J8); dfree(c->jscale); dfree(c->g64); dfree(c->g32); dfree(c->h1);
+  if (c->e_done) cudaEventDestroy(c->e_done);
   dfree(c->small);
   dfree(c->cfg8); dfree(c->cfgth);
   dfree(c->erexp); dfree(c->eJd);
@@ -677,6 +686,7 @@ static gda_status create_impl(const double* J, const double* g, int32_t N, int32
     if (st == GDA_OK && e != cudaSuccess) st = cuda_fail(c, e, "gda_create allocation");
   };
   step(energy_init());
+  step(cudaEventCreateWithFlags(&c->e_done, cudaEventDisableTiming));
   step(dalloc(&c->J64, Np * Np));
   step(dalloc(&c->J32, Np * Np));
   if (c->tc_ok) step(dalloc(&c->J16, Np * Np));
@@ -744,7 +754,13 @@ gda_status gda_set_energy_workspace(gda_ctx* c, int64_t bytes) {
 
 gda_status gda_set_stream(gda_ctx* c, void* stream) {
   if (!c) return GDA_ERR_INVALID;
-  c->stream = static_cast<cudaStream_t>(stream);
+  const cudaStream_t next = static_cast<cudaStream_t>(stream);
+  if (c->e_pending && next != c->stream) {
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(next, &cs) != cudaSuccess) cudaGetLastError();
+    if (cs == cudaStreamCaptureStatusNone) CK(cudaStreamWaitEvent(next, c->e_done, 0));
+  }
+  c->stream = next;
   return GDA_OK;
 }
 
