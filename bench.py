@@ -43,7 +43,7 @@ WORKLOADS = {
 METRIC = "time-to-target energy (s) & spin-updates/s: BF16+learned vs plain FP32 GDA"
 # DRAM bytes (read + write) per step of each workload's dominant kernel, from
 # one-launch ncu captures (profiles/): the streaming kernel's 3-step launch moved
-# 873.3 + 482.1 MB; None where no capture of the current kernel exists.
+# 841.1 + 478.5 MB; None where no capture of the current kernel exists.
 TRAFFIC = {"sk4096": (841.058048e6 + 478.54464e6) / 3, "xy1000": None}
 
 

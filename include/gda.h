@@ -80,9 +80,10 @@ typedef enum {
   GDA_FP8 = 2,  /* J.Psi on tcgen05 tensor cores, E4M3 operands, FP32 accum:
                  * J0_ij stored as e4m3(J0_ij / s_i), s_i = max_j |J0_ij| / 448
                  * (row scale), amplitudes as e4m3(psi * 64) (|psi| up to 7
-                 * before saturation), Y_i = acc_i * s_i / 64.  Per-step
-                 * schedule only; the energy tracking of energy_every uses
-                 * the BF16 product of the projected spins. */
+                 * before saturation), Y_i = acc_i * s_i / 64.  Launched per
+                 * step or streaming (gda_schedule), not resident; the
+                 * energy tracking of energy_every uses the BF16 product of
+                 * the projected spins. */
   GDA_SPARSE = 3 /* J.Psi over the nonzeros of J only (the paper's sparse
                  * 3-regular instances, Sec. 2): on first use J0 is compacted
                  * on the device into an ELL table of at most
@@ -238,12 +239,15 @@ gda_status gda_run(gda_ctx* ctx, const gda_params* p, int32_t R, int64_t steps);
 gda_status gda_sync(gda_ctx* ctx);
 
 /* Eq. (1) energy of the projected spins of every restart, in FP64 (exact for
- * Ising runs with integer J and g = 0).
+ * Ising runs with g = 0 and integer J, |J_ij| <= 2^31 and N^2 max |J_ij| <
+ * 2^53; of other J each row counts to 2^-55 of its largest entry).
  * E: R doubles on the host.  Synchronises. */
 gda_status gda_energy(gda_ctx* ctx, double* E);
 
 /* Same as gda_energy into R doubles on the device; stream ordered, does not
- * synchronise. */
+ * synchronise.  Recorded into a CUDA graph (after the state exists), replays
+ * evaluate the instance loaded and the amplitudes held when they run, for as
+ * long as no larger number of restarts makes the context reallocate its state. */
 gda_status gda_energy_dev(gda_ctx* ctx, double* E_dev);
 
 /* Bound, in bytes, on the device memory the context keeps for the energies'
@@ -278,7 +282,7 @@ gda_status gda_set_state(gda_ctx* ctx, const float* psi, const float* gamma, con
 /* The running best of the energy trace (S8): whenever a tracking evaluation
  * (energy_every > 0) finds a lower energy than any before it, the library
  * keeps that restart's amplitudes; this call evaluates the kept configuration
- * in FP64 (exact for integer-J Ising) and returns that energy, the restart,
+ * in FP64 (exact where gda_energy is) and returns that energy, the restart,
  * the step of the evaluation and optionally the configuration (cfg as in
  * gda_best).  The running best spans runs continued with init_mode 2 and is
  * cleared by a fresh run, gda_set_state and gda_load.  GDA_ERR_STATE if no
@@ -286,7 +290,7 @@ gda_status gda_set_state(gda_ctx* ctx, const float* psi, const float* gamma, con
  * visits, verified at the end.) */
 gda_status gda_best_seen(gda_ctx* ctx, double* E, int32_t* r, int64_t* step, void* cfg);
 
-/* FP64 Eq. (1) energies (exact for integer-J Ising) of the configurations the
+/* FP64 Eq. (1) energies (exact where gda_energy is) of the configurations the
  * trace of the last run names: trace entry k's configuration is the restart
  * with the lowest tracking energy at that evaluation, as it was at that step
  * (kept on the device when the evaluation ran).  E: `count` doubles (host)

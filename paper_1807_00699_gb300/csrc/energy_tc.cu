@@ -24,12 +24,14 @@
 // swizzled K-major form that tcgen05.mma reads, so a stage of the ring is two
 // plain 16 KB bulk copies.  Warp 0 loads, warp 1 issues MMAs into two
 // tensor-memory accumulators in turn, 16 warps drain them.  What bounds it is
-// the delivery of 32 KB of digits per 128 x 128 x 64 product from L2.
-// Measured (GB300): every restart's energy at XY N = 1000, R = 1024 takes 218
-// us here plus 83 us for the spins' digits, where the FP64 pipe took 4.10 ms;
-// the lowest of SK N = R = 4096 takes 1.1 ms, where ranking in compensated FP32
-// and evaluating the candidates in FP64 took 11.1 ms.  Against sums in
-// extended precision the energies are 2-5 times closer than the FP64 pipe's
+// that read-out into the int64 sums: ~3.5 us per accumulation, whether of 2 K
+// blocks (XY N = 100, R = 64: 28 in 98 us) or of 8 (N = 1000, R = 1024: 56 in 206).
+// Measured (GB300): every restart's energy at XY N = 1000, R = 1024 takes 206
+// us here plus 86 us for the spins' digits (and 38 us more for J's in the first
+// call after a load), where the FP64 pipe took 4.10 ms; those of SK N = R = 4096
+// take 0.87 ms (1.21 after a load), where ranking in compensated FP32 and
+// evaluating the candidates in FP64 took 11.1 ms.  Against sums in extended
+// precision the energies are 2-5 times closer than the FP64 pipe's
 // (relative error, N = 150 / 777 / 1000: 1.4e-16 / 1.4e-16 / 1.8e-16, before
 // 3.0e-16 / 7.2e-16 / 7.5e-16).
 #include "energy_tc.h"

@@ -8,8 +8,8 @@
 // its scratch (the per-tile partial energies) in a fixed-size file-scope
 // device array that every GPU loading this library holds until the process
 // exits.  It computes the same quantity as gda_energy (FP64 energies of the
-// projected spins) with the same tiled product, but projects the spins on the
-// fly instead of staging them in a context buffer.
+// projected spins) with a plain tiled FP64 product that projects the spins on
+// the fly.
 #include <mutex>
 
 #include "../../include/gda.h"
